@@ -26,8 +26,9 @@
 namespace soap {
 
 constexpr int kLinesPerChunk = 128;      // generic kernel
-constexpr int kWinLines = 32;             // windowed kernel: 32 lines span ~600 px here
+constexpr int kWinLines = 32;             // windowed kernel: lines per chunk at most
 constexpr int kWinMax = 768;              // staged pixels per block (window budget)
+constexpr int kWinSB32 = 16, kWinSB64 = 8; // windowed kernel: spectra per block (FP32, FP64)
 constexpr int kReduceSplit = 8;
 
 // Per line: validity and the box start a0 = u_l - h + 1/2 (pixel n covers [n, n+1) in a0 + s
@@ -119,10 +120,11 @@ __global__ void k_ccf_partial(int n_lines, const int* __restrict__ U, const T* _
 // spectra, in shared memory as padded rows [pixel][SB] (one 16-byte vector per VW spectra).
 // For each line the box position (integer pixel + fraction) is computed once and reused for
 // all SB spectra; the box covers at most NB pixels, handled branch-free (zero overlaps add
-// zero).  Chunks whose window does not fit fall back to global loads.
+// zero).  Chunks whose window does not fit fall back to global loads.  win_lines (at most
+// kWinLines) lines per chunk: see ccf_window_lines.
 template <typename T, int SB, int NB>
 __global__ void __launch_bounds__(256)
-k_ccf_window(int n_lines, const int* __restrict__ U, const T* __restrict__ f,
+k_ccf_window(int n_lines, int win_lines, const int* __restrict__ U, const T* __restrict__ f,
              const int* __restrict__ valid, const T* __restrict__ wl_, int n_v,
              const int* __restrict__ S, const T* __restrict__ g, double box, int64_t n_px,
              int n_spec, const T* __restrict__ spectra, T* __restrict__ partial) {
@@ -137,7 +139,7 @@ k_ccf_window(int n_lines, const int* __restrict__ U, const T* __restrict__ f,
     T* win = reinterpret_cast<T*>(smraw);
     const int s0 = blockIdx.y * SB;
     const int ns = min(SB, n_spec - s0);
-    const int n_chunks = (n_lines + kWinLines - 1) / kWinLines;
+    const int n_chunks = (n_lines + win_lines - 1) / win_lines;
     const T boxT = (T)box;
     const int k = threadIdx.x;
     const bool active = k < n_v;
@@ -147,8 +149,8 @@ k_ccf_window(int n_lines, const int* __restrict__ U, const T* __restrict__ f,
 #pragma unroll
     for (int s = 0; s < SB; s++) acc[s] = T(0);
     for (int chunk = blockIdx.x; chunk < n_chunks; chunk += gridDim.x) {
-        const int l0 = chunk * kWinLines;
-        const int l1 = min(n_lines, l0 + kWinLines);
+        const int l0 = chunk * win_lines;
+        const int l1 = min(n_lines, l0 + win_lines);
         // window [n_lo, n_hi) with a margin on both sides; pixels off the grid stage as 0
         const int64_t n_lo = (int64_t)U[l0] + S[0] - 2;
         const int64_t n_hi = (int64_t)U[l1 - 1] + S[n_v - 1] + NB + 2;
@@ -1168,6 +1170,18 @@ static cudaError_t fit_f32_launch(int n_spec, cudaStream_t st, bool early, int n
     return cudaLaunchKernelEx(&cfg, k_gauss_fit_f32<1>, n, n_v, v_lo, v_step, ccf, scratch, rv, fit, win);
 }
 
+// Lines per chunk of the windowed kernel.  A chunk of kWinLines lines costs one window, so it is
+// the cheapest per line, but a chunk is a block's whole work: with few lines there must be fewer
+// to a chunk for every SM to get some (four blocks per SM: 30 lines of a 4,096-pixel grid and 25
+// spectra in 2 blocks took 346 us; now one line to a chunk, and the whole
+// call of that size 117 us instead of 307), and where lines are sparse (136 pixels apart there), their
+// windows together must still fit the stage, else every overlap reads global memory.
+static int ccf_window_lines(int n_lines, int64_t n_px, double sweep, int nb, int spec_blocks, int sms) {
+    const double fill = (double)n_lines * spec_blocks / (4.0 * sms);
+    const double fit = (kWinMax - sweep - nb - 6) / ((double)n_px / n_lines);
+    return std::max(1, (int)std::min<double>(kWinLines, std::min(fill, fit)));
+}
+
 bool ccf_mask_same(const CcfState& st, const double* mask_lambda, const double* mask_weight,
                    int n_lines, double width_kms) {
     const std::vector<double>& k = st.mask_key;
@@ -1205,11 +1219,16 @@ soap_status ccf_prepare(soap_ctx* c, CcfState& st, const double* mask_lambda, co
     p.h = width_kms / (2.0 * kCKms * c->delta);
     // windowed kernel: one velocity per thread (n_v <= 256); blocks walk the chunks
     p.windowed = sorted && n_v <= 256 && 2.0 * width_kms / (2.0 * kCKms * c->delta) <= 15.0;
-    p.n_wgroups = (n_lines + kWinLines - 1) / kWinLines;   // one chunk of lines per block
-    p.n_chunks = p.windowed ? p.n_wgroups : (n_lines + kLinesPerChunk - 1) / kLinesPerChunk;
     int sms = 0, dev = 0;
     SOAP_CUDA(cudaGetDevice(&dev));
     SOAP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const int win_sb = f32 ? kWinSB32 : kWinSB64;
+    p.win_nb = 2.0 * p.h <= 1.0 ? 2 : (2.0 * p.h <= 7.0 ? 8 : 16);   // pixels a box covers at most
+    p.win_lines = ccf_window_lines(n_lines, c->n_px,
+                                   (std::atanh((v_lo + (n_v - 1) * v_step) / kCKms) - std::atanh(v_lo / kCKms)) / c->delta,
+                                   p.win_nb, (n_spec + win_sb - 1) / win_sb, sms);
+    p.n_wgroups = (n_lines + p.win_lines - 1) / p.win_lines;   // one chunk of lines per block
+    p.n_chunks = p.windowed ? p.n_wgroups : (n_lines + kLinesPerChunk - 1) / kLinesPerChunk;
     // register-tiled kernel (FP32, sorted mask): pixels a group of kTileVT velocities can reach
     // for one line, from the largest spread of kTileVT consecutive box positions
     if (f32 && sorted && n_v >= kTileVT) {
@@ -1349,25 +1368,26 @@ soap_status ccf_enqueue(soap_ctx* c, CcfState& st, const CcfPlan& p, const void*
     } else if (p.windowed) {
         const int threads = ((n_v + 31) / 32) * 32;
         const double box = 2.0 * p.h;
-        const bool small = box <= 1.0;                   // the box covers at most 2 pixels
-        dim3 grid32((unsigned)p.n_wgroups, (unsigned)((n_spec + 15) / 16));
-        dim3 grid64((unsigned)p.n_wgroups, (unsigned)((n_spec + 7) / 8));
-        const size_t smem32 = (size_t)kWinMax * (16 + 4) * 4;
-        const size_t smem64 = (size_t)kWinMax * (8 + 2) * 8;
+        dim3 grid32((unsigned)p.n_wgroups, (unsigned)((n_spec + kWinSB32 - 1) / kWinSB32));
+        dim3 grid64((unsigned)p.n_wgroups, (unsigned)((n_spec + kWinSB64 - 1) / kWinSB64));
+        const size_t smem32 = (size_t)kWinMax * (kWinSB32 + 4) * 4;
+        const size_t smem64 = (size_t)kWinMax * (kWinSB64 + 2) * 8;
 #define SOAP_CCF_LAUNCH(T, SB, NB, GRID, SMEM, F, WT, G, SPEC)                                    \
         do {                                                                                       \
             SOAP_CUDA(cudaFuncSetAttribute(k_ccf_window<T, SB, NB>,                                \
                                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM)); \
             k_ccf_window<T, SB, NB><<<GRID, threads, SMEM, c->stream>>>(                          \
-                n_lines, p.U, F, p.valid, WT, n_v, p.S, G, box, c->n_px, n_spec,                   \
+                n_lines, p.win_lines, p.U, F, p.valid, WT, n_v, p.S, G, box, c->n_px, n_spec,      \
                 (const T*)SPEC, reinterpret_cast<T*>(d_part));                                     \
         } while (0)
         if (p.f32) {
-            if (small) SOAP_CCF_LAUNCH(float, 16, 2, grid32, smem32, p.f32t, p.w32, p.g32, spectra_dev);
-            else SOAP_CCF_LAUNCH(float, 16, 16, grid32, smem32, p.f32t, p.w32, p.g32, spectra_dev);
+            if (p.win_nb == 2) SOAP_CCF_LAUNCH(float, kWinSB32, 2, grid32, smem32, p.f32t, p.w32, p.g32, spectra_dev);
+            else if (p.win_nb == 8) SOAP_CCF_LAUNCH(float, kWinSB32, 8, grid32, smem32, p.f32t, p.w32, p.g32, spectra_dev);
+            else SOAP_CCF_LAUNCH(float, kWinSB32, 16, grid32, smem32, p.f32t, p.w32, p.g32, spectra_dev);
         } else {
-            if (small) SOAP_CCF_LAUNCH(double, 8, 2, grid64, smem64, p.f64, p.w64, p.g64, spectra_dev);
-            else SOAP_CCF_LAUNCH(double, 8, 16, grid64, smem64, p.f64, p.w64, p.g64, spectra_dev);
+            if (p.win_nb == 2) SOAP_CCF_LAUNCH(double, kWinSB64, 2, grid64, smem64, p.f64, p.w64, p.g64, spectra_dev);
+            else if (p.win_nb == 8) SOAP_CCF_LAUNCH(double, kWinSB64, 8, grid64, smem64, p.f64, p.w64, p.g64, spectra_dev);
+            else SOAP_CCF_LAUNCH(double, kWinSB64, 16, grid64, smem64, p.f64, p.w64, p.g64, spectra_dev);
         }
 #undef SOAP_CCF_LAUNCH
     } else if (p.f32) {
