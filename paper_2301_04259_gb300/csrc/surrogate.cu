@@ -5,10 +5,10 @@
 // ranges or with a predicted error above a threshold go back to the plain method.
 //
 //  * network: 8 -> 4 x 256 (GELU) -> 129, BF16 weights and activations as GEMM operands, FP32
-//    accumulation, every product on the tensor cores (tc::gemm_tn), FP32 master weights and
-//    Adam moments; one training step = 5 forward GEMMs, a loss kernel, 9 backward GEMMs (GELU'
-//    fused into the epilogue of each dA GEMM), one bias-gradient kernel and one Adam kernel,
-//    captured once into a CUDA graph and replayed for every batch.
+//    accumulation, every product on the tensor cores, FP32 master weights and Adam moments.  One
+//    training step is three kernels, captured once into a CUDA graph and replayed for every batch:
+//    the forward, loss and backward chain of each 128 rows (mlp.cu k_mlp_train), all weight and
+//    bias gradients (k_mlp_dw), Adam.  Queries run their whole chain in one kernel (k_mlp_query).
 //  * PCA: randomized SVD with power iterations (Halko, Martinsson & Tropp 2011) over the
 //    mean-centred residuals, FP32 GEMMs on the SIMT cores, the small symmetric eigenproblems
 //    (l x l) in FP64 on the host (cyclic Jacobi).
@@ -21,7 +21,7 @@
 #include <random>
 #include <vector>
 
-#include "tc_gemm.cuh"
+#include "mlp.cuh"
 
 using bf16 = __nv_bfloat16;
 
@@ -63,15 +63,12 @@ struct soap_surrogate {
     float* coef_std = nullptr;
     float* w_out = nullptr;                   // [n_out] loss weights of the current stage
     // training buffers (batch rows)
-    bf16 *X0 = nullptr, *X0T = nullptr;
-    float* Z[4] = {};
+    bf16 *X0 = nullptr, *dY = nullptr;
+    float* Z[4] = {};                         // GELU'(z) of the hidden layers
     bf16* A[4] = {};
-    bf16* AT[4] = {};
-    float* Y = nullptr;
-    float* T = nullptr;
-    bf16 *dY = nullptr, *dYT = nullptr;
     bf16* dZ[4] = {};
-    bf16* dZT[4] = {};
+    soap::mlp::Weights maps{};                // TMA maps of the weights and of the training buffers
+    soap::mlp::Step step{};
     int* perm = nullptr;
     int64_t perm_cap = 0;
     int* d_step = nullptr;                    // [0] step within the epoch, [1] Adam step t
@@ -81,12 +78,9 @@ struct soap_surrogate {
     // training graph (captured per (data pointers, steps per epoch, stage))
     cudaGraphExec_t graph = nullptr;
     std::vector<uint64_t> graph_key;
-    // query buffers (chunk rows)
+    // query buffer (chunk rows)
     int q_cap = 0;
-    bf16 *qa = nullptr, *qb = nullptr;        // ping-pong activations [q_cap][256]
-    float* qy = nullptr;                      // [q_cap][n_out_pad]
     bf16* qsplit = nullptr;                   // [q_cap][3 n_coef]
-    bf16* qx0 = nullptr;                      // [q_cap][n_in] scaled query inputs
     // basis
     int64_t n_px = 0;
     float* mu = nullptr;                      // [n_px]
@@ -100,69 +94,6 @@ namespace sur {
 // ---------------------------------------------------------------------------------------
 // kernels
 // ---------------------------------------------------------------------------------------
-__device__ __forceinline__ float scale_in(float x, float lo, float hi) { return 2.0f * (x - lo) / (hi - lo) - 1.0f; }
-
-// Batch rows from the shuffled data set: scaled inputs (BF16, row-major and transposed) and
-// targets.  Step s of the epoch takes perm[s*B .. s*B + B).
-__global__ void k_gather(const float* __restrict__ x, const float* __restrict__ t, const int* __restrict__ perm,
-                         const int* __restrict__ d_step, int B, int n_in, int n_out, const float* __restrict__ lohi,
-                         bf16* __restrict__ X0, bf16* __restrict__ X0T, float* __restrict__ T) {
-    const int r = blockIdx.x;
-    const int src = perm[(int64_t)d_step[0] * B + r];
-    for (int i = threadIdx.x; i < n_in; i += blockDim.x) {
-        const bf16 v = __float2bfloat16_rn(scale_in(x[(int64_t)src * n_in + i], lohi[i], lohi[n_in + i]));
-        X0[(int64_t)r * n_in + i] = v;
-        X0T[(int64_t)i * B + r] = v;
-    }
-    for (int j = threadIdx.x; j < n_out; j += blockDim.x) T[(int64_t)r * n_out + j] = t[(int64_t)src * n_out + j];
-}
-
-// L = sum_b sum_j w_j (y - t)^2 / B; dY = bf16(2 w_j (y - t) / B), row-major and transposed
-// (zero in the padding columns j >= n_out).
-__global__ void k_loss(const float* __restrict__ Y, int ldy, const float* __restrict__ T, int n_out, int n_pad, int B,
-                       const float* __restrict__ w, bf16* __restrict__ dY, bf16* __restrict__ dYT, double* loss) {
-    __shared__ double s_part[8];
-    double part = 0;
-    const int64_t n_el = (int64_t)B * n_pad;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n_el; e += (int64_t)gridDim.x * blockDim.x) {
-        const int r = (int)(e / n_pad), j = (int)(e % n_pad);
-        float d = 0.0f;
-        if (j < n_out) {
-            const float res = Y[(int64_t)r * ldy + j] - T[(int64_t)r * n_out + j];
-            part += (double)w[j] * (double)res * (double)res;
-            d = 2.0f * w[j] * res / (float)B;
-        }
-        const bf16 v = __float2bfloat16_rn(d);
-        dY[(int64_t)r * n_pad + j] = v;
-        dYT[(int64_t)j * B + r] = v;
-    }
-    for (int o = 16; o > 0; o >>= 1) part += __shfl_down_sync(0xffffffffu, part, o);
-    if ((threadIdx.x & 31) == 0) s_part[threadIdx.x >> 5] = part;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double s = 0;
-        for (int k = 0; k < (int)(blockDim.x >> 5); k++) s += s_part[k];
-        atomicAdd(loss, s / B);
-    }
-}
-
-// Bias gradients: db[o] = sum_b g[o][b] over the transposed BF16 gradients of one layer.
-struct BiasJobs {
-    const bf16* gT[kLayers];
-    int rows[kLayers];
-    float* db[kLayers];
-};
-__global__ void k_bias_grad(BiasJobs jobs, int B) {
-    const int l = blockIdx.y;
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (warp >= jobs.rows[l]) return;
-    const bf16* row = jobs.gT[l] + (int64_t)warp * B;
-    float s = 0.0f;
-    for (int b = lane; b < B; b += 32) s += __bfloat162float(row[b]);
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if (lane == 0) jobs.db[l][warp] = s;
-}
-
 // Adam (Kingma & Ba 2015, Algorithm 1) over the flat parameters, then the BF16 copies W and
 // W^T.  mode 0 updates everything except the RV-error head (row n_coef of the last layer and its
 // bias), mode 1 only the head, mode 2 everything.
@@ -170,7 +101,7 @@ __global__ void k_adam(float* __restrict__ P, const float* __restrict__ G, float
                        float* __restrict__ V, int64_t n, const int* __restrict__ d_step, const float* __restrict__ d_lr,
                        float b1, float b2, float eps, int mode, int64_t head_w0, int head_len, int64_t head_b,
                        LayerTable lt) {
-    const int t = d_step[1] + 1;
+    const int t = d_step[1];                             // counted by the gradient kernel before
     const float lr = d_lr[0];
     const float c1 = 1.0f - powf(b1, (float)t), c2 = 1.0f - powf(b2, (float)t);
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
@@ -196,11 +127,6 @@ __global__ void k_adam(float* __restrict__ P, const float* __restrict__ G, float
     }
 }
 
-__global__ void k_step_inc(int* d_step, int steps_per_epoch) {
-    d_step[0] = (d_step[0] + 1) % steps_per_epoch;
-    d_step[1] += 1;
-}
-
 // BF16 copies of all weights from the FP32 master (after set_params).
 __global__ void k_cast_weights(const float* __restrict__ P, LayerTable lt) {
     const int l = blockIdx.y;
@@ -210,47 +136,6 @@ __global__ void k_cast_weights(const float* __restrict__ P, LayerTable lt) {
         const bf16 wb = __float2bfloat16_rn(P[lt.offW[l] + q]);
         lt.Wb[l][q] = wb;
         lt.WbT[l][(int64_t)i * lt.out_pad[l] + o] = wb;
-    }
-}
-
-// Query inputs: scaled BF16 rows and the in-range flag (every input inside [lo, hi]).
-__global__ void k_query_in(const float* __restrict__ x, int64_t n, int n_in, const float* __restrict__ lohi,
-                           bf16* __restrict__ X0, uint8_t* __restrict__ in_range) {
-    for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < n; r += (int64_t)gridDim.x * blockDim.x) {
-        bool ok = true;
-        for (int i = 0; i < n_in; i++) {
-            const float v = x[r * n_in + i];
-            ok = ok && v >= lohi[i] && v <= lohi[n_in + i];
-            X0[r * n_in + i] = __float2bfloat16_rn(scale_in(v, lohi[i], lohi[n_in + i]));
-        }
-        if (in_range) in_range[r] = ok ? 1 : 0;
-    }
-}
-
-// Network outputs -> coefficients in data units, predicted RV error (cm/s), acceptance, and the
-// split-BF16 rows [c_hi c_hi c_lo] for the reconstruction GEMM.
-__global__ void k_query_out(const float* __restrict__ Y, int ldy, const float* __restrict__ Yerr, int ldyerr,
-                            int64_t n, int n_coef, const float* __restrict__ mean,
-                            const float* __restrict__ sd, float thr_cms, uint8_t* __restrict__ accept,
-                            float* __restrict__ pred_err, float* __restrict__ coef_out, bf16* __restrict__ split) {
-    const int64_t n_el = n * (n_coef + 1);
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n_el; e += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t r = e / (n_coef + 1);
-        const int j = (int)(e % (n_coef + 1));
-        const float y = Y[r * ldy + j];
-        if (j == n_coef) {
-            const float err = exp10f(Yerr[r * ldyerr + j]);
-            if (pred_err) pred_err[r] = err;
-            if (accept) accept[r] = (accept[r] && err <= thr_cms) ? 1 : 0;
-            continue;
-        }
-        const float c = y * sd[j] + mean[j];
-        if (coef_out) coef_out[r * n_coef + j] = c;
-        const bf16 hi = __float2bfloat16_rn(c);
-        const bf16 lo = __float2bfloat16_rn(c - __bfloat162float(hi));
-        split[r * 3 * n_coef + j] = hi;
-        split[r * 3 * n_coef + n_coef + j] = hi;
-        split[r * 3 * n_coef + 2 * n_coef + j] = lo;
     }
 }
 
@@ -510,71 +395,25 @@ static LayerTable table(const soap_surrogate* s) {
     return lt;
 }
 
-// Forward pass of B rows from X0 (BF16 [B][n_in]).  Training keeps z (FP32), a (BF16) and a^T;
-// inference ping-pongs a between qa and qb.  Output y [B][n_out_pad] FP32.
-static soap_status forward(soap_surrogate* s, const bf16* X0, int B, bool train, float* Yout) {
-    const bf16* a = X0;
-    int64_t lda = s->n_in;
-    for (int l = 0; l < kLayers; l++) {
-        const Layer& L = s->L[l];
-        tc::Epilogue ep{};
-        ep.bias = s->P + L.offb;
-        if (l < kLayers - 1) {
-            ep.flags = tc::EPI_BIAS | tc::EPI_GELU | tc::EPI_A16;
-            if (train) {
-                ep.flags |= tc::EPI_Z32 | tc::EPI_A16T;
-                ep.c32 = s->Z[l]; ep.ldc32 = L.out;
-                ep.c16 = s->A[l]; ep.ldc16 = L.out;
-                ep.c16t = s->AT[l]; ep.ldc16t = B;
-            } else {
-                ep.c16 = (l % 2 == 0) ? s->qa : s->qb; ep.ldc16 = L.out;
-            }
-        } else {
-            ep.flags = tc::EPI_BIAS | tc::EPI_A32;
-            ep.c32 = Yout; ep.ldc32 = s->n_out_pad;
-        }
-        SOAP_TRY(tc::gemm_tn(a, lda, L.Wb, L.in, B, L.out, L.in, ep, s->stream, s->flags));
-        a = train ? s->A[l] : ((l % 2 == 0) ? s->qa : s->qb);
-        lda = L.out;
-    }
-    return SOAP_OK;
-}
-
-// Loss, backward pass and bias gradients for the batch in the training buffers; gradients into G.
-static soap_status backward(soap_surrogate* s, int B) {
-    const int blocks = grid1((int64_t)B * s->n_out_pad);
-    k_loss<<<blocks, 256, 0, s->stream>>>(s->Y, s->n_out_pad, s->T, s->n_out, s->n_out_pad, B, s->w_out, s->dY,
-                                          s->dYT, s->d_loss);
-    const bf16* g = s->dY;        // gradient wrt the outputs of layer l (row-major)
-    const bf16* gT = s->dYT;
-    int64_t ldg = s->n_out_pad;
-    BiasJobs bj{};
-    for (int l = kLayers - 1; l >= 0; l--) {
-        const Layer& L = s->L[l];
-        // dW_l = g^T a_{l-1}:  A = g^T [out][B], B = a_{l-1}^T [in][B]
-        tc::Epilogue ew{};
-        ew.flags = tc::EPI_A32;
-        ew.c32 = s->G + L.offW; ew.ldc32 = L.in;
-        const bf16* aT = l == 0 ? s->X0T : s->AT[l - 1];
-        SOAP_TRY(tc::gemm_tn(gT, B, aT, B, L.out, L.in, B, ew, s->stream, s->flags));
-        bj.gT[l] = gT; bj.rows[l] = L.out; bj.db[l] = s->G + L.offb;
-        if (l == 0) break;
-        // dz_{l-1} = (g W_l) * GELU'(z_{l-1}):  A = g [B][out_pad], B = W_l^T [in][out_pad]
-        tc::Epilogue ed{};
-        ed.flags = tc::EPI_DGELU | tc::EPI_A16 | tc::EPI_A16T;
-        ed.zin = s->Z[l - 1]; ed.ldzin = L.in;
-        ed.c16 = s->dZ[l - 1]; ed.ldc16 = L.in;
-        ed.c16t = s->dZT[l - 1]; ed.ldc16t = B;
-        SOAP_TRY(tc::gemm_tn(g, ldg, L.WbT, L.out_pad, B, L.in, L.out_pad, ed, s->stream, s->flags));
-        g = s->dZ[l - 1];
-        gT = s->dZT[l - 1];
-        ldg = L.in;
-    }
-    dim3 bg((unsigned)((std::max(s->hidden, s->n_out) * 32 + 255) / 256), kLayers);
-    k_bias_grad<<<bg, 256, 0, s->stream>>>(bj, B);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) { set_error("kernel launch failed: %s", cudaGetErrorString(e)); return SOAP_ECUDA; }
-    return SOAP_OK;
+// Forward, loss, backward and all gradients of one batch: rows perm[step B ..] of (x, t), or the
+// first B rows in order without perm.
+static soap_status gradients(soap_surrogate* s, const float* x, const float* t, const int* perm, int steps,
+                             bool advance) {
+    mlp::TrainArgs a{};
+    a.w = s->maps;
+    a.s = s->step;
+    a.x = x; a.t = t; a.perm = perm;
+    a.d_step = s->d_step;
+    a.lohi = s->d_lohi; a.w_out = s->w_out; a.loss = s->d_loss;
+    a.B = s->batch;
+    SOAP_TRY(mlp::train_step(a, s->stream, s->flags));
+    mlp::DwArgs d{};
+    d.s = s->step;
+    d.G = s->G;
+    for (int l = 0; l < kLayers; l++) { d.offW[l] = s->L[l].offW; d.offb[l] = s->L[l].offb; }
+    d.d_step = s->d_step;
+    d.B = s->batch; d.steps = steps; d.advance = advance ? 1 : 0;
+    return mlp::weight_grads(d, s->stream, s->flags);
 }
 
 static soap_status alloc(void** p, size_t bytes) {
@@ -586,38 +425,35 @@ static soap_status alloc(void** p, size_t bytes) {
 static soap_status ensure_query(soap_surrogate* s, int rows) {
     if (rows <= s->q_cap) return SOAP_OK;
     cudaStreamSynchronize(s->stream);
-    cudaFree(s->qa); cudaFree(s->qb); cudaFree(s->qy); cudaFree(s->qsplit); cudaFree(s->qx0);
-    s->qa = s->qb = nullptr; s->qy = nullptr; s->qsplit = nullptr; s->qx0 = nullptr; s->q_cap = 0;
-    SOAP_TRY(alloc((void**)&s->qa, (size_t)rows * s->hidden * sizeof(bf16)));
-    SOAP_TRY(alloc((void**)&s->qb, (size_t)rows * s->hidden * sizeof(bf16)));
-    SOAP_TRY(alloc((void**)&s->qy, (size_t)rows * s->n_out_pad * sizeof(float)));
+    cudaFree(s->qsplit);
+    s->qsplit = nullptr; s->q_cap = 0;
     SOAP_TRY(alloc((void**)&s->qsplit, (size_t)rows * 3 * s->n_coef * sizeof(bf16)));
-    SOAP_TRY(alloc((void**)&s->qx0, (size_t)rows * s->n_in * sizeof(bf16)));
     s->q_cap = rows;
     return SOAP_OK;
 }
 
-// The error network (if any) runs on the same scaled inputs, on the main network's stream.
-static soap_status error_net_forward(soap_surrogate* s, const bf16* X0, int m) {
-    if (!s->error_net) return SOAP_OK;
-    soap_surrogate* j = s->error_net;
-    SOAP_TRY(ensure_query(j, s->q_cap));
-    const cudaStream_t saved = j->stream;
-    j->stream = s->stream;
-    const soap_status st = forward(j, X0, m, false, j->qy);
-    j->stream = saved;
-    return st;
+// Network outputs of n queries: whichever of the outputs are wanted (the error network, if any,
+// predicts the RV error from the same inputs).
+static soap_status network(soap_surrogate* s, const float* x, int64_t n, float thr_cms, uint8_t* accept,
+                           float* pred_err, float* coef, bf16* split) {
+    mlp::QueryArgs a{};
+    a.w[0] = s->maps;
+    a.w[1] = s->error_net ? s->error_net->maps : s->maps;
+    a.nets = s->error_net ? 2 : 1;
+    a.x = x; a.n = n;
+    a.lohi = s->d_lohi;
+    a.mean = s->coef_mean; a.sd = s->coef_std;
+    a.thr_cms = thr_cms;
+    a.accept = accept; a.pred_err = pred_err; a.coef = coef; a.split = split;
+    return mlp::query(a, s->stream, s->flags);
 }
 
 static soap_status check(soap_surrogate* s) {
-    unsigned int h = 0, hj = 0;
+    unsigned int h = 0;
     SOAP_CUDA(cudaMemcpyAsync(&h, s->flags, sizeof(h), cudaMemcpyDeviceToHost, s->stream));
-    if (s->error_net) SOAP_CUDA(cudaMemcpyAsync(&hj, s->error_net->flags, sizeof(hj), cudaMemcpyDeviceToHost, s->stream));
     SOAP_CUDA(cudaStreamSynchronize(s->stream));
-    h |= hj;
     if (h) {
         SOAP_CUDA(cudaMemsetAsync(s->flags, 0, sizeof(unsigned int), s->stream));
-        if (s->error_net) SOAP_CUDA(cudaMemsetAsync(s->error_net->flags, 0, sizeof(unsigned int), s->stream));
         set_error("a tensor-core kernel gave up waiting (status 0x%x)", h);
         return SOAP_ETIMEOUT;
     }
@@ -626,17 +462,14 @@ static soap_status check(soap_surrogate* s) {
 
 static void free_all(soap_surrogate* s) {
     if (s->graph) cudaGraphExecDestroy(s->graph);
-    void* ptrs[] = {s->P, s->G, s->Mo, s->Vo, s->wbuf, s->d_lohi, s->coef_mean, s->coef_std, s->w_out, s->X0, s->X0T,
-                    s->Y, s->T, s->dY, s->dYT, s->perm, s->d_step, s->d_lr, s->d_loss, s->flags, s->qa, s->qb,
-                    s->qy, s->qsplit, s->qx0, s->mu, s->vsplit};
+    void* ptrs[] = {s->P, s->G, s->Mo, s->Vo, s->wbuf, s->d_lohi, s->coef_mean, s->coef_std, s->w_out, s->X0,
+                    s->dY, s->perm, s->d_step, s->d_lr, s->d_loss, s->flags, s->qsplit, s->mu, s->vsplit};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     for (int l = 0; l < 4; l++) {
         if (s->Z[l]) cudaFree(s->Z[l]);
         if (s->A[l]) cudaFree(s->A[l]);
-        if (s->AT[l]) cudaFree(s->AT[l]);
         if (s->dZ[l]) cudaFree(s->dZ[l]);
-        if (s->dZT[l]) cudaFree(s->dZT[l]);
     }
 }
 
@@ -682,14 +515,13 @@ soap_status soap_surrogate_create(const soap_surrogate_desc* d, void* cuda_strea
     A_(s->wbuf, nwb * sizeof(bf16));
     A_(s->d_lohi, 2 * s->n_in * 4);
     A_(s->coef_mean, s->n_coef * 4); A_(s->coef_std, s->n_coef * 4); A_(s->w_out, s->n_out * 4);
-    A_(s->X0, (size_t)B * s->n_in * sizeof(bf16)); A_(s->X0T, (size_t)B * s->n_in * sizeof(bf16));
+    A_(s->X0, (size_t)B * s->n_in * sizeof(bf16));
     for (int l = 0; l < 4; l++) {
         A_(s->Z[l], (size_t)B * s->hidden * 4);
-        A_(s->A[l], (size_t)B * s->hidden * sizeof(bf16)); A_(s->AT[l], (size_t)B * s->hidden * sizeof(bf16));
-        A_(s->dZ[l], (size_t)B * s->hidden * sizeof(bf16)); A_(s->dZT[l], (size_t)B * s->hidden * sizeof(bf16));
+        A_(s->A[l], (size_t)B * s->hidden * sizeof(bf16));
+        A_(s->dZ[l], (size_t)B * s->hidden * sizeof(bf16));
     }
-    A_(s->Y, (size_t)B * s->n_out_pad * 4); A_(s->T, (size_t)B * s->n_out * 4);
-    A_(s->dY, (size_t)B * s->n_out_pad * sizeof(bf16)); A_(s->dYT, (size_t)B * s->n_out_pad * sizeof(bf16));
+    A_(s->dY, (size_t)B * s->n_out_pad * sizeof(bf16));
     A_(s->d_step, 2 * sizeof(int)); A_(s->d_lr, sizeof(float)); A_(s->d_loss, sizeof(double));
     A_(s->flags, sizeof(unsigned int));
 #undef A_
@@ -699,6 +531,17 @@ soap_status soap_surrogate_create(const soap_surrogate_desc* d, void* cuda_strea
         Layer& L = s->L[l];
         L.Wb = wp; wp += (int64_t)L.out * L.in;
         L.WbT = wp; wp += (int64_t)L.in * L.out_pad;
+    }
+    {
+        const bf16 *W[kLayers], *WT[kLayers];
+        const float* bias[kLayers];
+        for (int l = 0; l < kLayers; l++) { W[l] = s->L[l].Wb; WT[l] = s->L[l].WbT; bias[l] = s->P + s->L[l].offb; }
+        bf16* act[kLayers] = {s->X0, s->A[0], s->A[1], s->A[2], s->A[3]};
+        bf16* grad[kLayers] = {s->dZ[0], s->dZ[1], s->dZ[2], s->dZ[3], s->dY};
+        st = mlp::weight_maps(s->maps, W, WT, bias);
+        if (st == SOAP_OK) st = mlp::step_maps(s->step, act, grad, B);
+        for (int l = 0; l < 4; l++) s->step.grad[l] = s->Z[l];
+        if (st != SOAP_OK) { free_all(s); delete s; return st; }
     }
     float lohi[32];
     for (int i = 0; i < s->n_in; i++) { lohi[i] = s->lo[i]; lohi[s->n_in + i] = s->hi[i]; }
@@ -765,21 +608,10 @@ soap_status soap_surrogate_gradients(soap_surrogate* s, const float* x, const fl
     clear_error();
     if (!s || !x || !t || !w_out || !loss || !grads) { set_error("NULL argument"); return SOAP_EINVAL; }
     if (n != s->batch) { set_error("n must equal the batch size (%d)", s->batch); return SOAP_EINVAL; }
-    std::vector<int> perm(n);
-    std::iota(perm.begin(), perm.end(), 0);
-    if (s->perm_cap < n) {
-        if (s->perm) cudaFree(s->perm);
-        SOAP_TRY(alloc((void**)&s->perm, (size_t)n * sizeof(int)));
-        s->perm_cap = n;
-    }
-    SOAP_CUDA(cudaMemcpyAsync(s->perm, perm.data(), (size_t)n * 4, cudaMemcpyHostToDevice, s->stream));
     SOAP_CUDA(cudaMemcpyAsync(s->w_out, w_out, s->n_out * 4, cudaMemcpyHostToDevice, s->stream));
     SOAP_CUDA(cudaMemsetAsync(s->d_step, 0, sizeof(int), s->stream));
     SOAP_CUDA(cudaMemsetAsync(s->d_loss, 0, sizeof(double), s->stream));
-    k_gather<<<n, 32, 0, s->stream>>>(x, t, s->perm, s->d_step, n, s->n_in, s->n_out, s->d_lohi, s->X0, s->X0T, s->T);
-    SOAP_CUDA(cudaGetLastError());
-    SOAP_TRY(forward(s, s->X0, n, true, s->Y));
-    SOAP_TRY(backward(s, n));
+    SOAP_TRY(gradients(s, x, t, nullptr, 1, false));
     SOAP_CUDA(cudaMemcpyAsync(loss, s->d_loss, sizeof(double), cudaMemcpyDeviceToHost, s->stream));
     SOAP_CUDA(cudaMemcpyAsync(grads, s->G, s->n_params * 4, cudaMemcpyDeviceToHost, s->stream));
     return check(s);
@@ -819,14 +651,10 @@ soap_status soap_surrogate_train(soap_surrogate* s, const float* x, const float*
         soap_status st = SOAP_OK;
         cudaGraph_t graph = nullptr;
         if (e == cudaSuccess) {
-            k_gather<<<B, 32, 0, cap>>>(x, t, s->perm, s->d_step, B, s->n_in, s->n_out, s->d_lohi, s->X0, s->X0T, s->T);
-            st = forward(s, s->X0, B, true, s->Y);
-            if (st == SOAP_OK) st = backward(s, B);
-            if (st == SOAP_OK) {
+            st = gradients(s, x, t, s->perm, steps, true);
+            if (st == SOAP_OK)
                 k_adam<<<grid1(s->n_params), 256, 0, cap>>>(s->P, s->G, s->Mo, s->Vo, s->n_params, s->d_step, s->d_lr,
                                                              0.9f, 0.999f, 1e-8f, stage, head_w0, last.in, head_b, table(s));
-                k_step_inc<<<1, 1, 0, cap>>>(s->d_step, steps);
-            }
             const cudaError_t e2 = cudaStreamEndCapture(cap, &graph);
             if (e == cudaSuccess) e = e2;
         }
@@ -861,25 +689,7 @@ soap_status soap_surrogate_predict(soap_surrogate* s, const float* x, int64_t n,
     clear_error();
     if (!s || !x) { set_error("NULL argument"); return SOAP_EINVAL; }
     if (n <= 0) return SOAP_OK;
-    const int chunk = 65536;
-    SOAP_TRY(ensure_query(s, (int)std::min<int64_t>(n, chunk)));
-    bf16* X0 = s->qx0;
-    soap_status st = SOAP_OK;
-    for (int64_t r0 = 0; r0 < n && st == SOAP_OK; r0 += chunk) {
-        const int m = (int)std::min<int64_t>(chunk, n - r0);
-        k_query_in<<<grid1(m), 256, 0, s->stream>>>(x + r0 * s->n_in, m, s->n_in, s->d_lohi, X0,
-                                                    accepted ? accepted + r0 : nullptr);
-        st = forward(s, X0, m, false, s->qy);
-        if (st == SOAP_OK) st = error_net_forward(s, X0, m);
-        if (st != SOAP_OK) break;
-        const float* ye = s->error_net ? s->error_net->qy : s->qy;
-        k_query_out<<<grid1((int64_t)m * (s->n_coef + 1)), 256, 0, s->stream>>>(
-            s->qy, s->n_out_pad, ye, s->n_out_pad, m, s->n_coef, s->coef_mean, s->coef_std, rv_err_max_cms,
-            accepted ? accepted + r0 : nullptr, pred_err_cms ? pred_err_cms + r0 : nullptr,
-            coef ? coef + r0 * s->n_coef : nullptr, s->qsplit);
-    }
-    SOAP_CUDA(cudaGetLastError());
-    if (st != SOAP_OK) return st;
+    SOAP_TRY(network(s, x, n, rv_err_max_cms, accepted, pred_err_cms, coef, nullptr));
     return check(s);
 }
 
@@ -921,18 +731,12 @@ soap_status soap_surrogate_query(soap_surrogate* s, const float* x, int64_t n, f
     if (n <= 0) return SOAP_OK;
     const int chunk = 65536;
     SOAP_TRY(ensure_query(s, (int)std::min<int64_t>(n, chunk)));
-    bf16* X0 = s->qx0;
     soap_status st = SOAP_OK;
     for (int64_t r0 = 0; r0 < n && st == SOAP_OK; r0 += chunk) {
         const int m = (int)std::min<int64_t>(chunk, n - r0);
-        k_query_in<<<grid1(m), 256, 0, s->stream>>>(x + r0 * s->n_in, m, s->n_in, s->d_lohi, X0, accepted + r0);
-        st = forward(s, X0, m, false, s->qy);
-        if (st == SOAP_OK) st = error_net_forward(s, X0, m);
+        st = network(s, x + r0 * s->n_in, m, rv_err_max_cms, accepted + r0, pred_err_cms ? pred_err_cms + r0 : nullptr,
+                     nullptr, s->qsplit);
         if (st != SOAP_OK) break;
-        const float* ye = s->error_net ? s->error_net->qy : s->qy;
-        k_query_out<<<grid1((int64_t)m * (s->n_coef + 1)), 256, 0, s->stream>>>(
-            s->qy, s->n_out_pad, ye, s->n_out_pad, m, s->n_coef, s->coef_mean, s->coef_std, rv_err_max_cms,
-            accepted + r0, pred_err_cms ? pred_err_cms + r0 : nullptr, nullptr, s->qsplit);
         tc::Epilogue ep{};
         ep.flags = tc::EPI_BIAS | tc::EPI_A32;
         ep.bias = s->mu;

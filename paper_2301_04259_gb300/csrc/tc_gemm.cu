@@ -22,8 +22,7 @@ static PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
 }
 
 // Row-major BF16 matrix [rows][cols] with row stride ld (elements), boxes of box_rows x 64.
-static soap_status make_map(CUtensorMap* map, const void* base, int64_t rows, int64_t cols, int64_t ld,
-                            int box_rows) {
+soap_status operand_map(CUtensorMap* map, const void* base, int64_t rows, int64_t cols, int64_t ld, int box_rows) {
     auto fn = encode_fn();
     if (!fn) { set_error("cuTensorMapEncodeTiled is not available from the driver"); return SOAP_ECUDA; }
     if ((reinterpret_cast<uintptr_t>(base) & 15) || (ld * 2) % 16 || ld < cols) {
@@ -86,8 +85,8 @@ soap_status gemm_tn(const __nv_bfloat16* A, int64_t lda, const __nv_bfloat16* B,
     if (M <= 0 || N <= 0 || K <= 0) { set_error("GEMM sizes must be positive"); return SOAP_EINVAL; }
     const int BN = N <= 64 ? 64 : (N <= 128 ? 128 : 256);
     CUtensorMap ma, mb;
-    SOAP_TRY(make_map(&ma, A, M, K, lda, BM));
-    SOAP_TRY(make_map(&mb, B, N, K, ldb, BN));
+    SOAP_TRY(operand_map(&ma, A, M, K, lda, BM));
+    SOAP_TRY(operand_map(&mb, B, N, K, ldb, BN));
     if (BN == 64) return launch<64>(ma, mb, M, N, K, ep, st, flags);
     if (BN == 128) return launch<128>(ma, mb, M, N, K, ep, st, flags);
     return launch<256>(ma, mb, M, N, K, ep, st, flags);

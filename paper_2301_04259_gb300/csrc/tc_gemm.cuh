@@ -318,6 +318,10 @@ k_gemm_tn(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUt
     }
 }
 
+// Row-major BF16 matrix [rows][cols] with row stride ld (elements): boxes of box_rows x 64, 128-byte
+// swizzle, zero fill outside.
+soap_status operand_map(CUtensorMap* map, const void* base, int64_t rows, int64_t cols, int64_t ld, int box_rows);
+
 // Tiled tensor map without swizzle (BF16 elements unless dt says otherwise): dims[0] innermost
 // (elements), strides in bytes of dims 1 .. rank-1, box in elements.  Zero fill outside the tensor.
 soap_status encode_map(CUtensorMap* map, int rank, const void* base, const uint64_t* dims,
