@@ -738,10 +738,9 @@ soap_status soap_surrogate_query(soap_surrogate* s, const float* x, int64_t n, f
                      nullptr, s->qsplit);
         if (st != SOAP_OK) break;
         tc::Epilogue ep{};
-        ep.flags = tc::EPI_BIAS | tc::EPI_A32;
         ep.bias = s->mu;
-        ep.c32 = out + r0 * s->n_px;
-        ep.ldc32 = s->n_px;
+        ep.c = out + r0 * s->n_px;
+        ep.ldc = s->n_px;
         st = tc::gemm_tn(s->qsplit, 3 * s->n_coef, s->vsplit, 3 * s->n_coef, m, (int)s->n_px, 3 * s->n_coef, ep,
                          s->stream, s->flags);
     }
@@ -760,10 +759,9 @@ soap_status soap_surrogate_reconstruct(soap_surrogate* s, const float* coef, int
         k_split_rows<<<grid1((int64_t)m * s->n_coef), 256, 0, s->stream>>>(coef + r0 * s->n_coef, m, s->n_coef,
                                                                            s->qsplit);
         tc::Epilogue ep{};
-        ep.flags = tc::EPI_BIAS | tc::EPI_A32;
         ep.bias = s->mu;
-        ep.c32 = out + r0 * s->n_px;
-        ep.ldc32 = s->n_px;
+        ep.c = out + r0 * s->n_px;
+        ep.ldc = s->n_px;
         SOAP_TRY(tc::gemm_tn(s->qsplit, 3 * s->n_coef, s->vsplit, 3 * s->n_coef, m, (int)s->n_px, 3 * s->n_coef,
                              ep, s->stream, s->flags));
     }

@@ -1,6 +1,7 @@
 // tc_gemm.cu -- host side of the tcgen05 BF16 GEMM: tensor maps, tile choice, launch.
 #include <cudaTypedefs.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "tc_gemm.cuh"
@@ -66,15 +67,15 @@ soap_status encode_map(CUtensorMap* map, int rank, const void* base, const uint6
 
 template <int BN>
 static soap_status launch(const CUtensorMap& ma, const CUtensorMap& mb, int M, int N, int K, const Epilogue& ep,
-                          cudaStream_t st, unsigned int* flags) {
+                          int sms, cudaStream_t st, unsigned int* flags) {
     static bool configured = false;     // per instantiation; attribute set is idempotent
     if (!configured) {
         SOAP_CUDA(cudaFuncSetAttribute(k_gemm_tn<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        Smem<BN>::kBytes));
         configured = true;
     }
-    dim3 grid((unsigned)((N + BN - 1) / BN), (unsigned)((M + BM - 1) / BM));
-    k_gemm_tn<BN><<<grid, kThreads, Smem<BN>::kBytes, st>>>(ma, mb, M, N, K, ep, flags);
+    const int64_t tiles = (int64_t)((M + BM - 1) / BM) * ((N + BN - 1) / BN);
+    k_gemm_tn<BN><<<(unsigned)std::min<int64_t>(tiles, sms), kThreads, Smem<BN>::kBytes, st>>>(ma, mb, M, N, K, ep, flags);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) { set_error("GEMM launch failed: %s", cudaGetErrorString(e)); return SOAP_ECUDA; }
     return SOAP_OK;
@@ -83,13 +84,19 @@ static soap_status launch(const CUtensorMap& ma, const CUtensorMap& mb, int M, i
 soap_status gemm_tn(const __nv_bfloat16* A, int64_t lda, const __nv_bfloat16* B, int64_t ldb, int M, int N,
                     int K, const Epilogue& ep, cudaStream_t st, unsigned int* flags) {
     if (M <= 0 || N <= 0 || K <= 0) { set_error("GEMM sizes must be positive"); return SOAP_EINVAL; }
-    const int BN = N <= 64 ? 64 : (N <= 128 ? 128 : 256);
+    int dev = 0, sms = 0;
+    SOAP_CUDA(cudaGetDevice(&dev));
+    SOAP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    // 256 columns per tile read the fewest operand bytes per output; with fewer such tiles than SMs
+    // narrower ones share the work out (7 x 16,834 x 384: 66 tiles of 256 columns, 132 of 128)
+    const int64_t tiles_m = (M + BM - 1) / BM;
+    const int BN = N <= 64 ? 64 : (N <= 128 || tiles_m * ((N + 255) / 256) < sms ? 128 : 256);
     CUtensorMap ma, mb;
     SOAP_TRY(operand_map(&ma, A, M, K, lda, BM));
     SOAP_TRY(operand_map(&mb, B, N, K, ldb, BN));
-    if (BN == 64) return launch<64>(ma, mb, M, N, K, ep, st, flags);
-    if (BN == 128) return launch<128>(ma, mb, M, N, K, ep, st, flags);
-    return launch<256>(ma, mb, M, N, K, ep, st, flags);
+    if (BN == 64) return launch<64>(ma, mb, M, N, K, ep, sms, st, flags);
+    if (BN == 128) return launch<128>(ma, mb, M, N, K, ep, sms, st, flags);
+    return launch<256>(ma, mb, M, N, K, ep, sms, st, flags);
 }
 
 }  // namespace tc
@@ -112,10 +119,10 @@ extern "C" soap_status soap_gemm_bf16_tn(int32_t M, int32_t N, int32_t K, const 
     SOAP_CUDA(cudaGetSymbolAddress((void**)&flags, g_gemm_flags));
     SOAP_CUDA(cudaMemsetAsync(flags, 0, sizeof(unsigned int), st));
     tc::Epilogue ep{};
-    ep.flags = tc::EPI_A32 | (bias ? tc::EPI_BIAS : 0) | (activation ? tc::EPI_GELU : 0);
     ep.bias = bias;
-    ep.c32 = C;
-    ep.ldc32 = ldc;
+    ep.gelu = activation;
+    ep.c = C;
+    ep.ldc = ldc;
     SOAP_TRY(tc::gemm_tn((const __nv_bfloat16*)A, lda, (const __nv_bfloat16*)B, ldb, M, N, K, ep, st, flags));
     unsigned int h = 0;
     SOAP_CUDA(cudaMemcpyAsync(&h, flags, sizeof(h), cudaMemcpyDeviceToHost, st));

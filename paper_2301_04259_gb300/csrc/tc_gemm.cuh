@@ -1,12 +1,16 @@
 // tc_gemm.cuh -- BF16 GEMM on the fifth-generation tensor cores (tcgen05) of sm_103a.
 //
-//   C[m][n] = epilogue( sum_k A[m][k] * B[n][k] )        ("TN": both operands K-contiguous)
+//   C[m][n] = act( sum_k A[m][k] * B[n][k] + bias[n] )        ("TN": both operands K-contiguous)
 //
-// One CTA computes a 128 x BN tile.  Warp 0 streams 128 x 64 (A) and BN x 64 (B) BF16 tiles
-// into shared memory with TMA (128-byte swizzle) through a ring of mbarriers (2 to 4 stages);
-// warp 1 owns the tensor-memory accumulator (128 lanes x BN FP32 columns) and issues
-// tcgen05.mma (M = 128, N = BN, K = 16 per instruction) from one thread; warps 2..5 read the
-// accumulator back with tcgen05.ld (one row per thread) and apply the epilogue.
+// Persistent: one CTA per SM takes 128 x BN output tiles in turn (columns fastest: the CTAs at work
+// share A panels and write neighbouring pieces of the same rows; 0.73 against 0.82 ms for the
+// product below with rows fastest).  Warp 0 streams 128 x 64 (A) and BN x 64 (B) BF16 tiles into
+// shared memory with TMA (128-byte swizzle) through a ring of mbarriers; warp 1 issues tcgen05.mma
+// (M = 128, N = BN, K = 16 per instruction) from one thread into one of two tensor-memory
+// accumulators (128 lanes x BN FP32 columns); warps 2 .. 9 read the other accumulator back and
+// write the tile through shared memory, 64 consecutive columns of a row per store instruction.
+// With one tile per CTA and four epilogue warps the wide product of the surrogate's reconstruction
+// (40,000 x 16,834 x 384, 2.69 GB out) waited on loads, MMAs and stores in turn: 1.89 ms.
 //
 // Every wait is bounded (about a second of clock cycles); a wait that gives up sets
 // kFlagTimeout in the caller's status word, the CTA stops issuing work, waits (bounded) for
@@ -16,6 +20,8 @@
 #include <cuda.h>
 #include <cuda_bf16.h>
 
+#include <type_traits>
+
 #include "soap_internal.cuh"
 
 namespace soap {
@@ -23,25 +29,14 @@ namespace tc {
 
 constexpr int BM = 128;        // rows per CTA (TMEM lanes)
 constexpr int BK = 64;         // K elements per stage: one 128-byte swizzle atom of BF16
-constexpr int kThreads = 192;
-// Pipeline depth per tile width: two CTAs fit on an SM (shared memory and 512 TMEM columns), so
-// one CTA's loads and MMAs overlap the other's epilogue.
-template <int BN> struct Stages { static constexpr int value = BN >= 256 ? 2 : (BN >= 128 ? 3 : 4); };
-
-// Epilogue: z = acc (+ bias[n]); a = GELU(z) when EPI_GELU, a = z * GELU'(zin[m][n]) when
-// EPI_DGELU, else a = z.  Outputs (any subset): c32 <- z (EPI_Z32) or a (EPI_A32), c16 <- bf16(a),
-// c16t[n][m] <- bf16(a) (transposed copy).
-enum Epi : int {
-    EPI_BIAS = 1, EPI_GELU = 2, EPI_DGELU = 4, EPI_Z32 = 8, EPI_A32 = 16, EPI_A16 = 32, EPI_A16T = 64
-};
+constexpr int kEpiWarps = 8;   // two column halves of each group of 32 accumulator lanes
+constexpr int kThreads = 64 + 32 * kEpiWarps;
+template <int BN> struct Stages { static constexpr int value = BN >= 256 ? 3 : (BN >= 128 ? 4 : 6); };
 
 struct Epilogue {
-    int flags;
-    const float* bias;
-    const float* zin; int64_t ldzin;
-    float* c32; int64_t ldc32;
-    __nv_bfloat16* c16; int64_t ldc16;
-    __nv_bfloat16* c16t; int64_t ldc16t;
+    const float* bias;          // [N] or NULL
+    int gelu;
+    float* c; int64_t ldc;
 };
 
 __device__ __forceinline__ float gelu(float z) { return 0.5f * z * (1.0f + erff(z * 0.70710678118654752f)); }
@@ -151,9 +146,11 @@ struct Smem {
     static constexpr int kA = BM * BK * 2;          // bytes per stage
     static constexpr int kB = BN * BK * 2;
     static constexpr int kStage = kA + kB;
-    static constexpr int kTile = 32 * 33 * 4;       // per epilogue warp: 32 x 32 floats, padded rows
-    static_assert(4 * kTile <= STAGES * kStage, "epilogue tiles reuse the operand ring");
-    static constexpr int kBytes = STAGES * kStage + 1024 /* alignment slack */ + 256 /* barriers */;
+    static constexpr int kCols = BN / 2 < 64 ? BN / 2 : 64;       // columns an epilogue warp stages at a time
+    static constexpr int kPitch = kCols + 2;        // floats: 8-byte pairs of 16 rows fall on distinct banks
+    static constexpr int kTile = 32 * kPitch * 4;
+    static constexpr int kBytes = STAGES * kStage + kEpiWarps * kTile + 1024 /* alignment slack */ + 256 /* barriers */;
+    static_assert(kBytes <= 227 * 1024, "shared memory of one CTA");
 };
 
 // Row-major store of a warp's 32 x 32 block through its shared tile: lane r holds row r's 32
@@ -179,36 +176,40 @@ __device__ __forceinline__ void store_rows(float (*tile)[33], const float (&v)[3
     __syncwarp();
 }
 
+// 40,000 x 16,834 x 384 (2.69 GB out): about 0.66 ms, 4.1 TB/s.  What bounds it there is the SM's
+// shared-memory path: per 128 x 256 tile the MMAs read 288 KB of operands, the copies fill as much,
+// and the output passes in and out (about 8,700 cycles at 128 bytes a cycle, of 9,100 measured;
+// HBM alone would allow 6,100).
 template <int BN>
-__global__ void __launch_bounds__(kThreads, 2)
+__global__ void __launch_bounds__(kThreads, 1)
 k_gemm_tn(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, int M, int N,
           int K, Epilogue ep, unsigned int* flags) {
-    static_assert(BN % 16 == 0 && BN >= 16 && BN <= 256, "tcgen05 N for M = 128");
-    constexpr int STAGES = Smem<BN>::STAGES;
+    static_assert(BN % 64 == 0 && BN <= 256, "tcgen05 N for M = 128, two accumulators in 512 columns");
+    using SM = Smem<BN>;
+    constexpr int STAGES = SM::STAGES;
     extern __shared__ unsigned char smem_raw[];
-    // 1024-byte aligned operand ring (the swizzle atom), barriers after it
+    // 1024-byte aligned operand ring (the swizzle atom), epilogue tiles and barriers after it
     unsigned char* ring = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-    uint64_t* full = reinterpret_cast<uint64_t*>(ring + STAGES * Smem<BN>::kStage);
+    unsigned char* tiles = ring + STAGES * SM::kStage;
+    uint64_t* full = reinterpret_cast<uint64_t*>(tiles + kEpiWarps * SM::kTile);
     uint64_t* empty = full + STAGES;
-    uint64_t* accum = empty + STAGES;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(accum + 1);
-    // epilogue tiles: the operand ring, free once the accumulator is complete (every copy has
-    // been consumed by an MMA that has finished)
-    float (*tiles)[32][33] = reinterpret_cast<float (*)[32][33]>(ring);
+    uint64_t* acc_full = empty + STAGES;               // [2] accumulator complete
+    uint64_t* acc_free = acc_full + 2;                 // [2] accumulator read back
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_free + 2);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int n0 = blockIdx.x * BN, m0 = blockIdx.y * BM;
     const int n_kb = (K + BK - 1) / BK;
-    constexpr uint32_t kCols = BN <= 32 ? 32 : (BN <= 64 ? 64 : (BN <= 128 ? 128 : 256));
+    const int tiles_n = (N + BN - 1) / BN;
+    const int64_t n_tiles = (int64_t)((M + BM - 1) / BM) * tiles_n;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; s++) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
-        mbar_init(accum, 1);
+        for (int b = 0; b < 2; b++) { mbar_init(&acc_full[b], 1); mbar_init(&acc_free[b], kEpiWarps); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                     ::"r"(smem_u32(tmem_slot)), "r"(kCols) : "memory");
+                     ::"r"(smem_u32(tmem_slot)), "r"(2 * BN) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -217,96 +218,131 @@ k_gemm_tn(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUt
     const uint32_t tmem = *tmem_slot;
 
     if (warp == 0 && lane == 0) {
-        // producer
-        int armed = 0;
+        // producer: it counts K blocks over all of this CTA's tiles
+        int64_t it = 0;
         bool ok = true;
-        for (int kb = 0; kb < n_kb && ok; kb++) {
-            const int s = kb % STAGES;
-            const uint32_t ph = (kb / STAGES) & 1;
-            if (!mbar_wait(&empty[s], ph ^ 1, flags)) { ok = false; break; }
-            unsigned char* a = ring + s * Smem<BN>::kStage;
-            mbar_expect_tx(&full[s], Smem<BN>::kStage);
-            tma_load_2d(a, &map_a, kb * BK, m0, &full[s]);
-            tma_load_2d(a + Smem<BN>::kA, &map_b, kb * BK, n0, &full[s]);
-            armed = kb + 1;
+        for (int64_t tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
+            const int m0 = (int)(tile / tiles_n) * BM, n0 = (int)(tile % tiles_n) * BN;
+            for (int kb = 0; kb < n_kb; kb++, it++) {
+                const int s = (int)(it % STAGES);
+                if (!mbar_wait(&empty[s], (uint32_t)((it / STAGES) & 1) ^ 1, flags)) { ok = false; break; }
+                unsigned char* a = ring + s * SM::kStage;
+                mbar_expect_tx(&full[s], SM::kStage);
+                tma_load_2d(a, &map_a, kb * BK, m0, &full[s]);
+                tma_load_2d(a + SM::kA, &map_b, kb * BK, n0, &full[s]);
+            }
         }
         // the last copies issued must land before the CTA may exit
-        for (int kb = armed - 1; kb >= 0 && kb >= armed - STAGES; kb--)
-            mbar_wait(&full[kb % STAGES], (kb / STAGES) & 1, flags);
+        for (int64_t k = it - 1; k >= 0 && k >= it - STAGES; k--)
+            mbar_wait(&full[k % STAGES], (uint32_t)((k / STAGES) & 1), flags);
     } else if (warp == 1 && lane == 0) {
         // MMA issuer
         constexpr uint32_t idesc = idesc_bf16(BN);
+        int64_t it = 0;
+        int n = 0;                                     // tiles so far
         bool ok = true;
-        int issued = 0;
-        for (int kb = 0; kb < n_kb; kb++) {
-            const int s = kb % STAGES;
-            if (!mbar_wait(&full[s], (kb / STAGES) & 1, flags)) { ok = false; break; }
+        for (int64_t tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x, n++) {
+            const int buf = n & 1;
+            if (!mbar_wait(&acc_free[buf], (uint32_t)((n >> 1) & 1) ^ 1, flags)) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t a = smem_u32(ring + s * Smem<BN>::kStage);
-            const uint32_t b = a + Smem<BN>::kA;
+            for (int kb = 0; kb < n_kb; kb++, it++) {
+                const int s = (int)(it % STAGES);
+                if (!mbar_wait(&full[s], (uint32_t)((it / STAGES) & 1), flags)) { ok = false; break; }
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                const uint32_t a = smem_u32(ring + s * SM::kStage);
+                const uint32_t b = a + SM::kA;
 #pragma unroll
-            for (int k = 0; k < BK / 16; k++)
-                mma_bf16(tmem, sdesc(a + k * 32), sdesc(b + k * 32), idesc, (kb | k) != 0);
-            mma_commit(&empty[s]);
-            issued = kb + 1;
+                for (int k = 0; k < BK / 16; k++)
+                    mma_bf16(tmem + (uint32_t)(buf * BN), sdesc(a + k * 32), sdesc(b + k * 32), idesc, (kb | k) != 0);
+                mma_commit(&empty[s]);
+            }
+            mma_commit(&acc_full[buf]);                // arrives once every MMA issued above has completed
         }
-        (void)ok;
-        mma_commit(accum);          // arrives once every MMA issued above has completed
-        mbar_wait(accum, 0, flags); // (bounded) before the tensor memory can be released
-        (void)issued;
+        // (bounded) every MMA has completed before the tensor memory can be released
+        for (int k = n - 1; k >= 0 && k >= n - 2; k--) mbar_wait(&acc_full[k & 1], (uint32_t)((k >> 1) & 1), flags);
     } else if (warp >= 2) {
-        // epilogue: TMEM lanes 32*(warp % 4) .. +31
-        const int lane_base = 32 * (warp & 3);
-        const int m = m0 + lane_base + lane;
-        // warp-uniform decision: tcgen05.ld is a warp-wide (.sync.aligned) instruction
-        const bool done = __all_sync(0xffffffffu, mbar_wait(accum, 0, flags));
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        if (done) {
-            float (*tile)[33] = tiles[warp - 2];
-            const int m_first = m0 + lane_base;
+        // epilogue: TMEM lanes 32 (warp % 4) .. +31, columns of one half of the tile.  Lane r holds
+        // row r's values; staged through the warp's tile, the lanes then run along the columns.
+        constexpr int C = SM::kCols;
+        const int lg = warp & 3, half = (warp - 2) >> 2;
+        float* mine = reinterpret_cast<float*>(tiles + (warp - 2) * SM::kTile);
+        const bool vec2 = (ep.ldc & 1) == 0 && (reinterpret_cast<uintptr_t>(ep.c) & 7) == 0;
+        int n = 0;
+        for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, n++) {
+            const int buf = n & 1;
+            const int m0 = (int)(tile / tiles_n) * BM + 32 * lg, n0 = (int)(tile % tiles_n) * BN + half * (BN / 2);
+            // warp-uniform decision: tcgen05.ld is a warp-wide (.sync.aligned) instruction
+            if (!__all_sync(0xffffffffu, mbar_wait(&acc_full[buf], (uint32_t)((n >> 1) & 1), flags))) break;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t src = tmem + ((uint32_t)(32 * lg) << 16) + (uint32_t)(buf * BN + half * (BN / 2));
 #pragma unroll 1
-            for (int c = 0; c < BN; c += 32) {
-                if (n0 + c >= N) break;
-                float v[32];
-                tmem_ld32(tmem + ((uint32_t)lane_base << 16) + (uint32_t)c, v);
-                float a[32];
-                if (ep.flags & EPI_DGELU) {
-                    // GELU'(z_in) at this block: staged through the tile so the reads are by row
-                    float zi[32];
-#pragma unroll 4
-                    for (int r = 0; r < 32; r++) {
-                        const int mm = m_first + r, nn = n0 + c + lane;
-                        tile[r][lane] = (mm < M && nn < N) ? ep.zin[(int64_t)mm * ep.ldzin + nn] : 0.0f;
-                    }
-                    __syncwarp();
+            for (int c = 0; c < BN / 2; c += C) {
 #pragma unroll
-                    for (int i = 0; i < 32; i++) zi[i] = tile[lane][i];
-                    __syncwarp();
+                for (int q = 0; q < C; q += 32) {
+                    float v[32];
+                    tmem_ld32(src + (uint32_t)(c + q), v);
 #pragma unroll
-                    for (int i = 0; i < 32; i++) {
-                        const float z = (ep.flags & EPI_BIAS) && n0 + c + i < N ? v[i] + ep.bias[n0 + c + i] : v[i];
-                        v[i] = z;
-                        a[i] = z * gelu_grad(zi[i]);
+                    for (int i = 0; i < 16; i++)
+                        *reinterpret_cast<float2*>(mine + lane * SM::kPitch + q + 2 * i) = make_float2(v[2 * i], v[2 * i + 1]);
+                }
+                if (c + C >= BN / 2) {                 // the accumulator is read: the next tile's MMAs may have it
+                    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0)
+                        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&acc_free[buf])) : "memory");
+                }
+                __syncwarp();
+                const int rows = min(32, M - m0), cols = min(C, N - n0 - c);
+                float* dst = ep.c + (int64_t)m0 * ep.ldc + n0 + c;
+                if (C == 64 && vec2 && rows == 32 && cols == 64) {
+                    // whole block: sixteen rows in flight, no branches
+                    const int j = 2 * lane;
+                    const float2 b = ep.bias ? make_float2(__ldg(ep.bias + n0 + c + j), __ldg(ep.bias + n0 + c + j + 1))
+                                             : make_float2(0.0f, 0.0f);
+                    float* d = dst + j;
+                    auto half_block = [&](int r0, auto with_bias, auto with_gelu) {
+                        float2 x[16];
+#pragma unroll
+                        for (int r = 0; r < 16; r++)
+                            x[r] = *reinterpret_cast<const float2*>(mine + (r0 + r) * SM::kPitch + j);
+#pragma unroll
+                        for (int r = 0; r < 16; r++) {
+                            if (with_bias) { x[r].x += b.x; x[r].y += b.y; }
+                            if (with_gelu) { x[r].x = gelu(x[r].x); x[r].y = gelu(x[r].y); }
+                            *reinterpret_cast<float2*>(d) = x[r];
+                            d += ep.ldc;
+                        }
+                    };
+                    const bool hb = ep.bias != nullptr;
+                    if (ep.gelu) { half_block(0, hb, true); half_block(16, hb, true); }
+                    else if (hb) { half_block(0, std::true_type{}, std::false_type{}); half_block(16, std::true_type{}, std::false_type{}); }
+                    else { half_block(0, std::false_type{}, std::false_type{}); half_block(16, std::false_type{}, std::false_type{}); }
+                } else if (C == 64 && vec2) {
+                    const int j = 2 * lane;
+                    const float b0 = ep.bias && j < cols ? __ldg(ep.bias + n0 + c + j) : 0.0f;
+                    const float b1 = ep.bias && j + 1 < cols ? __ldg(ep.bias + n0 + c + j + 1) : 0.0f;
+#pragma unroll 8
+                    for (int r = 0; r < rows; r++, dst += ep.ldc) {
+                        float2 x = *reinterpret_cast<const float2*>(mine + r * SM::kPitch + j);
+                        if (ep.bias) { x.x += b0; x.y += b1; }
+                        if (ep.gelu) { x.x = gelu(x.x); x.y = gelu(x.y); }
+                        if (j + 1 < cols) *reinterpret_cast<float2*>(dst + j) = x;
+                        else if (j < cols) dst[j] = x.x;
                     }
                 } else {
-#pragma unroll
-                    for (int i = 0; i < 32; i++) {
-                        const int n = n0 + c + i;
-                        const float z = (ep.flags & EPI_BIAS) && n < N ? v[i] + ep.bias[n] : v[i];
-                        v[i] = z;
-                        a[i] = (ep.flags & EPI_GELU) ? gelu(z) : z;
+#pragma unroll 1
+                    for (int j = lane; j < cols; j += 32) {
+                        const float b0 = ep.bias ? __ldg(ep.bias + n0 + c + j) : 0.0f;
+                        float* d = dst + j;
+#pragma unroll 4
+                        for (int r = 0; r < rows; r++, d += ep.ldc) {
+                            float x = mine[r * SM::kPitch + j];
+                            if (ep.bias) x += b0;
+                            *d = ep.gelu ? gelu(x) : x;
+                        }
                     }
                 }
-                if (ep.flags & EPI_Z32) store_rows(tile, v, lane, ep.c32, ep.ldc32, m_first, M, n0 + c, N);
-                if (ep.flags & EPI_A32) store_rows(tile, a, lane, ep.c32, ep.ldc32, m_first, M, n0 + c, N);
-                if (ep.flags & EPI_A16) store_rows(tile, a, lane, ep.c16, ep.ldc16, m_first, M, n0 + c, N);
-                if ((ep.flags & EPI_A16T) && m < M) {
-#pragma unroll
-                    for (int i = 0; i < 32; i++) {
-                        const int n = n0 + c + i;
-                        if (n < N) ep.c16t[(int64_t)n * ep.ldc16t + m] = __float2bfloat16_rn(a[i]);
-                    }
-                }
+                __syncwarp();
             }
         }
     }
@@ -314,7 +350,7 @@ k_gemm_tn(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUt
     __syncthreads();
     if (warp == 1) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kCols) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * BN) : "memory");
     }
 }
 
@@ -328,7 +364,7 @@ soap_status encode_map(CUtensorMap* map, int rank, const void* base, const uint6
                        const uint64_t* strides, const uint32_t* box,
                        CUtensorMapDataType dt = CU_TENSOR_MAP_DATA_TYPE_BFLOAT16);
 
-// C = epilogue(A B^T): A [M][K] (row stride lda), B [N][K] (row stride ldb), BF16, device, with
+// C = act(A B^T + bias): A [M][K] (row stride lda), B [N][K] (row stride ldb), BF16, device, with
 // 16-byte aligned bases and strides that are multiples of 8 elements.  Asynchronous on `st`.
 soap_status gemm_tn(const __nv_bfloat16* A, int64_t lda, const __nv_bfloat16* B, int64_t ldb, int M, int N,
                     int K, const Epilogue& ep, cudaStream_t st, unsigned int* flags);
