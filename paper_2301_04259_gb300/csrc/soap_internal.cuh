@@ -310,6 +310,13 @@ inline soap_status fit_dynamic_smem(Kernel kernel, size_t dynamic) {
     return SOAP_OK;
 }
 
+// PCA projection coef = (X - mean) basis^T on the tensor cores at FP32 accuracy (pca_tc.cu);
+// synchronises the stream
+namespace pca {
+soap_status project(const float* x, int64_t n, int64_t p, const float* mean, const float* basis, int k, float* coef,
+                    cudaStream_t st);
+}
+
 soap_status geometry_init(soap_ctx* c);                          // per-cell geometry + quiet kernels (on aux)
 soap_status join_geometry(soap_ctx* c);                          // main stream waits for a pending geometry
 

@@ -867,17 +867,7 @@ soap_status soap_pca_project(const float* X, int64_t n, int64_t p, const float* 
                              float* coef, void* cuda_stream) {
     clear_error();
     if (!X || !mean || !basis || !coef || n < 1 || p < 1 || k < 1) { set_error("invalid argument"); return SOAP_EINVAL; }
-    cudaStream_t st = (cudaStream_t)cuda_stream;
-    float* v = nullptr;
-    SOAP_TRY(alloc((void**)&v, (size_t)k * 4));
-    // coef = X basis^T - 1 (mu . basis^T)
-    soap_status rc = sgemm((int)n, k, p, 1.0f, X, p, 1, basis, 1, p, 0.0f, coef, k, st);
-    if (rc == SOAP_OK) rc = sgemm(1, k, p, 1.0f, mean, 0, 1, basis, 1, p, 0.0f, v, k, st);
-    if (rc == SOAP_OK) k_rank1_sub<<<grid1(n * k), 256, 0, st>>>(coef, k, n, k, nullptr, v, true);
-    cudaStreamSynchronize(st);
-    cudaFree(v);
-    if (rc == SOAP_OK && cudaGetLastError() != cudaSuccess) { set_error("PCA projection failed"); rc = SOAP_ECUDA; }
-    return rc;
+    return pca::project(X, n, p, mean, basis, k, coef, (cudaStream_t)cuda_stream);
 }
 
 }  // extern "C"
