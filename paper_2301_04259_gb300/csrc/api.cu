@@ -221,7 +221,7 @@ static void free_ctx_memory(soap_ctx* c) {
         if (p) cudaFree(p);
     DevBuf* bufs[] = {&c->stage_in, &c->fq, &c->contrast, &c->kphase, &c->jobs, &c->coefs, &c->job_counters,
                       &c->regions, &c->region_geo, &c->phases, &c->out_stage, &c->partial, &c->ccf.tmp,
-                      &c->ccf.tab, &c->lsf_taps, &c->lsf_tmp, &c->bis_tab, &c->tc_coef, &c->ccf.m,
+                      &c->ccf.tab, &c->lsf_taps, &c->lsf_tmp, &c->bis_tab, &c->tc_coef, &c->ccf.m, &c->ccf.ramp.tab,
                       &c->tm_planes, &c->tm_coef, &c->dir_cells, &c->dir_count, &c->dir_rows};
     for (DevBuf* b : bufs) release(*b);
     release_host(c->host_stage);

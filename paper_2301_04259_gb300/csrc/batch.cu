@@ -399,9 +399,9 @@ void batch_release(soap_ctx* c) {
                       &c->b_pblocks, &c->b_order, &c->b_cellIfx, &c->b_IB, &c->b_colj, &c->b_colw, &c->b_kq,
                       &c->b_qtoff, &c->b_qgs, &c->b_qc32, &c->b_fq, &c->b_geo, &c->b_kfix,
                       &c->b_counters, &c->b_toff, &c->b_gstart, &c->b_coefs, &c->b_ticket,
-                      &c->b_win, &c->b_ccf.tab, &c->b_ccf.tmp, &c->b_ccf.m};
+                      &c->b_win, &c->b_ccf.tab, &c->b_ccf.tmp, &c->b_ccf.m, &c->b_ccf.ramp.tab};
     for (DevBuf* b : bufs) release(*b);
-    c->b_ccf.lines_ok = c->b_ccf.m_ok = false;
+    c->b_ccf.lines_ok = c->b_ccf.m_ok = c->b_ccf.ramp.ok = false;
     c->b_ccf.mask_key.clear();
 }
 
@@ -618,9 +618,10 @@ soap_status batch_run(soap_ctx* c, const soap_batch_item* items, int n_items, co
     for (const DevBuf* q : bufs) putp(q->p);
     putp(rv);
     if (rv) {
-        putp(c->b_win.p); putp(c->b_ccf.tab.p); putp(c->b_ccf.tmp.p); putp(c->b_ccf.m.p);
+        putp(c->b_win.p); putp(c->b_ccf.tab.p); putp(c->b_ccf.tmp.p); putp(c->b_ccf.m.p); putp(c->b_ccf.ramp.tab.p);
         put(rvp.n_lines); put(rvp.n_v); put(rvp.n_chunks); put(rvp.n_wgroups); put(rvp.windowed);
         put(rvp.win_lines); put(rvp.win_nb);
+        put(rvp.ramp_L); put(rvp.ramp_rows); put(rvp.ramp_units); put(rvp.ramp_per_block);
         put(rvp.tile_np); put(rvp.tile_blocks); put(rvp.tile_lines); put((uint64_t)rvp.tc_chunk);
         putd(rvp.v_lo); putd(rvp.v_step); putd(rvp.h);
     }

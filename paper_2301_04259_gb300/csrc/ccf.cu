@@ -7,10 +7,11 @@
 //
 // Line and velocity tables (k_ccf_lines, k_ccf_velocities) split each box start into an integer
 // pixel and an exact fraction (FP64: they carry cm/s shifts) and are kept while the mask and the
-// velocity grid are unchanged.  Partial CCF sums per chunk of lines come from one of three
+// velocity grid are unchanged.  Partial CCF sums per chunk of lines come from one of four
 // kernels: k_ccf_tile (FP32 spectra, mask sorted by wavelength: register tiles of 4 velocities x
-// 16 spectra per thread over staged pixel windows), k_ccf_window (FP64 spectra or boxes too wide
-// for the tiles: staged windows, one velocity per thread) and k_ccf_partial (any line order).
+// 16 spectra per thread over staged pixel windows), k_ccf_ramp (ccf_ramp.cu: FP64 spectra, sorted
+// mask, boxes no wider than a pixel), k_ccf_window (boxes too wide for those: staged windows, one
+// velocity per thread) and k_ccf_partial (any line order).
 // k_ccf_reduce adds the partials in a fixed order (FP64, or float pairs with TwoSum); k_gauss_fit
 // fits A + B exp(-(v - mu)^2 / (2 s^2)) per spectrum (one block each: FP32 Levenberg-Marquardt,
 // then Newton steps with FP64 residuals; see its comment).
@@ -1260,6 +1261,9 @@ soap_status ccf_prepare(soap_ctx* c, CcfState& st, const double* mask_lambda, co
             p.n_chunks = p.tile_blocks;
         }
     }
+    if (!same_tab) st.ramp.ok = false;
+    // FP64 spectra, boxes no wider than a pixel, sorted mask
+    const bool ramp = sorted && !f32 && ccf_ramp_plan(c, st, mask_lambda, p, sms);
     // tensor-core form (FP32 spectra, sorted mask): pixel chunks of one wave of CTAs
     if (tc && f32 && sorted && ccf_tc_fits(n_v)) {
         p.tc_chunk = ccf_tc_chunk(c->n_px, n_spec, sms);
@@ -1333,6 +1337,7 @@ soap_status ccf_prepare(soap_ctx* c, CcfState& st, const double* mask_lambda, co
         if (tb) timer_end(c, SOAP_TIMER_CCF_AUX, tb);
     }
     if (p.tc_chunk && !st.m_ok) SOAP_TRY(ccf_tc_build_m(c, st, p));
+    if (ramp) SOAP_TRY(ccf_ramp_build(c, st, p));
     return SOAP_OK;
 }
 
@@ -1345,6 +1350,8 @@ soap_status ccf_enqueue(soap_ctx* c, CcfState& st, const CcfPlan& p, const void*
     const int threads = n_v >= 256 ? 256 : ((n_v + 31) / 32) * 32;
     if (p.tc_chunk) {
         SOAP_TRY(ccf_tc(c, st, p, (const float*)spectra_dev, reinterpret_cast<float*>(d_part)));
+    } else if (p.ramp_L) {
+        SOAP_TRY(ccf_ramp(c, st, p, (const double*)spectra_dev, d_part));
     } else if (p.tile_np) {
         const int tthreads = (((n_v + kTileVT - 1) / kTileVT + 15) / 16 * 16 * kTileLP + 31) / 32 * 32;
         const float box = (float)(2.0 * p.h);

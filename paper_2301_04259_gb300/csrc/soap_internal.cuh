@@ -112,11 +112,25 @@ struct TapGroup {
     int mask;          // bit e: offset 4q + e is one of the taps
 };
 
+// Tables of the FP64 CCF form for narrow boxes (ccf_ramp.cu): events of the velocity grid, lines ordered
+// within their units, and the plan for the last number of spectra.
+struct RampState {
+    DevBuf tab;
+    bool ok = false;                     // built for the current mask and velocity grid
+    int l0 = 0, l1 = 0;                  // lines that can be valid
+    int groups = 0, o_min = 0, n_events = 0, n_slots = 0;
+    size_t o_start = 0, o_fin = 0, o_lines = 0;
+    int plan_tiles = -1;                 // blocks of spectra planned for
+    int L = 0, rows = 0, per_block = 1;
+    int built_L = 0;                     // unit size of the line tables
+};
+
 // CCF state of one user of the CCF (the single-star calls, or the batched form): line and
 // velocity tables (kept while the mask and the velocity grid stay the same), the cached mask
 // matrix of the tensor-core form, and per-call scratch (partial sums, CCF, scaled CCF).
 struct CcfState {
     DevBuf tab, tmp, m;
+    RampState ramp;
     std::vector<double> mask_key;        // mask_lambda, mask_weight, then width
     double vel_key[3] = {0, 0, -1};      // v_lo, v_step, n_v
     bool lines_ok = false;
@@ -134,6 +148,7 @@ struct CcfPlan {
     int tile_np = 0, tile_blocks = 0, tile_lines = 0;
     int64_t tc_chunk = 0;
     int tc_smin = 0, tc_smax = 0;
+    int ramp_L = 0, ramp_rows = 0, ramp_units = 0, ramp_per_block = 0;
     // device tables (in CcfState::tab) and scratch (in CcfState::tmp)
     int* U = nullptr; double* f64 = nullptr; float* f32t = nullptr; float* w32 = nullptr;
     int* valid = nullptr; double* w64 = nullptr;
@@ -407,6 +422,10 @@ bool ccf_tc_fits(int n_v);
 int64_t ccf_tc_chunk(int64_t n_px, int n_spec, int sms);
 // Mask matrix of the tensor-core form for the tables of `st` (once per mask and grid).
 soap_status ccf_tc_build_m(soap_ctx* c, CcfState& st, const CcfPlan& p);
+// the FP64 CCF of boxes no wider than a pixel (ccf_ramp.cu)
+bool ccf_ramp_plan(soap_ctx* c, CcfState& st, const double* mask_lambda, CcfPlan& p, int sms);
+soap_status ccf_ramp_build(soap_ctx* c, CcfState& st, const CcfPlan& p);
+soap_status ccf_ramp(soap_ctx* c, const CcfState& st, const CcfPlan& p, const double* spectra, double* partial);
 soap_status ccf_tc(soap_ctx* c, CcfState& st, const CcfPlan& p, const float* spectra, float* partial);
 
 }  // namespace soap
