@@ -136,10 +136,11 @@ __global__ void k_phase_hist(int N, int n_regions, const RegionGeo* __restrict__
 // ---------------------------------------------------------------------------------------
 // contraction
 // ---------------------------------------------------------------------------------------
-// One block: pixel tile blockIdx.x of phase block blockIdx.y, effect blockIdx.z.  Eight blocks
-// per SM (at most 64 registers with 128 threads) keep the occupancy the tap loads need.
+// One block: pixel tile blockIdx.x of phase block blockIdx.y, effect blockIdx.z.  FP32: eight blocks
+// per SM (at most 64 registers with 128 threads) keep the occupancy the tap loads need; FP64: four,
+// the pipe needs few warps and its accumulators more registers.
 template <typename T, int PB, int R, int THREADS>
-__global__ void __launch_bounds__(THREADS, THREADS == 128 ? 8 : 1)
+__global__ void __launch_bounds__(THREADS, sizeof(T) == 8 ? 4 : 8)
 k_contract(int64_t n_px, Rows<T> rows, const long long* __restrict__ toff, const int* __restrict__ gstart,
            int G, int max_taps, const T* __restrict__ coefs, ClassTypes ctype, const T* __restrict__ contrast,
            const T* __restrict__ fq, int n_phases, EffectList effs, T* __restrict__ out,
@@ -156,7 +157,7 @@ k_contract(int64_t n_px, Rows<T> rows, const long long* __restrict__ toff, const
         const int* gs = gstart + (int64_t)pb * (G + 1);
         const T* cb = coefs + (int64_t)pb * max_taps * PB;
         const int eff = effs.e[blockIdx.z];
-        if constexpr (sizeof(T) == 4 && R % 2 == 0) {
+        if constexpr (sizeof(T) == 4) {
             if (eff == SOAP_EFFECT_FLUX)
                 contract_tile_fold32<PB, R, THREADS, SOAP_EFFECT_FLUX>(n_px, rows, tt, gs, G, cb, con, fq, blockIdx.x, np,
                                                                        out_rows);
@@ -167,7 +168,15 @@ k_contract(int64_t n_px, Rows<T> rows, const long long* __restrict__ toff, const
                 contract_tile_fold32<PB, R, THREADS, SOAP_EFFECT_TOT>(n_px, rows, tt, gs, G, cb, con, fq, blockIdx.x, np,
                                                                       out_rows);
         } else {
-            contract_tile_fold<T, PB, R, THREADS>(n_px, rows, tt, gs, G, cb, con, fq, eff, blockIdx.x, np, out_rows);
+            if (eff == SOAP_EFFECT_FLUX)
+                contract_tile_fold64<PB, R, THREADS, SOAP_EFFECT_FLUX>(n_px, rows, tt, gs, G, cb, con, fq, blockIdx.x, np,
+                                                                       out_rows);
+            else if (eff == SOAP_EFFECT_BCONV)
+                contract_tile_fold64<PB, R, THREADS, SOAP_EFFECT_BCONV>(n_px, rows, tt, gs, G, cb, con, fq, blockIdx.x, np,
+                                                                        out_rows);
+            else
+                contract_tile_fold64<PB, R, THREADS, SOAP_EFFECT_TOT>(n_px, rows, tt, gs, G, cb, con, fq, blockIdx.x, np,
+                                                                      out_rows);
         }
         return;
     }
@@ -211,7 +220,13 @@ static soap_status launch_contract(soap_ctx* c, int n_blocks, int G, int max_tap
 #ifndef SOAP_R32
 #define SOAP_R32 4
 #endif
-constexpr int kPB64 = 4, kR64 = 2, kT64 = 128;
+#ifndef SOAP_PB64
+#define SOAP_PB64 2
+#endif
+#ifndef SOAP_R64
+#define SOAP_R64 4
+#endif
+constexpr int kPB64 = SOAP_PB64, kR64 = SOAP_R64, kT64 = 128;
 constexpr int kPB32 = SOAP_PB32, kR32 = SOAP_R32, kT32 = 128;
 
 // tap-table + coefficient scratch for a kernel set kfix with n_phases "phases" in blocks of PB

@@ -201,12 +201,18 @@ __device__ __forceinline__ void contract_tile(int64_t n_px, const Rows<T>& rows,
 // for the convective blueshift effect, so that out[p][m] = F_q[m] + sum_cl sum_taps K X (the
 // quiet group's kernel is -sum_cl K_cl): one coefficient vector and one FMA per phase and pixel
 // per tap instead of two.  Classes with a contrast row per mu bin keep contract_tile.
-template <typename T, int PB, int R, int THREADS, class Con>
-__device__ __forceinline__ void contract_tile_fold(int64_t n_px, const Rows<T>& rows,
-                                                   const long long* __restrict__ toff, const int* __restrict__ gs,
-                                                   int G, const T* __restrict__ cb, const Con& con,
-                                                   const T* __restrict__ fq, int eff, int64_t tile, int np,
-                                                   T* __restrict__ out_rows) {
+// FP64 form, the effect fixed at compile time: X = C S_a - S_q (TOT), S_a - S_q (BCONV),
+// (C - 1) S_q (FLUX), one FP64 instruction each (two as fma(a, S_a, b S_q) with the effect's factors
+// in registers).  The FP64 pipe is the bound, so the block is small: two phases share the taps of
+// either (100 phases x 205,800 pixels, the whole step: 1.48 ms with two phases x four pixels a
+// thread, 1.55 with 3 x 2, 1.62 with 4 x 2, 1.8 with 8 x 2; skipping the zero coefficients of larger
+// blocks by branches cost more than it saved, 1.60 with 4 x 2).
+template <int PB, int R, int THREADS, int EFF, class Con>
+__device__ __forceinline__ void contract_tile_fold64(int64_t n_px, const Rows<double>& rows,
+                                                     const long long* __restrict__ toff, const int* __restrict__ gs,
+                                                     int G, const double* __restrict__ cb, const Con& con,
+                                                     const double* __restrict__ fq, int64_t tile, int np,
+                                                     double* __restrict__ out_rows) {
     const int64_t m0 = tile * THREADS * R + threadIdx.x;
     int64_t mcl[R];
 #pragma unroll
@@ -214,36 +220,41 @@ __device__ __forceinline__ void contract_tile_fold(int64_t n_px, const Rows<T>& 
         const int64_t m = m0 + (int64_t)r * THREADS;
         mcl[r] = m < n_px ? m : n_px - 1;
     }
-    T acc[PB][R];
+    double acc[PB][R];
 #pragma unroll
     for (int p = 0; p < PB; p++)
 #pragma unroll
-        for (int r = 0; r < R; r++) acc[p][r] = T(0);
-    const T* bq = rows.q + m0;
+        for (int r = 0; r < R; r++) acc[p][r] = 0.0;
+    const double* bq = rows.q + m0;
     for (int g = 0; g < G; g++) {
         const int t0 = gs[g], t1 = gs[g + 1];
         if (t0 == t1) continue;
-        const T* ba = (eff == SOAP_EFFECT_FLUX ? rows.q : rows.a[con.type(g) == SOAP_FACULA ? 1 : 0]) + m0;
-        T ca[R], cq[R];
+        const double* ba = rows.a[con.type(g) == SOAP_FACULA ? 1 : 0] + m0;
+        double cc[R];                                      // C (TOT) or C - 1 (FLUX)
 #pragma unroll
         for (int r = 0; r < R; r++) {
-            const T C = eff == SOAP_EFFECT_BCONV ? T(1) : con.at(g, mcl[r]);
-            ca[r] = eff == SOAP_EFFECT_FLUX ? T(0) : C;
-            cq[r] = eff == SOAP_EFFECT_FLUX ? C - T(1) : T(-1);
+            if constexpr (EFF == SOAP_EFFECT_BCONV) cc[r] = 1.0;
+            else if constexpr (EFF == SOAP_EFFECT_FLUX) cc[r] = con.at(g, mcl[r]) - 1.0;
+            else cc[r] = con.at(g, mcl[r]);
         }
 #pragma unroll 4
         for (int t = t0; t < t1; t++) {
             const long long off = __ldg(toff + t);
-            T x[R];
+            double cv[PB];
+            load_coefs<double, PB>(cb + (int64_t)t * PB, cv);
+            double x[R];
 #pragma unroll
-            for (int r = 0; r < R; r++)
-                x[r] = fma(ca[r], __ldg(ba + off + r * THREADS), cq[r] * __ldg(bq + off + r * THREADS));
-            T cv[PB];
-            load_coefs<T, PB>(cb + (int64_t)t * PB, cv);
+            for (int r = 0; r < R; r++) {
+                const double q = __ldg(bq + off + r * THREADS);
+                if constexpr (EFF == SOAP_EFFECT_FLUX) x[r] = cc[r] * q;
+                else if constexpr (EFF == SOAP_EFFECT_BCONV) x[r] = __ldg(ba + off + r * THREADS) - q;
+                else x[r] = fma(cc[r], __ldg(ba + off + r * THREADS), -q);
+            }
 #pragma unroll
-            for (int p = 0; p < PB; p++)
+            for (int p = 0; p < PB; p++) {
 #pragma unroll
                 for (int r = 0; r < R; r++) acc[p][r] = fma(cv[p], x[r], acc[p][r]);
+            }
         }
     }
 #pragma unroll
@@ -257,7 +268,7 @@ __device__ __forceinline__ void contract_tile_fold(int64_t n_px, const Rows<T>& 
     }
 }
 
-// FP32 form of contract_tile_fold with the effect fixed at compile time: X = C S_a - S_q (TOT),
+// FP32 form with the effect fixed at compile time: X = C S_a - S_q (TOT),
 // S_a - S_q (BCONV), (C - 1) S_q (FLUX, no active row read), the same roundings as the generic
 // form, and the accumulators of pixel pairs (r, r+1) in 64-bit registers updated by two-wide
 // FMAs (fma.rn.f32x2: two independent IEEE FMAs), so the results are the same.
