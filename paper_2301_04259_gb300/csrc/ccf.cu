@@ -511,6 +511,38 @@ k_ccf_reduce(int n_chunks, int n_spec, int n_v, const TP* __restrict__ partial, 
     }
 }
 
+// The same sums for few chunks and many outputs (the batched form): one thread per output runs the
+// kReduceSplit sums and their tree in registers, so that a thread has up to 2 kReduceSplit loads in
+// flight instead of one or two and no barrier.  56,060 spectra x 241 velocities x 9 chunks: 555 us
+// with a block of eight warps per 32 outputs, 139 us so.
+constexpr int kReduceFew = 2 * kReduceSplit;
+__global__ void __launch_bounds__(256)
+k_ccf_reduce_few(int n_chunks, int64_t total, const float* __restrict__ partial, double* __restrict__ ccf) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int64_t t = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    if (t >= total) return;
+    float x[kReduceFew];
+#pragma unroll
+    for (int c = 0; c < kReduceFew; c++)
+        if (c < n_chunks) x[c] = partial[(int64_t)c * total + t];
+    float hi[kReduceSplit], lo[kReduceSplit];
+#pragma unroll
+    for (int y = 0; y < kReduceSplit; y++) {
+        hi[y] = lo[y] = 0.0f;
+        if (y < n_chunks) pair_add(hi[y], lo[y], x[y]);
+        if (y + kReduceSplit < n_chunks) pair_add(hi[y], lo[y], x[y + kReduceSplit]);
+    }
+#pragma unroll
+    for (int o = kReduceSplit / 2; o > 0; o >>= 1)
+#pragma unroll
+        for (int y = 0; y < o; y++) {
+            pair_add(hi[y], lo[y], hi[y + o]);
+            lo[y] += lo[y + o];
+        }
+    ccf[t] = (double)hi[0] + (double)lo[0];
+}
+
 __device__ __forceinline__ double warp_sum(double v) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
@@ -1419,9 +1451,17 @@ soap_status ccf_enqueue(soap_ctx* c, CcfState& st, const CcfPlan& p, const void*
     const bool early = p.tc_chunk != 0;
     if ((p.windowed || p.tile_np || p.tc_chunk) && p.f32) {  // FP32 partial sums (converted exactly to FP64 here)
         cudaLaunchAttribute attr[1];
-        const cudaLaunchConfig_t cfg = pdl_config(dim3(rblocks), dim3(32, kReduceSplit), c->stream, early, attr);
-        SOAP_CUDA(cudaLaunchKernelEx(&cfg, k_ccf_reduce<float>, p.n_chunks, n_spec, n_v,
-                                     reinterpret_cast<const float*>(d_part), d_ccf));
+        const int64_t outputs = (int64_t)n_spec * n_v;
+        // a thread per output while the chunks fit its registers and the outputs fill the GPU
+        if (p.n_chunks <= kReduceFew && outputs >= 152 * 2048) {
+            const cudaLaunchConfig_t cfg = pdl_config(dim3((unsigned)((outputs + 255) / 256)), dim3(256), c->stream, early, attr);
+            SOAP_CUDA(cudaLaunchKernelEx(&cfg, k_ccf_reduce_few, p.n_chunks, outputs,
+                                         reinterpret_cast<const float*>(d_part), d_ccf));
+        } else {
+            const cudaLaunchConfig_t cfg = pdl_config(dim3(rblocks), dim3(32, kReduceSplit), c->stream, early, attr);
+            SOAP_CUDA(cudaLaunchKernelEx(&cfg, k_ccf_reduce<float>, p.n_chunks, n_spec, n_v,
+                                         reinterpret_cast<const float*>(d_part), d_ccf));
+        }
     } else
         k_ccf_reduce<double><<<rblocks, dim3(32, kReduceSplit), 0, c->stream>>>(p.n_chunks, n_spec, n_v,
                                                                                 d_part, d_ccf);
