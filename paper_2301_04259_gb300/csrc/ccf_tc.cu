@@ -163,26 +163,23 @@ struct CcArgs {
     int64_t n_px;
     int64_t chunk;            // pixels per chunk (a multiple of kCcK)
     int n_v, n_pad, n_spec;
-    int vec4;                 // rows are 16-byte aligned: 16-byte loads
+    int vec2;                 // rows are 8-byte aligned: pixel pairs in one load
     int ra;                   // spectrum rows an A stage holds (a multiple of 8, at most 128)
     uint32_t tmem_cols;
 };
 
 
-// 32 spectrum values of row frow at pixels pa .. pa+31, zero at and past P1 (or for no row)
-__device__ __forceinline__ void cc_load_row(float (&a)[32], const float* frow, bool row_on, int vec4,
-                                            int64_t pa, int64_t P1) {
-    if (row_on && vec4 && pa + 32 <= P1) {
-        const float4* src = reinterpret_cast<const float4*>(frow + pa);
-#pragma unroll
-        for (int q = 0; q < 8; q++) {
-            const float4 v = __ldg(src + q);
-            a[4 * q] = v.x; a[4 * q + 1] = v.y; a[4 * q + 2] = v.z; a[4 * q + 3] = v.w;
-        }
-    } else {
-#pragma unroll
-        for (int e = 0; e < 32; e++) a[e] = (row_on && pa + e < P1) ? __ldg(frow + pa + e) : 0.0f;
-    }
+// Loads of the next block's values, issued a block ahead.  Volatile: the compiler would otherwise
+// sink a read-only load past the waits to its use, which undoes the prefetch.
+__device__ __forceinline__ float cc_ld1(const float* p) {
+    float v;
+    asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float2 cc_ld2(const float* p) {
+    float2 v;
+    asm volatile("ld.global.nc.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+    return v;
 }
 
 // Warp-specialised form.  Warp 0, one lane: the mask tiles of K block kb, one bulk copy of both
@@ -198,9 +195,13 @@ __device__ __forceinline__ void cc_load_row(float (&a)[32], const float* frow, b
 //    the MMAs have released it (fullR); the splitters read it back (lanes along the pixels of two
 //    rows per warp access), agree on a named barrier that every value was read, and overwrite the
 //    stage with its BF16 hi/lo tiles.  No spectrum value passes through the load queues.
-//  - registers (any alignment): two threads per spectrum row load the row's values of block kb + 1
-//    while block kb is split, and write block kb once the MMAs have released its stage.
+//  - registers (any alignment): each warp loads its 16 rows kCcAhead blocks ahead of the one that is
+//    split and written, once the MMAs have released its stage.  (With two threads per row, each loading 32
+//    pixels of its own, a warp's load touched 32 rows: 1.85 ms for the CCF of 56,060 spectra of
+//    16,834 pixels; 1.79 so with one block ahead, 1.62 with two or three, 1.63 to 1.77 with the rows
+//    also prefetched to L2 in pieces of 1 to 4 KB.  Without any loads 1.05.)
 constexpr int kCcWsThreads = 352;
+constexpr int kCcAhead = 2;                // blocks the register splitters load ahead
 // A (spectra) stages: three when they are filled by TMA; two when the splitters load the values
 // through L1 themselves (the smaller ring leaves more of the SM's memory to L1)
 __host__ __device__ constexpr int cc_sa(bool tma) { return tma ? 3 : 2; }
@@ -371,30 +372,52 @@ k_ccf_tc(const __grid_constant__ CcArgs g, const __grid_constant__ CUtensorMap m
             cc_mbar_arrive(&fullA[sa]);
         }
     } else {
-        // splitters from registers: spectrum row r, pixels 32 h .. 32 h + 31 of each K block
-        const int u = t - 64;
-        const int r = u & (kCcM - 1), half = u >> 7;
-        const bool row_on = s0 + r < g.n_spec;
-        const float* frow = g.spectra + (int64_t)(row_on ? s0 + r : 0) * g.n_px;
+        // splitters from registers: warp w' = warp - 2 takes rows 16 w' .. 16 w' + 15, a lane two
+        // pixels of each row (whole 256-byte pieces of a row per load, whatever its alignment).  Rows
+        // past the last spectrum repeat it (their lanes of the accumulator are never read).
+        const int r0 = 16 * (warp - 2), first = min(s0 + r0, g.n_spec - 1), left = g.n_spec - 1 - first;
+        const float* src = g.spectra + (int64_t)first * g.n_px + P0 + 2 * lane;
         asm volatile("griddepcontrol.wait;" ::: "memory");     // the spectra's writer has finished
-        float a[32], a1[32];
-        cc_load_row(a, frow, row_on, g.vec4, P0 + 32 * half, P1);
-        auto split = [&](int kb, float (&cur)[32], float (&nxt)[32]) -> bool {
-            if (kb + 1 < n_kb) cc_load_row(nxt, frow, row_on, g.vec4, P0 + (int64_t)(kb + 1) * kCcK + 32 * half, P1);
+        float2 v[kCcAhead][16];
+        auto load = [&](int kb, float2 (&d)[16]) {
+            // pixels of this lane past the end are zero
+            const int64_t px = P0 + (int64_t)kb * kCcK + 2 * lane;
+            const int past = px + 2 > P1 ? (int)(px + 2 - P1) : 0;
+            const float* row = src + (int64_t)kb * kCcK;
+#pragma unroll
+            for (int i = 0; i < 16; i++) {
+                if (past == 0) d[i] = g.vec2 ? cc_ld2(row) : make_float2(cc_ld1(row), cc_ld1(row + 1));
+                else d[i] = make_float2(past == 1 ? cc_ld1(row) : 0.0f, 0.0f);
+                if (i < left) row += g.n_px;
+            }
+        };
+        auto split = [&](int kb, float2 (&d)[16]) -> bool {
             const int sa = kb % SA;
             if (!tc::mbar_wait(&emptyA[sa], ((kb / SA) & 1) ^ 1, flags)) return false;
             unsigned char* st = ringA + (size_t)sa * 2 * ab;
-            if (r < g.ra) {
 #pragma unroll
-                for (int q = 0; q < 4; q++) cc_put8(st, st + ab, cc_sw128(r, 4 * half + q), cur + 8 * q);
+            for (int i = 0; i < 16; i++) {
+                const int r = r0 + i;
+                if (r >= g.ra) continue;
+                uint32_t hw, lw;
+                cc_split2(d[i].x, d[i].y, hw, lw);
+                const uint32_t off = cc_sw128(r, lane >> 2) + (uint32_t)(lane & 3) * 4;
+                *reinterpret_cast<uint32_t*>(st + off) = hw;
+                *reinterpret_cast<uint32_t*>(st + ab + off) = lw;
             }
+            if (kb + kCcAhead < n_kb) load(kb + kCcAhead, d);
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");     // visible to the tensor cores
             cc_mbar_arrive(&fullA[sa]);
             return true;
         };
-        for (int kb = 0; kb < n_kb; kb += 2) {
-            if (!split(kb, a, a1)) break;
-            if (kb + 1 < n_kb && !split(kb + 1, a1, a)) break;
+#pragma unroll
+        for (int q = 0; q < kCcAhead; q++)
+            if (q < n_kb) load(q, v[q]);
+        bool ok = true;
+        for (int kb = 0; kb < n_kb && ok; kb += kCcAhead) {
+#pragma unroll
+            for (int q = 0; q < kCcAhead; q++)
+                if (ok && kb + q < n_kb) ok = split(kb + q, v[q]);
         }
     }
 
@@ -482,7 +505,8 @@ soap_status ccf_tc(soap_ctx* c, CcfState& st, const CcfPlan& p, const float* spe
     a.n_v = p.n_v;
     a.n_pad = n_pad;
     a.n_spec = p.n_spec;
-    a.vec4 = (reinterpret_cast<uintptr_t>(spectra) % 16 == 0 && c->n_px % 4 == 0) ? 1 : 0;
+    const bool vec4 = reinterpret_cast<uintptr_t>(spectra) % 16 == 0 && c->n_px % 4 == 0;
+    a.vec2 = (reinterpret_cast<uintptr_t>(spectra) % 8 == 0 && c->n_px % 2 == 0) ? 1 : 0;
     uint32_t cols = 32;
     while ((int)cols < n_pad) cols <<= 1;
     a.tmem_cols = cols;
@@ -503,7 +527,7 @@ soap_status ccf_tc(soap_ctx* c, CcfState& st, const CcfPlan& p, const float* spe
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     CUtensorMap map_f{};
-    if (a.vec4 && c->n_px < INT_MAX && p.n_spec < INT_MAX) {
+    if (vec4 && c->n_px < INT_MAX && p.n_spec < INT_MAX) {
         // spectra [n_spec][n_px] FP32, boxes of ra rows x 64 pixels
         const uint64_t dims[2] = {(uint64_t)c->n_px, (uint64_t)p.n_spec};
         const uint64_t strides[1] = {(uint64_t)c->n_px * 4};
