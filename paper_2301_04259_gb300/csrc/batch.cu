@@ -218,10 +218,16 @@ __global__ void k_batch_hist(int N, int max_r, const int* __restrict__ phase_ite
     }
 }
 
-// Stage 6: persistent.  A unit is one phase block over all pixel tiles; blocks take the next
-// unit in `order` with an atomic ticket until none is left (no block waits on another).  The
+// Stage 6: persistent.  A unit is one phase block over kUnitTiles pixel tiles; blocks take the next
+// unit (phase blocks in `order`, costly ones first) with an atomic ticket until none is left (no
+// block waits on another).  The cost of a phase block varies by more than a factor of ten with its
+// spots and vsini: with all its tiles as one unit the last costly ones kept a few SMs busy while
+// the others were done (16,834 pixels: 3,001 single phases 690 us, 382 with units of four tiles;
+// 6,996 phases of 64 items 1,094, 388; 56,060 phases 2.64 ms, 2.53; with units of one tile 2.83, of
+// eight 2.52).  The
 // contrast of the item's classes is evaluated per pixel (Planck ratio), so items may carry any
 // temperatures.  fq == nullptr: residual output F - F_q.
+constexpr int kUnitTiles = 4;
 template <int PB, int R, int THREADS>
 __global__ void __launch_bounds__(THREADS)
 k_batch_contract(int64_t n_px, Rows<float> rows, const long long* __restrict__ toff, const int* __restrict__ gstart,
@@ -236,7 +242,8 @@ k_batch_contract(int64_t n_px, Rows<float> rows, const long long* __restrict__ t
         const int u = s_u;
         __syncthreads();
         if (u >= n_units) break;
-        const int pbk = order[u];
+        const int n_groups = (n_tiles + kUnitTiles - 1) / kUnitTiles;
+        const int pbk = order[u / n_groups], tile0 = u % n_groups * kUnitTiles;
         const PBlockDev pb = pblocks[pbk];
         const long long* tt = toff + (int64_t)pbk * max_taps;
         const int* gs = gstart + (int64_t)pbk * (G + 1);
@@ -244,7 +251,7 @@ k_batch_contract(int64_t n_px, Rows<float> rows, const long long* __restrict__ t
         const float* fqi = fq ? fq + (int64_t)pb.item * n_px : nullptr;
         float* orow = out + (int64_t)pb.first_phase * n_px;
         const PlanckContrast32 con{aq, fd, items[pb.item].cls_type, items[pb.item].cls_a};
-        for (int tile = 0; tile < n_tiles; tile++)
+        for (int tile = tile0; tile < min(tile0 + kUnitTiles, n_tiles); tile++)
             contract_tile_fold32<PB, R, THREADS, SOAP_EFFECT_TOT>(n_px, rows, tt, gs, G, cb, con, fqi, tile, pb.np,
                                                                   orow);
     }
@@ -535,7 +542,7 @@ soap_status batch_run(soap_ctx* c, const soap_batch_item* items, int n_items, co
     b.max_r = max_r;
     b.n_pblocks = (int)pbl.size();
     b.n_tiles = (int)((c->n_px + kBatchThreads * V.R - 1) / (kBatchThreads * V.R));
-    b.n_units = b.n_pblocks;
+    b.n_units = b.n_pblocks * ((b.n_tiles + kUnitTiles - 1) / kUnitTiles);   // (bounded by the output's size)
     b.variant = variant;
     b.n_class = n_class;
     b.residual = residual ? 1 : 0;
@@ -561,7 +568,7 @@ soap_status batch_run(soap_ctx* c, const soap_batch_item* items, int n_items, co
     SOAP_TRY(ensure(c->b_phase_item, (size_t)n_phases * sizeof(int)));
     SOAP_TRY(ensure(c->b_phase_block, (size_t)n_phases * sizeof(int)));
     SOAP_TRY(ensure(c->b_pblocks, (size_t)b.n_pblocks * sizeof(PBlockDev)));
-    SOAP_TRY(ensure(c->b_order, (size_t)b.n_units * sizeof(int)));
+    SOAP_TRY(ensure(c->b_order, (size_t)b.n_pblocks * sizeof(int)));
     SOAP_TRY(ensure(c->b_cellIfx, (size_t)N * N * sizeof(long long)));
     SOAP_TRY(ensure(c->b_IB, (size_t)N * c->n_mu * sizeof(long long)));
     SOAP_TRY(ensure(c->b_colj, (size_t)n_items * N * sizeof(int)));
@@ -593,7 +600,7 @@ soap_status batch_run(soap_ctx* c, const soap_batch_item* items, int n_items, co
     SOAP_CUDA(cudaMemcpyAsync(c->b_phase_item.p, phase_item.data(), (size_t)n_phases * sizeof(int), cudaMemcpyHostToDevice, c->stream));
     SOAP_CUDA(cudaMemcpyAsync(c->b_phase_block.p, phase_block.data(), (size_t)n_phases * sizeof(int), cudaMemcpyHostToDevice, c->stream));
     SOAP_CUDA(cudaMemcpyAsync(c->b_pblocks.p, pbl.data(), (size_t)b.n_pblocks * sizeof(PBlockDev), cudaMemcpyHostToDevice, c->stream));
-    SOAP_CUDA(cudaMemcpyAsync(c->b_order.p, order.data(), (size_t)b.n_units * sizeof(int), cudaMemcpyHostToDevice, c->stream));
+    SOAP_CUDA(cudaMemcpyAsync(c->b_order.p, order.data(), (size_t)b.n_pblocks * sizeof(int), cudaMemcpyHostToDevice, c->stream));
     if (rv)
         SOAP_CUDA(cudaMemcpyAsync(c->b_win.p, win.data(), (size_t)n_phases * 2 * sizeof(int), cudaMemcpyHostToDevice,
                                   c->stream));

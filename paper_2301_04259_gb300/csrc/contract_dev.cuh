@@ -67,7 +67,8 @@ struct PlanckContrast32 {
     const float* a;          // [n_class]: h c / (lambda_s k T_class)
     __device__ __forceinline__ int type(int cl) const { return types[cl]; }
     __device__ __forceinline__ float at(int cl, int64_t m) const {
-        const float inv = expf(-(float)m * fd);            // lambda_s / lambda_m
+        // (a pixel index fits 32 bits; a 64-bit integer converts on the FP64 pipe)
+        const float inv = expf(-(float)(int)m * fd);       // lambda_s / lambda_m
         return expm1f(aq * inv) / expm1f(a[cl] * inv);
     }
 };
