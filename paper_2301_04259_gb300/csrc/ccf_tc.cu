@@ -195,7 +195,7 @@ __device__ __forceinline__ float2 cc_ld2(const float* p) {
 //    the MMAs have released it (fullR); the splitters read it back (lanes along the pixels of two
 //    rows per warp access), agree on a named barrier that every value was read, and overwrite the
 //    stage with its BF16 hi/lo tiles.  No spectrum value passes through the load queues.
-//  - registers (any alignment): each warp loads its 16 rows kCcAhead blocks ahead of the one that is
+//  - registers (any alignment): each warp loads every eighth row kCcAhead blocks ahead of the one that is
 //    split and written, once the MMAs have released its stage.  (With two threads per row, each loading 32
 //    pixels of its own, a warp's load touched 32 rows: 1.85 ms for the CCF of 56,060 spectra of
 //    16,834 pixels; 1.79 so with one block ahead, 1.62 with two or three, 1.63 to 1.77 with the rows
@@ -372,11 +372,13 @@ k_ccf_tc(const __grid_constant__ CcArgs g, const __grid_constant__ CUtensorMap m
             cc_mbar_arrive(&fullA[sa]);
         }
     } else {
-        // splitters from registers: warp w' = warp - 2 takes rows 16 w' .. 16 w' + 15, a lane two
-        // pixels of each row (whole 256-byte pieces of a row per load, whatever its alignment).  Rows
-        // past the last spectrum repeat it (their lanes of the accumulator are never read).
-        const int r0 = 16 * (warp - 2), first = min(s0 + r0, g.n_spec - 1), left = g.n_spec - 1 - first;
-        const float* src = g.spectra + (int64_t)first * g.n_px + P0 + 2 * lane;
+        // splitters from registers: warp w' = warp - 2 takes the stage's rows w', w' + 8, .., a lane two
+        // pixels of each (whole 256-byte pieces of a row per load, whatever its alignment).  Rows past
+        // the last spectrum repeat it (their lanes of the accumulator are never read).
+        const int r0 = warp - 2, n_rows = (g.ra - r0 + 7) >> 3;
+        const int64_t pitch = 8 * g.n_px;
+        const float* src = g.spectra + (int64_t)min(s0 + r0, g.n_spec - 1) * g.n_px + P0 + 2 * lane;
+        const int left = max(0, (g.n_spec - 1 - s0 - r0) >> 3);        // further rows that exist
         asm volatile("griddepcontrol.wait;" ::: "memory");     // the spectra's writer has finished
         float2 v[kCcAhead][16];
         auto load = [&](int kb, float2 (&d)[16]) {
@@ -386,9 +388,10 @@ k_ccf_tc(const __grid_constant__ CcArgs g, const __grid_constant__ CUtensorMap m
             const float* row = src + (int64_t)kb * kCcK;
 #pragma unroll
             for (int i = 0; i < 16; i++) {
+                if (i >= n_rows) break;
                 if (past == 0) d[i] = g.vec2 ? cc_ld2(row) : make_float2(cc_ld1(row), cc_ld1(row + 1));
                 else d[i] = make_float2(past == 1 ? cc_ld1(row) : 0.0f, 0.0f);
-                if (i < left) row += g.n_px;
+                if (i < left) row += pitch;
             }
         };
         auto split = [&](int kb, float2 (&d)[16]) -> bool {
@@ -397,8 +400,8 @@ k_ccf_tc(const __grid_constant__ CcArgs g, const __grid_constant__ CUtensorMap m
             unsigned char* st = ringA + (size_t)sa * 2 * ab;
 #pragma unroll
             for (int i = 0; i < 16; i++) {
-                const int r = r0 + i;
-                if (r >= g.ra) continue;
+                if (i >= n_rows) break;
+                const int r = r0 + 8 * i;
                 uint32_t hw, lw;
                 cc_split2(d[i].x, d[i].y, hw, lw);
                 const uint32_t off = cc_sw128(r, lane >> 2) + (uint32_t)(lane & 3) * 4;
