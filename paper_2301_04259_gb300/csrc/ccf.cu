@@ -26,7 +26,7 @@
 
 namespace soap {
 
-constexpr int kLinesPerChunk = 128;      // generic kernel
+constexpr int kLinesPerChunk = 128;      // generic kernel (at most)
 constexpr int kWinLines = 32;             // windowed kernel: lines per chunk at most
 constexpr int kWinMax = 768;              // staged pixels per block (window budget)
 constexpr int kWinSB32 = 16, kWinSB64 = 8; // windowed kernel: spectra per block (FP32, FP64)
@@ -68,11 +68,11 @@ __global__ void k_ccf_partial(int n_lines, const int* __restrict__ U, const T* _
                               const int* __restrict__ valid, const double* __restrict__ weight,
                               int n_v, const int* __restrict__ S, const T* __restrict__ g,
                               double box, int64_t n_px, int n_spec, const T* __restrict__ spectra,
-                              double* __restrict__ partial) {
+                              double* __restrict__ partial, int chunk_lines) {
     const int chunk = blockIdx.x;
     const int s0 = blockIdx.y * SB;
-    const int l0 = chunk * kLinesPerChunk;
-    const int l1 = min(n_lines, l0 + kLinesPerChunk);
+    const int l0 = chunk * chunk_lines;
+    const int l1 = min(n_lines, l0 + chunk_lines);
     const int ns = min(SB, n_spec - s0);
     const T boxT = (T)box;
     for (int k = threadIdx.x; k < n_v; k += blockDim.x) {
@@ -1203,6 +1203,9 @@ static cudaError_t fit_f32_launch(int n_spec, cudaStream_t st, bool early, int n
     return cudaLaunchKernelEx(&cfg, k_gauss_fit_f32<1>, n, n_v, v_lo, v_step, ccf, scratch, rv, fit, win);
 }
 
+// pixels a box of half width h covers at most, as a window's NB
+static int ccf_window_nb(double h) { return 2.0 * h <= 1.0 ? 2 : (2.0 * h <= 7.0 ? 8 : 16); }
+
 // Lines per chunk of the windowed kernel.  A chunk of kWinLines lines costs one window, so it is
 // the cheapest per line, but a chunk is a block's whole work: with few lines there must be fewer
 // to a chunk for every SM to get some (four blocks per SM: 30 lines of a 4,096-pixel grid and 25
@@ -1256,7 +1259,7 @@ soap_status ccf_prepare(soap_ctx* c, CcfState& st, const double* mask_lambda, co
     SOAP_CUDA(cudaGetDevice(&dev));
     SOAP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const int win_sb = f32 ? kWinSB32 : kWinSB64;
-    p.win_nb = 2.0 * p.h <= 1.0 ? 2 : (2.0 * p.h <= 7.0 ? 8 : 16);   // pixels a box covers at most
+    p.win_nb = ccf_window_nb(p.h);
     p.win_lines = ccf_window_lines(n_lines, c->n_px,
                                    (std::atanh((v_lo + (n_v - 1) * v_step) / kCKms) - std::atanh(v_lo / kCKms)) / c->delta,
                                    p.win_nb, (n_spec + win_sb - 1) / win_sb, sms);
@@ -1434,13 +1437,13 @@ soap_status ccf_enqueue(soap_ctx* c, CcfState& st, const CcfPlan& p, const void*
         dim3 grid((unsigned)p.n_chunks, (unsigned)((n_spec + SB - 1) / SB));
         k_ccf_partial<float, SB><<<grid, threads, 0, c->stream>>>(
             n_lines, p.U, p.f32t, p.valid, p.w64, n_v, p.S, p.g32, 2.0 * p.h, c->n_px, n_spec,
-            (const float*)spectra_dev, d_part);
+            (const float*)spectra_dev, d_part, kLinesPerChunk);
     } else {
         constexpr int SB = 8;
         dim3 grid((unsigned)p.n_chunks, (unsigned)((n_spec + SB - 1) / SB));
         k_ccf_partial<double, SB><<<grid, threads, 0, c->stream>>>(
             n_lines, p.U, p.f64, p.valid, p.w64, n_v, p.S, p.g64, 2.0 * p.h, c->n_px, n_spec,
-            (const double*)spectra_dev, d_part);
+            (const double*)spectra_dev, d_part, kLinesPerChunk);
     }
     SOAP_LAUNCHED(c);
     if (tb) timer_end(c, SOAP_TIMER_CCF, tb);
@@ -1565,8 +1568,21 @@ extern "C" soap_status soap_rv_ccf_static(double lambda_start_A, double lambda_e
     const double h = mask_width_kms / (2.0 * kCKms * delta);
     if (2.0 * h > 14.0) { set_error("mask box spans more than 14 pixels"); return SOAP_ERANGE; }
     if (n_spec == 0) return SOAP_OK;
-    // scratch layout, as in rv_ccf_run (generic line order kernel)
-    const int n_chunks = (n_lines + kLinesPerChunk - 1) / kLinesPerChunk;
+    // FP32: as many lines to a chunk as soap_rv_ccf takes (at most), so that the FP32 sums of either, a
+    // chunk each, end at the same lines
+    int dev = 0, sms = 0;
+    SOAP_CUDA(cudaGetDevice(&dev));
+    SOAP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    int chunk_lines = kLinesPerChunk;
+    if (spectra_f32)
+        chunk_lines = ccf_window_lines(n_lines, n_px, (std::atanh(v_hi / kCKms) - std::atanh(v_lo / kCKms)) / delta,
+                                       ccf_window_nb(h), (n_spec + kWinSB32 - 1) / kWinSB32, sms);
+    // scratch layout, as in rv_ccf_run (generic line order kernel); chunks of kLinesPerChunk where the
+    // shorter ones' partial sums would not fit
+    if (((int64_t)(n_lines / chunk_lines) + 3) * n_spec * n_v * 8 + (int64_t)n_lines * 24 + n_v * 16 + 4096 >
+        (int64_t)kStaticScratchBytes)
+        chunk_lines = kLinesPerChunk;
+    const int n_chunks = (n_lines + chunk_lines - 1) / chunk_lines;
     auto al = [](size_t x) { return (x + 255) / 256 * 256; };
     size_t o_U = 0;
     size_t o_f64 = al(o_U + (size_t)n_lines * 4);
@@ -1614,13 +1630,13 @@ extern "C" soap_status soap_rv_ccf_static(double lambda_start_A, double lambda_e
         dim3 grid((unsigned)n_chunks, (unsigned)((n_spec + SB - 1) / SB));
         k_ccf_partial<float, SB><<<grid, threads, 0, stream>>>(
             n_lines, d_U, d_f32, d_valid, mask_weight, n_v, d_S, d_g32, 2.0 * h, n_px, n_spec,
-            (const float*)spectra, d_part);
+            (const float*)spectra, d_part, chunk_lines);
     } else {
         constexpr int SB = 8;
         dim3 grid((unsigned)n_chunks, (unsigned)((n_spec + SB - 1) / SB));
         k_ccf_partial<double, SB><<<grid, threads, 0, stream>>>(
             n_lines, d_U, d_f64, d_valid, mask_weight, n_v, d_S, d_g64, 2.0 * h, n_px, n_spec,
-            (const double*)spectra, d_part);
+            (const double*)spectra, d_part, chunk_lines);
     }
     SOAP_CUDA(cudaGetLastError());
     k_ccf_reduce<double><<<(unsigned)(((int64_t)n_spec * n_v + 31) / 32), dim3(32, kReduceSplit), 0, stream>>>(
