@@ -153,9 +153,8 @@ __global__ void k_batch_hist(int N, int max_r, const int* __restrict__ phase_ite
                              const int32_t* __restrict__ cell_bin, const long long* __restrict__ cell_Ifx,
                              const int* __restrict__ colj, const unsigned int* __restrict__ colw,
                              int tap_min, int n_taps, int n_mu, int n_class, long long* kfix, int use_smem,
-                             int PB, double inv_scale, int fx_bits, int64_t row_len, int64_t pad, long long* toff,
-                             int* gstart,
-                             float* c32, int max_taps, int* counters, int taps_smem, unsigned int* flags,
+                             int PB, double inv_scale, int fx_bits, int64_t row_len, int64_t pad, TapGroup* grp,
+                             int* gcount, float* c32, int gstride, int* counters, int taps_smem, unsigned int* flags,
                              const double* __restrict__ cell_x) {
     __shared__ RegionGeo sg[SOAP_MAX_REGIONS];
     extern __shared__ long long hist_sm[];
@@ -213,8 +212,9 @@ __global__ void k_batch_hist(int N, int max_r, const int* __restrict__ phase_ite
         __threadfence();
         // tables of the classes only (mode 2): the contraction folds the quiet rows into their operands
         build_taps_dev(kfix + (int64_t)pbd.first_phase * nb, 0, pbd.np, n_class, n_mu, n_taps, tap_min, PB, 2,
-                       inv_scale, fx_bits, row_len, pad, toff + (int64_t)pbk * max_taps, gstart + (int64_t)pbk * (n_class + 1),
-                       nullptr, c32 + (int64_t)pbk * max_taps * PB, max_taps, taps_smem ? hist_sm : nullptr, flags);
+                       inv_scale, fx_bits, row_len, pad, nullptr, nullptr, nullptr, c32 + (int64_t)pbk * gstride * (8 * PB), 0,
+                       taps_smem ? hist_sm : nullptr, flags, nullptr, grp + (int64_t)pbk * gstride,
+                       gcount + pbk, gstride);
     }
 }
 
@@ -222,19 +222,20 @@ __global__ void k_batch_hist(int N, int max_r, const int* __restrict__ phase_ite
 // unit (phase blocks in `order`, costly ones first) with an atomic ticket until none is left (no
 // block waits on another).  The cost of a phase block varies by more than a factor of ten with its
 // spots and vsini: with all its tiles as one unit the last costly ones kept a few SMs busy while
-// the others were done (16,834 pixels: 3,001 single phases 690 us, 382 with units of four tiles;
-// 6,996 phases of 64 items 1,094, 388; 56,060 phases 2.64 ms, 2.53; with units of one tile 2.83, of
-// eight 2.52).  The
-// contrast of the item's classes is evaluated per pixel (Planck ratio), so items may carry any
-// temperatures.  fq == nullptr: residual output F - F_q.
+// the others were done (16,834 pixels, tap by tap: 3,001 single phases 690 us, 382 with units of
+// four tiles; 6,996 phases of 64 items 1,094, 388; 56,060 phases 2.64 ms, 2.53; now 236 us and 1.90
+// ms, with units of eight tiles 249 and 1.88).  The contrast of the item's classes is evaluated on the
+// spot (Planck ratio), so items may carry any temperatures.  fq == nullptr: residual output F - F_q.
 constexpr int kUnitTiles = 4;
+// (blocks per SM: as many as the accumulators leave registers for)
 template <int PB, int R, int THREADS>
-__global__ void __launch_bounds__(THREADS)
-k_batch_contract(int64_t n_px, Rows<float> rows, const long long* __restrict__ toff, const int* __restrict__ gstart,
-                 int G, int max_taps, const float* __restrict__ c32, const BatchItemDev* __restrict__ items,
-                 float aq, float fd, const float* __restrict__ fq, const PBlockDev* __restrict__ pblocks,
+__global__ void __launch_bounds__(THREADS, (PB * R <= 8 ? 12 : PB * R <= 32 ? 9 : PB * R <= 64 ? 5 : 4) * 64 / THREADS)
+k_batch_contract(int64_t n_px, Rows<float> rows, const TapGroup* __restrict__ grp, const int* __restrict__ gcount,
+                 int gstride, const float* __restrict__ c32, const BatchItemDev* __restrict__ items,
+                 float aq, float fd, int linear, const float* __restrict__ fq, const PBlockDev* __restrict__ pblocks,
                  const int* __restrict__ order, int n_units, int n_tiles, unsigned int* ticket,
                  float* __restrict__ out) {
+    __shared__ Fold32Smem<PB, R, THREADS> sm;
     __shared__ int s_u;
     while (true) {
         if (threadIdx.x == 0) s_u = (int)atomicAdd(ticket, 1u);
@@ -245,35 +246,35 @@ k_batch_contract(int64_t n_px, Rows<float> rows, const long long* __restrict__ t
         const int n_groups = (n_tiles + kUnitTiles - 1) / kUnitTiles;
         const int pbk = order[u / n_groups], tile0 = u % n_groups * kUnitTiles;
         const PBlockDev pb = pblocks[pbk];
-        const long long* tt = toff + (int64_t)pbk * max_taps;
-        const int* gs = gstart + (int64_t)pbk * (G + 1);
-        const float* cb = c32 + (int64_t)pbk * max_taps * PB;
+        const TapGroup* gr = grp + (int64_t)pbk * gstride;
+        const int n_grp = gcount[pbk];
+        const float* cb = c32 + (int64_t)pbk * gstride * (8 * PB);
         const float* fqi = fq ? fq + (int64_t)pb.item * n_px : nullptr;
         float* orow = out + (int64_t)pb.first_phase * n_px;
-        const PlanckContrast32 con{aq, fd, items[pb.item].cls_type, items[pb.item].cls_a};
+        const PlanckContrast32 con{aq, fd, items[pb.item].cls_type, items[pb.item].cls_a, linear};
         for (int tile = tile0; tile < min(tile0 + kUnitTiles, n_tiles); tile++)
-            contract_tile_fold32<PB, R, THREADS, SOAP_EFFECT_TOT>(n_px, rows, tt, gs, G, cb, con, fqi, tile, pb.np,
-                                                                  orow);
+            contract_tile_fold32<PB, R, THREADS, SOAP_EFFECT_TOT>(n_px, rows, gr, n_grp, 1, cb, con, fqi, tile, pb.np,
+                                                                  orow, sm, tile > tile0);
     }
 }
 
 // ---------------------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------------------
-constexpr int kBatchThreads = 128;
+constexpr int kBatchTile = 512;              // pixels of a block's tile: kBatchTile / R threads
 
 // Variants the autotuner chooses from: (phases per block, pixels per thread).
 struct BatchVariant {
     int PB, R;
 };
-static const BatchVariant kVariants[] = {{1, 4}, {2, 4}, {4, 2}, {4, 4}, {8, 2}, {8, 4}, {16, 2}, {16, 4}};
+static const BatchVariant kVariants[] = {{1, 8}, {2, 8}, {4, 4}, {4, 8}, {8, 4}, {8, 8}, {16, 4}, {16, 8}};
 constexpr int kNumVariants = sizeof(kVariants) / sizeof(kVariants[0]);
 constexpr int kDefaultVariant = 3;
 
 // Sizes of one batch, fixed by the host preparation and baked into the captured graph.
 struct BatchShape {
     int n_items, n_phases, max_r, n_pblocks, n_units, n_tiles, variant, n_class, residual;
-    int G, max_taps;
+    int gstride, linear;
     int64_t nbk;               // per-phase kernel size n_class * n_mu * n_taps
     int use_smem, taps_smem;
     size_t hist_smem;
@@ -293,14 +294,14 @@ static soap_status launch_batch_contract(soap_ctx* c, const BatchShape& b, const
     int dev = 0, sms = 152, per_sm = 4;
     SOAP_CUDA(cudaGetDevice(&dev));
     SOAP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    SOAP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_batch_contract<PB, R, kBatchThreads>,
-                                                            kBatchThreads, 0));
+    constexpr int kThreads = kBatchTile / R;
+    SOAP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_batch_contract<PB, R, kThreads>, kThreads, 0));
     const int grid = std::max(1, std::min(b.n_units, sms * std::max(1, per_sm)));
     SOAP_TIMED(c, SOAP_TIMER_CONTRACT,
-               k_batch_contract<PB, R, kBatchThreads><<<grid, kBatchThreads, 0, c->stream>>>(
-                   c->n_px, rows, c->b_toff.as<long long>(), c->b_gstart.as<int>(), b.G, b.max_taps,
+               k_batch_contract<PB, R, kThreads><<<grid, kThreads, 0, c->stream>>>(
+                   c->n_px, rows, c->b_groups.as<TapGroup>(), c->b_gcount.as<int>(), b.gstride,
                    c->b_coefs.as<float>(), c->b_items.as<BatchItemDev>(), (float)planck_aq(c), (float)c->delta,
-                   b.residual ? nullptr : c->b_fq.as<float>(), c->b_pblocks.as<PBlockDev>(), c->b_order.as<int>(),
+                   b.linear, b.residual ? nullptr : c->b_fq.as<float>(), c->b_pblocks.as<PBlockDev>(), c->b_order.as<int>(),
                    b.n_units, b.n_tiles, c->b_ticket.as<unsigned int>(), out);
                SOAP_LAUNCHED(c));
     return SOAP_OK;
@@ -363,7 +364,7 @@ static soap_status enqueue_batch(soap_ctx* c, const BatchShape& b, float* out, d
                    c->b_colw.as<unsigned int>(), c->tap_min, c->n_taps, c->n_mu, b.n_class,
                    c->b_kfix.as<long long>(), b.use_smem, kVariants[b.variant].PB, inv_scale, c->fx_bits, c->row_len,
                    c->pad,
-                   c->b_toff.as<long long>(), c->b_gstart.as<int>(), c->b_coefs.as<float>(), b.max_taps,
+                   c->b_groups.as<TapGroup>(), c->b_gcount.as<int>(), c->b_coefs.as<float>(), b.gstride,
                    c->b_counters.as<int>(), b.taps_smem, c->flags, c->cell_x);
                SOAP_LAUNCHED(c));
     // 6 persistent contraction
@@ -371,14 +372,14 @@ static soap_status enqueue_batch(soap_ctx* c, const BatchShape& b, float* out, d
     const float* a0 = c->active_set[0] ? c->a32[0] : c->a32[1];
     const float* a1 = c->active_set[1] ? c->a32[1] : c->a32[0];
     switch (b.variant) {
-        case 0: SOAP_TRY((launch_batch_contract<1, 4>(c, b, a0, a1, out))); break;
-        case 1: SOAP_TRY((launch_batch_contract<2, 4>(c, b, a0, a1, out))); break;
-        case 2: SOAP_TRY((launch_batch_contract<4, 2>(c, b, a0, a1, out))); break;
-        case 3: SOAP_TRY((launch_batch_contract<4, 4>(c, b, a0, a1, out))); break;
-        case 4: SOAP_TRY((launch_batch_contract<8, 2>(c, b, a0, a1, out))); break;
-        case 5: SOAP_TRY((launch_batch_contract<8, 4>(c, b, a0, a1, out))); break;
-        case 6: SOAP_TRY((launch_batch_contract<16, 2>(c, b, a0, a1, out))); break;
-        default: SOAP_TRY((launch_batch_contract<16, 4>(c, b, a0, a1, out))); break;
+        case 0: SOAP_TRY((launch_batch_contract<1, 8>(c, b, a0, a1, out))); break;
+        case 1: SOAP_TRY((launch_batch_contract<2, 8>(c, b, a0, a1, out))); break;
+        case 2: SOAP_TRY((launch_batch_contract<4, 4>(c, b, a0, a1, out))); break;
+        case 3: SOAP_TRY((launch_batch_contract<4, 8>(c, b, a0, a1, out))); break;
+        case 4: SOAP_TRY((launch_batch_contract<8, 4>(c, b, a0, a1, out))); break;
+        case 5: SOAP_TRY((launch_batch_contract<8, 8>(c, b, a0, a1, out))); break;
+        case 6: SOAP_TRY((launch_batch_contract<16, 4>(c, b, a0, a1, out))); break;
+        default: SOAP_TRY((launch_batch_contract<16, 8>(c, b, a0, a1, out))); break;
     }
     // 7 radial velocities of the output rows (Sect. 4.1), each fitted in its item's window
     if (rv) SOAP_TRY(ccf_enqueue(c, c->b_ccf, *rvp, out, rv, nullptr, nullptr, c->b_win.as<int>()));
@@ -393,8 +394,8 @@ void batch_variant_info(int v, int* pb, int* r) {
 }
 
 int batch_default_variant(int max_phases_per_item) {
-    if (max_phases_per_item <= 1) return 0;      // (1, 4)
-    if (max_phases_per_item == 2) return 1;      // (2, 4)
+    if (max_phases_per_item <= 1) return 0;      // (1, 8)
+    if (max_phases_per_item == 2) return 1;      // (2, 8)
     return kDefaultVariant;
 }
 
@@ -405,7 +406,7 @@ void batch_release(soap_ctx* c) {
     DevBuf* bufs[] = {&c->b_items, &c->b_regions, &c->b_phases, &c->b_phase_item, &c->b_phase_block,
                       &c->b_pblocks, &c->b_order, &c->b_cellIfx, &c->b_IB, &c->b_colj, &c->b_colw, &c->b_kq,
                       &c->b_qtoff, &c->b_qgs, &c->b_qc32, &c->b_fq, &c->b_geo, &c->b_kfix,
-                      &c->b_counters, &c->b_toff, &c->b_gstart, &c->b_coefs, &c->b_ticket,
+                      &c->b_counters, &c->b_groups, &c->b_gcount, &c->b_coefs, &c->b_ticket,
                       &c->b_win, &c->b_ccf.tab, &c->b_ccf.tmp, &c->b_ccf.m, &c->b_ccf.ramp.tab};
     for (DevBuf* b : bufs) release(*b);
     c->b_ccf.lines_ok = c->b_ccf.m_ok = c->b_ccf.ramp.ok = false;
@@ -439,6 +440,7 @@ soap_status batch_run(soap_ctx* c, const soap_batch_item* items, int n_items, co
     // the item's classes, in first-appearance order
     std::vector<RegionDev> rd;
     int n_class = 0;
+    double x_max = planck_aq(c);
     bool uses[3] = {false, false, false};
     // configurations, phase ownership, phase blocks and their estimated cost
     std::vector<BatchItemDev> it(std::max(1, n_items));
@@ -480,6 +482,7 @@ soap_status batch_run(soap_ctx* c, const soap_batch_item* items, int n_items, co
                 d.cls_type[cl] = g.type;
                 ctemp[cl] = g.temp_K;
                 d.cls_a[cl] = (float)planck_aq(c, g.temp_K);
+                x_max = std::max(x_max, planck_aq(c, g.temp_K));
                 uses[g.type] = true;
             }
             rd.push_back(RegionDev{g.lat_deg, g.lon_deg, g.radius_rstar, g.temp_K, g.type, cl});
@@ -541,13 +544,15 @@ soap_status batch_run(soap_ctx* c, const soap_batch_item* items, int n_items, co
     b.n_phases = n_phases;
     b.max_r = max_r;
     b.n_pblocks = (int)pbl.size();
-    b.n_tiles = (int)((c->n_px + kBatchThreads * V.R - 1) / (kBatchThreads * V.R));
+    b.n_tiles = (int)((c->n_px + kBatchTile - 1) / kBatchTile);
     b.n_units = b.n_pblocks * ((b.n_tiles + kUnitTiles - 1) / kUnitTiles);   // (bounded by the output's size)
     b.variant = variant;
     b.n_class = n_class;
     b.residual = residual ? 1 : 0;
-    b.G = n_class;                                     // class groups (quiet rows folded in)
-    b.max_taps = std::max(b.G, 1) * c->n_mu * c->n_taps;
+    b.gstride = fold_groups(std::max(n_class, 1), c->n_mu, c->n_taps);
+    // contrast by a line over every eight pixels (PlanckContrast32): the largest exponent is the coolest
+    // region's (or the quiet star's) at the first wavelength
+    b.linear = 49.0 / 8.0 * c->delta * c->delta * x_max * (x_max + 1.0) <= std::ldexp(1.0, -26);
     b.nbk = (int64_t)n_class * c->n_mu * c->n_taps;
     const size_t hist_bytes = (size_t)b.nbk * sizeof(long long);
     const size_t kslice_bytes = (size_t)V.PB * b.nbk * sizeof(long long);
@@ -581,9 +586,9 @@ soap_status batch_run(soap_ctx* c, const soap_batch_item* items, int n_items, co
     SOAP_TRY(ensure(c->b_geo, (size_t)n_phases * std::max(1, max_r) * sizeof(RegionGeo)));
     SOAP_TRY(ensure(c->b_kfix, (size_t)n_phases * std::max<int64_t>(1, b.nbk) * sizeof(long long)));
     SOAP_TRY(ensure(c->b_counters, (size_t)b.n_pblocks * sizeof(int)));
-    SOAP_TRY(ensure(c->b_toff, (size_t)b.n_pblocks * b.max_taps * sizeof(long long)));
-    SOAP_TRY(ensure(c->b_gstart, (size_t)b.n_pblocks * (b.G + 1) * sizeof(int)));
-    SOAP_TRY(ensure(c->b_coefs, (size_t)b.n_pblocks * b.max_taps * V.PB * sizeof(float)));
+    SOAP_TRY(ensure(c->b_groups, (size_t)b.n_pblocks * b.gstride * sizeof(TapGroup)));
+    SOAP_TRY(ensure(c->b_gcount, (size_t)b.n_pblocks * sizeof(int)));
+    SOAP_TRY(ensure(c->b_coefs, (size_t)b.n_pblocks * b.gstride * 8 * V.PB * sizeof(float)));
     SOAP_TRY(ensure(c->b_ticket, sizeof(unsigned int)));
     // RVs: fit windows, CCF tables and scratch (tables built here, before any capture)
     CcfPlan rvp;
@@ -612,7 +617,7 @@ soap_status batch_run(soap_ctx* c, const soap_batch_item* items, int n_items, co
     auto putd = [&](double v) { uint64_t u; memcpy(&u, &v, 8); key.push_back(u); };
     auto putp = [&](const void* p) { key.push_back((uint64_t)(uintptr_t)p); };
     put(b.n_items); put(b.n_phases); put(b.max_r); put(b.n_pblocks); put(b.n_units); put(b.n_tiles);
-    put(b.variant); put(b.n_class); put(b.residual); put(b.use_smem); put(b.taps_smem); put(b.hist_smem);
+    put(b.variant); put(b.n_class); put(b.linear); put(b.residual); put(b.use_smem); put(b.taps_smem); put(b.hist_smem);
     put(N); put(c->n_mu); put(c->n_taps); put((uint64_t)c->tap_min); put(c->fx_bits);
     put(c->n_px); put(c->row_len); put(c->pad);
     putd(c->delta); putd(c->lam_s); putd(c->t_quiet);
@@ -621,7 +626,7 @@ soap_status batch_run(soap_ctx* c, const soap_batch_item* items, int n_items, co
     const DevBuf* bufs[] = {&c->b_items, &c->b_regions, &c->b_phases, &c->b_phase_item, &c->b_phase_block,
                             &c->b_pblocks, &c->b_order, &c->b_cellIfx, &c->b_IB, &c->b_colj, &c->b_colw, &c->b_kq,
                             &c->b_qtoff, &c->b_qgs, &c->b_qc32, &c->b_fq, &c->b_geo, &c->b_kfix,
-                            &c->b_counters, &c->b_toff, &c->b_gstart, &c->b_coefs, &c->b_ticket};
+                            &c->b_counters, &c->b_groups, &c->b_gcount, &c->b_coefs, &c->b_ticket};
     for (const DevBuf* q : bufs) putp(q->p);
     putp(rv);
     if (rv) {

@@ -74,7 +74,8 @@ __global__ void k_phase_hist(int N, int n_regions, const RegionGeo* __restrict__
                              int use_smem, int PB, double inv_scale, int fx_bits, int64_t row_len, int64_t pad,
                              long long* toff, int* gstart, double* c64, float* c32, int max_taps,
                              int* counters, int taps_smem, unsigned int* flags, int* bstart,
-                             const double* __restrict__ cell_x, int mode) {
+                             const double* __restrict__ cell_x, int mode, TapGroup* grp, int* grp_start,
+                             int grp_stride, int grp_per_bin) {
     __shared__ RegionGeo sg[SOAP_MAX_REGIONS];
     extern __shared__ long long hist_sm[];
     const int p = blockIdx.x;
@@ -129,18 +130,46 @@ __global__ void k_phase_hist(int N, int n_regions, const RegionGeo* __restrict__
     if (s_last) {
         __threadfence();
         build_taps_dev(kout, pbk, (int)gridDim.x, n_class, n_mu, n_taps, tap_min, PB, mode, inv_scale, fx_bits, row_len,
-                       pad, toff, gstart, c64, c32, max_taps, taps_smem ? hist_sm : nullptr, flags, bstart);
+                       pad, toff, gstart, c64, c32, max_taps, taps_smem ? hist_sm : nullptr, flags, bstart, grp, grp_start, grp_stride, grp_per_bin);
     }
 }
 
 // ---------------------------------------------------------------------------------------
 // contraction
 // ---------------------------------------------------------------------------------------
-// One block: pixel tile blockIdx.x of phase block blockIdx.y, effect blockIdx.z.  FP32: eight blocks
-// per SM (at most 64 registers with 128 threads) keep the occupancy the tap loads need; FP64: four,
-// the pipe needs few warps and its accumulators more registers.
+// FP32, taps as aligned groups: pixel tile blockIdx.x of phase block blockIdx.y, effect blockIdx.z.
+template <int PB, int R, int THREADS>
+__global__ void __launch_bounds__(THREADS, 9)
+k_contract_fold32(int64_t n_px, Rows<float> rows, const TapGroup* __restrict__ grp, const int* __restrict__ gcount,
+                  int n_sub, int stride, const float* __restrict__ coefs, ClassTypes ctype,
+                  const float* __restrict__ contrast, const float* __restrict__ fq, int n_phases, EffectList effs,
+                  float* __restrict__ out) {
+    // a kernel launched after this one with an early start (the tensor-core CCF) may begin once
+    // every CTA here has started: it waits for this grid before it reads the output
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    __shared__ Fold32Smem<PB, R, THREADS> sm;
+    const int pb = blockIdx.y, np = min(PB, n_phases - pb * PB);
+    float* out_rows = out + (int64_t)blockIdx.z * n_phases * n_px + (int64_t)pb * PB * n_px;
+    const TableContrast<float> con{contrast, n_px, ctype};
+    const TapGroup* gr = grp + (int64_t)pb * stride;
+    const int n_grp = gcount[pb];
+    const float* cb = coefs + (int64_t)pb * stride * (8 * PB);
+    const int eff = effs.e[blockIdx.z];
+    if (eff == SOAP_EFFECT_FLUX)
+        contract_tile_fold32<PB, R, THREADS, SOAP_EFFECT_FLUX>(n_px, rows, gr, n_grp, n_sub, cb, con, fq, blockIdx.x,
+                                                               np, out_rows, sm, false);
+    else if (eff == SOAP_EFFECT_BCONV)
+        contract_tile_fold32<PB, R, THREADS, SOAP_EFFECT_BCONV>(n_px, rows, gr, n_grp, n_sub, cb, con, fq, blockIdx.x,
+                                                                np, out_rows, sm, false);
+    else
+        contract_tile_fold32<PB, R, THREADS, SOAP_EFFECT_TOT>(n_px, rows, gr, n_grp, n_sub, cb, con, fq, blockIdx.x,
+                                                              np, out_rows, sm, false);
+}
+
+// FP64 (and the quiet star).  One block: pixel tile blockIdx.x of phase block blockIdx.y, effect
+// blockIdx.z; four blocks per SM: the pipe needs few warps and its accumulators many registers.
 template <typename T, int PB, int R, int THREADS>
-__global__ void __launch_bounds__(THREADS, sizeof(T) == 8 ? 4 : 8)
+__global__ void __launch_bounds__(THREADS, 4)
 k_contract(int64_t n_px, Rows<T> rows, const long long* __restrict__ toff, const int* __restrict__ gstart,
            int G, int max_taps, const T* __restrict__ coefs, ClassTypes ctype, const T* __restrict__ contrast,
            const T* __restrict__ fq, int n_phases, EffectList effs, T* __restrict__ out,
@@ -157,27 +186,15 @@ k_contract(int64_t n_px, Rows<T> rows, const long long* __restrict__ toff, const
         const int* gs = gstart + (int64_t)pb * (G + 1);
         const T* cb = coefs + (int64_t)pb * max_taps * PB;
         const int eff = effs.e[blockIdx.z];
-        if constexpr (sizeof(T) == 4) {
-            if (eff == SOAP_EFFECT_FLUX)
-                contract_tile_fold32<PB, R, THREADS, SOAP_EFFECT_FLUX>(n_px, rows, tt, gs, G, cb, con, fq, blockIdx.x, np,
-                                                                       out_rows);
-            else if (eff == SOAP_EFFECT_BCONV)
-                contract_tile_fold32<PB, R, THREADS, SOAP_EFFECT_BCONV>(n_px, rows, tt, gs, G, cb, con, fq, blockIdx.x, np,
-                                                                        out_rows);
-            else
-                contract_tile_fold32<PB, R, THREADS, SOAP_EFFECT_TOT>(n_px, rows, tt, gs, G, cb, con, fq, blockIdx.x, np,
-                                                                      out_rows);
-        } else {
-            if (eff == SOAP_EFFECT_FLUX)
-                contract_tile_fold64<PB, R, THREADS, SOAP_EFFECT_FLUX>(n_px, rows, tt, gs, G, cb, con, fq, blockIdx.x, np,
-                                                                       out_rows);
-            else if (eff == SOAP_EFFECT_BCONV)
-                contract_tile_fold64<PB, R, THREADS, SOAP_EFFECT_BCONV>(n_px, rows, tt, gs, G, cb, con, fq, blockIdx.x, np,
-                                                                        out_rows);
-            else
-                contract_tile_fold64<PB, R, THREADS, SOAP_EFFECT_TOT>(n_px, rows, tt, gs, G, cb, con, fq, blockIdx.x, np,
-                                                                      out_rows);
-        }
+        if (eff == SOAP_EFFECT_FLUX)
+            contract_tile_fold64<PB, R, THREADS, SOAP_EFFECT_FLUX>(n_px, rows, tt, gs, G, cb, con, fq, blockIdx.x, np,
+                                                                   out_rows);
+        else if (eff == SOAP_EFFECT_BCONV)
+            contract_tile_fold64<PB, R, THREADS, SOAP_EFFECT_BCONV>(n_px, rows, tt, gs, G, cb, con, fq, blockIdx.x, np,
+                                                                    out_rows);
+        else
+            contract_tile_fold64<PB, R, THREADS, SOAP_EFFECT_TOT>(n_px, rows, tt, gs, G, cb, con, fq, blockIdx.x, np,
+                                                                  out_rows);
         return;
     }
     contract_tile<T, PB, R, THREADS>(n_px, rows, toff + (int64_t)pb * max_taps, gstart + (int64_t)pb * (G + 1), G,
@@ -218,7 +235,7 @@ static soap_status launch_contract(soap_ctx* c, int n_blocks, int G, int max_tap
 #define SOAP_PB32 4
 #endif
 #ifndef SOAP_R32
-#define SOAP_R32 4
+#define SOAP_R32 8
 #endif
 #ifndef SOAP_PB64
 #define SOAP_PB64 2
@@ -227,7 +244,7 @@ static soap_status launch_contract(soap_ctx* c, int n_blocks, int G, int max_tap
 #define SOAP_R64 4
 #endif
 constexpr int kPB64 = SOAP_PB64, kR64 = SOAP_R64, kT64 = 128;
-constexpr int kPB32 = SOAP_PB32, kR32 = SOAP_R32, kT32 = 128;
+constexpr int kPB32 = SOAP_PB32, kR32 = SOAP_R32, kT32 = 512 / SOAP_R32;
 
 // tap-table + coefficient scratch for a kernel set kfix with n_phases "phases" in blocks of PB
 static soap_status tap_buffers(soap_ctx* c, int n_phases, int n_class, int PB, int mode, long long** toff,
@@ -419,12 +436,26 @@ soap_status toeplitz_active(soap_ctx* c, const RegionDev* regions_host, int n_re
     long long* kfix = c->kphase.as<long long>();
     // tap tables are built by the last block of each phase block (fused into k_phase_hist)
     const int PB = f64 ? kPB64 : kPB32;
-    long long* toff; int* gstart; double* c64; float* c32; int nbk, G, mt; int* bstart = nullptr;
+    long long* toff = nullptr; int* gstart = nullptr; double* c64 = nullptr; float* c32 = nullptr;
+    int nbk = (n_phases + PB - 1) / PB, G = 0, mt = 0, *bstart = nullptr;
     // tables without the quiet group (mode 2: the contraction folds the quiet rows into the classes'
-    // operands) unless the contrast has a row per mu bin (mode 1, per-bin folds)
-    const int tmode = per_bin ? 1 : 2;
-    SOAP_TRY(tap_buffers(c, n_phases, ncl, PB, tmode, &toff, &gstart, &c64, &c32, &nbk, &G, &mt,
-                         per_bin ? &bstart : nullptr));
+    // operands) unless an FP64 contrast has a row per mu bin (mode 1, per-bin folds)
+    const int tmode = f64 && per_bin ? 1 : 2;
+    // FP32: aligned tap groups, at most ceil((n_taps + 7) / 8) of each class and mu bin
+    TapGroup* grp = nullptr;
+    const int n_sub = per_bin ? c->n_mu : 1;
+    const int gstride = f64 ? 0 : fold_groups(ncl, c->n_mu, c->n_taps);
+    if (f64) {
+        SOAP_TRY(tap_buffers(c, n_phases, ncl, PB, tmode, &toff, &gstart, &c64, &c32, &nbk, &G, &mt,
+                             per_bin ? &bstart : nullptr));
+    } else {
+        const size_t g_bytes = ((size_t)nbk * gstride * sizeof(TapGroup) + 255) / 256 * 256;
+        SOAP_TRY(ensure(c->jobs, g_bytes + (size_t)nbk * sizeof(int)));
+        SOAP_TRY(ensure(c->coefs, (size_t)nbk * gstride * 8 * PB * sizeof(float)));
+        grp = c->jobs.as<TapGroup>();
+        gstart = (int*)(c->jobs.as<char>() + g_bytes);
+        c32 = c->coefs.as<float>();
+    }
     SOAP_TRY(ensure(c->job_counters, (size_t)nbk * sizeof(int)));
     SOAP_CUDA(cudaMemsetAsync(c->job_counters.p, 0, (size_t)nbk * sizeof(int), c->stream));
     const size_t hist_bytes = (size_t)nb * sizeof(long long);
@@ -460,7 +491,8 @@ soap_status toeplitz_active(soap_ctx* c, const RegionDev* regions_host, int n_re
                        c->N, n_regions, c->region_geo.as<RegionGeo>(), c->cell_mu, c->cell_mu32, c->cell_j,
                        c->cell_bin, c->cell_k0, c->cell_k1, c->tap_min, c->n_taps, c->n_mu, ncl, kfix,
                        use_smem, PB, std::ldexp(1.0, -c->fx_bits), c->fx_bits, c->row_len, c->pad, toff, gstart, c64,
-                       c32, mt, c->job_counters.as<int>(), taps_smem, c->flags, bstart, c->cell_x, tmode);
+                       c32, mt, c->job_counters.as<int>(), taps_smem, c->flags, bstart, c->cell_x, tmode, grp, gstart, gstride,
+                       per_bin);
                    SOAP_LAUNCHED(c));
         SOAP_CUDA(cudaEventRecord(c->ev_ph, c->stream));
     }
@@ -489,9 +521,15 @@ soap_status toeplitz_active(soap_ctx* c, const RegionDev* regions_host, int n_re
         return launch_contract<double, kPB64, kR64, kT64>(c, nbk, G, mt, toff, gstart, c64, ct, con64,
                                                          c->fq.as<double>(), n_phases, el, n_eff,
                                                          (double*)dst, c->q64, a64s, a64f, bstart, tmode == 2);
-    return launch_contract<float, kPB32, kR32, kT32>(c, nbk, G, mt, toff, gstart, c32, ct, con32,
-                                                    c->fq.as<float>(), n_phases, el, n_eff,
-                                                    (float*)dst, c->q32, a32s, a32f, bstart, tmode == 2);
+    Rows<float> rows;
+    rows.q = c->q32; rows.a[0] = a32s; rows.a[1] = a32f;
+    const dim3 grid((unsigned)((c->n_px + kT32 * kR32 - 1) / (kT32 * kR32)), (unsigned)nbk, (unsigned)n_eff);
+    SOAP_TIMED(c, SOAP_TIMER_CONTRACT,
+               k_contract_fold32<kPB32, kR32, kT32><<<grid, kT32, 0, c->stream>>>(
+                   c->n_px, rows, grp, gstart, n_sub, gstride, c32, ct, con32, c->fq.as<float>(), n_phases, el,
+                   (float*)dst);
+               SOAP_LAUNCHED(c));
+    return SOAP_OK;
 }
 
 }  // namespace soap

@@ -59,17 +59,48 @@ struct TableContrast {
     ClassTypes ct;
     __device__ __forceinline__ int type(int cl) const { return ct.t[cl]; }
     __device__ __forceinline__ T at(int cl, int64_t m) const { return rows[(int64_t)cl * n_px + m]; }
+    // row k at pixels m .. m + R - 1 (m a multiple of 4; past the last pixel its value)
+    template <int R>
+    __device__ __forceinline__ void load(int k, int64_t m, int64_t n, T (&c)[R]) const {
+        const T* row = rows + (int64_t)k * n_px;
+        if ((n_px & 3) == 0 && m + R <= n) {
+#pragma unroll
+            for (int q = 0; q < R / 4; q++) {
+                const float4 v = __ldg(reinterpret_cast<const float4*>(row + m) + q);
+                c[4 * q] = v.x; c[4 * q + 1] = v.y; c[4 * q + 2] = v.z; c[4 * q + 3] = v.w;
+            }
+        } else {
+#pragma unroll
+            for (int r = 0; r < R; r++) c[r] = row[m + r < n ? m + r : n - 1];
+        }
+    }
 };
 
 struct PlanckContrast32 {
     float aq, fd;            // h c / (lambda_s k T_quiet), grid step Delta
     const int* types;        // [n_class]
     const float* a;          // [n_class]: h c / (lambda_s k T_class)
+    int linear;              // load() by a line over every eight pixels
     __device__ __forceinline__ int type(int cl) const { return types[cl]; }
     __device__ __forceinline__ float at(int cl, int64_t m) const {
         // (a pixel index fits 32 bits; a 64-bit integer converts on the FP64 pipe)
         const float inv = expf(-(float)(int)m * fd);       // lambda_s / lambda_m
         return expm1f(aq * inv) / expm1f(a[cl] * inv);
+    }
+    // At pixels m .. m + R - 1.  Linear between the first and the last of eight pixels where its error,
+    // (7 Delta)^2 / 8 |C''| with |C''| <= C x (x + 1) (x the largest Planck exponent; ' by ln lambda),
+    // is below 2^-26 C: two evaluations instead of eight.
+    template <int R>
+    __device__ __forceinline__ void load(int cl, int64_t m, int64_t n, float (&c)[R]) const {
+        if (linear) {
+            const int64_t m8 = m & ~7ll;
+            const float c0 = at(cl, m8), s = (at(cl, m8 + 7) - c0) * (1.0f / 7.0f), r0 = m & 4 ? 4.0f : 0.0f;
+#pragma unroll
+            for (int r = 0; r < R; r++) c[r] = fmaf(s, r0 + (float)r, c0);
+        } else {
+#pragma unroll
+            for (int r = 0; r < R; r++) c[r] = at(cl, m + r);
+        }
     }
 };
 
@@ -269,10 +300,28 @@ __device__ __forceinline__ void contract_tile_fold64(int64_t n_px, const Rows<do
     }
 }
 
-// FP32 form with the effect fixed at compile time: X = C S_a - S_q (TOT),
-// S_a - S_q (BCONV), (C - 1) S_q (FLUX, no active row read), the same roundings as the generic
-// form, and the accumulators of pixel pairs (r, r+1) in 64-bit registers updated by two-wide
-// FMAs (fma.rn.f32x2: two independent IEEE FMAs), so the results are the same.
+// FP32 form with the effect fixed at compile time: X = C S_a - S_q (TOT), S_a - S_q (BCONV),
+// (C - 1) S_q (FLUX, no active row read), from the taps as aligned groups of eight row offsets
+// (build_taps_dev).
+//
+// Tap by tap the loads bound it: two row values a tap and pixel from L1 are 8 + 2 of its cycles a tap
+// and 128 pixels, against 5 cycles of FMAs for four phases.  So a thread owns R = 8 consecutive pixels
+// and reads the 15 row values that a group's taps need as two 32-byte loads a row (the taps of a class
+// and mu bin are about 3.5 consecutive ones, in 1.3 groups of eight); the taps a group lacks are
+// skipped by its (uniform) mask.  The phase block's groups and coefficients are staged in shared
+// memory, which takes their latency out of the loop, and the registers are held to nine blocks of 64
+// threads an SM: the row loads (60% from L1, the others from L2) need the warps more than the next
+// group's values in registers ahead of time.  Taps are added in falling order of offset, that is
+// rising tap, with the roundings of the form tap by tap; the accumulators of pixel pairs are updated
+// by two-wide FMAs (fma.rn.f32x2: two independent IEEE FMAs).  A contrast with a row per mu bin
+// (n_sub = n_mu) is a segment of one bin each.
+//
+// 100 phases x 205,800 pixels, 3 classes: 73 -> 57 us; 37 phases x 61,747 pixels, a contrast row per
+// bin: 66 -> 29 us; batches of 16,834 pixels: 56,060 phases 2.53 -> 1.90 ms, 3,001 single phases
+// 382 -> 236 us (both with the contrast by a line, PlanckContrast32: 250 and 85 us of it).
+// On the way (the batch of 56,060): 16-byte loads 32 bytes apart 2.77 ms, coefficients from global
+// memory 2.41, the next group's values loaded ahead 2.17 at 7 blocks, 8 blocks 2.02, 10 blocks 1.92,
+// eight phases a block 2.02, two 2.54, R = 4 2.90, the values shared by neighbouring groups kept 1.97.
 __device__ __forceinline__ unsigned long long ct_pack(float lo, float hi) {
     unsigned long long v;
     asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(lo), "f"(hi));
@@ -285,71 +334,182 @@ __device__ __forceinline__ void ct_fma2(unsigned long long& d, unsigned long lon
     asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
 }
 
+// most aligned groups of a phase block: a run of n taps touches at most ceil((n + 7) / 8)
+inline int fold_groups(int n_class, int n_mu, int n_taps) { return n_class * n_mu * ((n_taps + 14) / 8); }
+
+// Shared memory of a block: a chunk of a phase block's groups and coefficients, and two rows of each
+// warp's results, skewed so that 16-byte stores of neighbouring threads fall into different banks.
+template <int PB, int R, int THREADS>
+struct Fold32Smem {
+    static constexpr int kChunk = PB <= 4 ? 32 : 128 / PB;
+    static constexpr int kRow = 32 * R + (R == 8 ? 32 : 0);
+    TapGroup g[kChunk];
+    float4 c[kChunk * 8 * PB / 4];
+    float4 row[THREADS / 32][2][kRow / 4];
+};
+
+// The R + 8 row values from p (a multiple of R values): R = 8 in 32-byte loads, so that a warp's
+// addresses are contiguous (16-byte loads 32 bytes apart take twice the L1 cycles).
+template <int R>
+__device__ __forceinline__ void load_window(const float* __restrict__ p, float (&w)[R + 8]) {
+    if constexpr (R == 8) {
+#pragma unroll
+        for (int k = 0; k < 2; k++)
+            asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                : "=f"(w[8 * k]), "=f"(w[8 * k + 1]), "=f"(w[8 * k + 2]), "=f"(w[8 * k + 3]), "=f"(w[8 * k + 4]),
+                  "=f"(w[8 * k + 5]), "=f"(w[8 * k + 6]), "=f"(w[8 * k + 7])
+                : "l"(p + 8 * k));
+    } else {
+#pragma unroll
+        for (int k = 0; k < R / 4 + 2; k++) {
+            const float4 v = __ldg(reinterpret_cast<const float4*>(p) + k);
+            w[4 * k] = v.x; w[4 * k + 1] = v.y; w[4 * k + 2] = v.z; w[4 * k + 3] = v.w;
+        }
+    }
+}
+
 template <int PB, int R, int THREADS, int EFF, class Con>
 __device__ __forceinline__ void contract_tile_fold32(int64_t n_px, const Rows<float>& rows,
-                                                     const long long* __restrict__ toff,
-                                                     const int* __restrict__ gs, int G, const float* __restrict__ cb,
-                                                     const Con& con, const float* __restrict__ fq, int64_t tile,
-                                                     int np, float* __restrict__ out_rows) {
-    static_assert(R % 2 == 0, "pixel pairs");
-    const int64_t m0 = tile * THREADS * R + threadIdx.x;
-    int64_t mcl[R];
-#pragma unroll
-    for (int r = 0; r < R; r++) {
-        const int64_t m = m0 + (int64_t)r * THREADS;
-        mcl[r] = m < n_px ? m : n_px - 1;
-    }
+                                                     const TapGroup* __restrict__ grp, int n_grp, int n_sub,
+                                                     const float* __restrict__ cb, const Con& con,
+                                                     const float* __restrict__ fq, int64_t tile, int np,
+                                                     float* __restrict__ out_rows, Fold32Smem<PB, R, THREADS>& sm,
+                                                     bool staged) {
+    static_assert(R == 4 || R == 8, "consecutive pixels of a thread");
+    constexpr int kChunk = Fold32Smem<PB, R, THREADS>::kChunk;
+    constexpr bool kActive = EFF != SOAP_EFFECT_FLUX, kCon = EFF != SOAP_EFFECT_BCONV;
+    const int64_t m0 = tile * THREADS * R + threadIdx.x * R;
     unsigned long long acc[PB][R / 2];
 #pragma unroll
     for (int p = 0; p < PB; p++)
 #pragma unroll
         for (int k = 0; k < R / 2; k++) acc[p][k] = 0ull;
     const float* bq = rows.q + m0;
-    for (int g = 0; g < G; g++) {
-        const int t0 = gs[g], t1 = gs[g + 1];
-        if (t0 == t1) continue;
-        const float* ba = rows.a[con.type(g) == SOAP_FACULA ? 1 : 0] + m0;
-        float cc[R];                                       // C (TOT) or C - 1 (FLUX)
-#pragma unroll
-        for (int r = 0; r < R; r++) {
-            if constexpr (EFF == SOAP_EFFECT_BCONV) cc[r] = 1.0f;
-            else if constexpr (EFF == SOAP_EFFECT_FLUX) cc[r] = con.at(g, mcl[r]) - 1.0f;
-            else cc[r] = con.at(g, mcl[r]);
-        }
-#pragma unroll 4
-        for (int t = t0; t < t1; t++) {
-            const long long off = __ldg(toff + t);
-            float x[R];
-#pragma unroll
-            for (int r = 0; r < R; r++) {
-                const float q = __ldg(bq + off + r * THREADS);
-                if constexpr (EFF == SOAP_EFFECT_FLUX) x[r] = cc[r] * q;
-                else if constexpr (EFF == SOAP_EFFECT_BCONV) x[r] = __ldg(ba + off + r * THREADS) - q;
-                else x[r] = fmaf(cc[r], __ldg(ba + off + r * THREADS), -q);
+    const float* ba0 = rows.a[0] + m0;
+    const float* ba1 = rows.a[1] + m0;
+    float cc[R];                                           // C (TOT) or C - 1 (FLUX) of segment `seg`
+    int seg = -1;
+    for (int c0 = 0; c0 < n_grp; c0 += kChunk) {
+        const int nc = min(kChunk, n_grp - c0);
+        if (!staged || n_grp > kChunk) {
+            __syncthreads();                               // the chunk before is consumed
+            for (int i = threadIdx.x; i < nc; i += THREADS) {
+                TapGroup d = grp[c0 + i];
+                if (con.type(d.tap0 / n_sub) == SOAP_FACULA) d.mask |= 256;
+                sm.g[i] = d;
             }
-            unsigned long long x2[R / 2];
+            const float4* src = reinterpret_cast<const float4*>(cb + (int64_t)c0 * (8 * PB));
+            for (int i = threadIdx.x; i < nc * (2 * PB); i += THREADS) sm.c[i] = src[i];
+            __syncthreads();
+        }
+#pragma unroll 1
+        for (int i = 0; i < nc; i++) {
+            const TapGroup d = sm.g[i];
+            float Q[R + 8], A[R + 8];
+            load_window<R>(bq + d.off4, Q);
+            if constexpr (kActive) load_window<R>((d.mask & 256 ? ba1 : ba0) + d.off4, A);
+            if constexpr (kCon) {
+                if (d.tap0 != seg) {
+                    seg = d.tap0;
+                    con.template load<R>(seg, m0, n_px, cc);
+                    if constexpr (EFF == SOAP_EFFECT_FLUX) {
 #pragma unroll
-            for (int k = 0; k < R / 2; k++) x2[k] = ct_pack(x[2 * k], x[2 * k + 1]);
-            float cv[PB];
-            load_coefs<float, PB>(cb + (int64_t)t * PB, cv);
+                        for (int r = 0; r < R; r++) cc[r] -= 1.0f;
+                    }
+                }
+            }
+            const float* cg = reinterpret_cast<const float*>(sm.c) + i * (8 * PB);
 #pragma unroll
-            for (int p = 0; p < PB; p++) {
-                const unsigned long long c2 = ct_pack(cv[p], cv[p]);
+            for (int e = 7; e >= 0; e--) {
+                if (!((d.mask >> e) & 1)) continue;
+                float cv[PB];
+                if constexpr (PB % 4 == 0) {
 #pragma unroll
-                for (int k = 0; k < R / 2; k++) ct_fma2(acc[p][k], c2, x2[k]);
+                    for (int q = 0; q < PB / 4; q++) {
+                        const float4 t = reinterpret_cast<const float4*>(cg + (7 - e) * PB)[q];
+                        cv[4 * q] = t.x; cv[4 * q + 1] = t.y; cv[4 * q + 2] = t.z; cv[4 * q + 3] = t.w;
+                    }
+                } else {
+#pragma unroll
+                    for (int p = 0; p < PB; p++) cv[p] = cg[(7 - e) * PB + p];
+                }
+                unsigned long long x2[R / 2];
+#pragma unroll
+                for (int k = 0; k < R / 2; k++) {
+                    float x[2];
+#pragma unroll
+                    for (int h = 0; h < 2; h++) {
+                        const int r = 2 * k + h;
+                        if constexpr (EFF == SOAP_EFFECT_FLUX) x[h] = cc[r] * Q[e + r];
+                        else if constexpr (EFF == SOAP_EFFECT_BCONV) x[h] = A[e + r] - Q[e + r];
+                        else x[h] = fmaf(cc[r], A[e + r], -Q[e + r]);
+                    }
+                    x2[k] = ct_pack(x[0], x[1]);
+                }
+#pragma unroll
+                for (int p = 0; p < PB; p++) {
+                    const unsigned long long c2 = ct_pack(cv[p], cv[p]);
+#pragma unroll
+                    for (int k = 0; k < R / 2; k++) ct_fma2(acc[p][k], c2, x2[k]);
+                }
             }
         }
     }
+    // results: rows of a multiple of eight pixels directly, else a warp's 32 R pixels of one phase at
+    // a time through its own part of shared memory
+    if (R == 8 && (n_px & 7) == 0 && (reinterpret_cast<uintptr_t>(out_rows) & 31) == 0) {
+        if (m0 >= n_px) return;
+        float base[R];
+#pragma unroll
+        for (int r = 0; r < R; r++) base[r] = 0.0f;
+        if (fq) {
+#pragma unroll
+            for (int k = 0; k < R / 4; k++) {
+                const float4 v = *reinterpret_cast<const float4*>(fq + m0 + 4 * k);
+                base[4 * k] = v.x; base[4 * k + 1] = v.y; base[4 * k + 2] = v.z; base[4 * k + 3] = v.w;
+            }
+        }
+#pragma unroll
+        for (int p = 0; p < PB; p++) {
+            if (p >= np) break;
+            float y[R];
+#pragma unroll
+            for (int k = 0; k < R / 2; k++) ct_unpack(acc[p][k], y[2 * k], y[2 * k + 1]);
+            if (fq) {
+#pragma unroll
+                for (int r = 0; r < R; r++) y[r] = base[r] + y[r];
+            }
+            if constexpr (R == 8)
+                asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(out_rows + (int64_t)p * n_px + m0),
+                             "f"(y[0]), "f"(y[1]), "f"(y[2]), "f"(y[3]), "f"(y[4]), "f"(y[5]), "f"(y[6]), "f"(y[7])
+                             : "memory");
+        }
+        return;
+    }
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t w0 = tile * THREADS * R + warp * 32 * R + lane;
+    float base[R];
+#pragma unroll
+    for (int k = 0; k < R; k++) base[k] = fq && w0 + 32 * k < n_px ? fq[w0 + 32 * k] : 0.0f;
+    __syncwarp();
 #pragma unroll
     for (int p = 0; p < PB; p++) {
         if (p >= np) break;
-        float y[R];
+        float* s = reinterpret_cast<float*>(sm.row[warp][p & 1]);
+        float* mine = s + lane * R + (R == 8 ? (lane >> 2) * 4 : 0);
 #pragma unroll
-        for (int k = 0; k < R / 2; k++) ct_unpack(acc[p][k], y[2 * k], y[2 * k + 1]);
+        for (int k = 0; k < R / 4; k++) {
+            float4 v;
+            ct_unpack(acc[p][2 * k], v.x, v.y);
+            ct_unpack(acc[p][2 * k + 1], v.z, v.w);
+            *reinterpret_cast<float4*>(mine + 4 * k) = v;
+        }
+        __syncwarp();
 #pragma unroll
-        for (int r = 0; r < R; r++) {
-            const int64_t m = m0 + (int64_t)r * THREADS;
-            if (m < n_px) out_rows[(int64_t)p * n_px + m] = fq ? fq[mcl[r]] + y[r] : y[r];
+        for (int k = 0; k < R; k++) {
+            const int64_t m = w0 + 32 * k;
+            const float y = s[32 * k + lane + (R == 8 ? 4 * k : 0)];
+            if (m < n_px) out_rows[(int64_t)p * n_px + m] = fq ? base[k] + y : y;
         }
     }
 }

@@ -105,11 +105,12 @@ enum DeviceFlag : unsigned int {
     kFlagTimeout = 16u         // a tensor-core kernel's bounded barrier wait gave up
 };
 
-// The taps of one (group, mu bin) of a tap table at row offsets 4q .. 4q + 3 (build_taps_dev).
+// The taps of one (group, mu bin) of a tap table at row offsets 4q .. 4q + 3, or 8q .. 8q + 7
+// (build_taps_dev).
 struct TapGroup {
-    long long off4;    // 4q: row offset of the group's first value (a multiple of 4)
-    int tap0;          // tap index of offset 4q (offset 4q + e is tap tap0 - e)
-    int mask;          // bit e: offset 4q + e is one of the taps
+    long long off4;    // row offset of the group's first value (a multiple of 4, or of 8)
+    int tap0;          // tap index of that offset (offset off4 + e is tap tap0 - e), or the group's class
+    int mask;          // bit e: offset off4 + e is one of the taps
 };
 
 // Tables of the FP64 CCF form for narrow boxes (ccf_ramp.cu): events of the velocity grid, lines ordered
@@ -283,7 +284,7 @@ struct soap_ctx {
     // batched form: grow-only buffers, the captured graph and the key of what it baked in
     soap::DevBuf b_items, b_regions, b_phases, b_phase_item, b_phase_block, b_pblocks, b_order;
     soap::DevBuf b_cellIfx, b_IB, b_colj, b_colw, b_kq, b_qtoff, b_qgs, b_qc32, b_fq;
-    soap::DevBuf b_geo, b_kfix, b_counters, b_toff, b_gstart, b_coefs, b_ticket;
+    soap::DevBuf b_geo, b_kfix, b_counters, b_groups, b_gcount, b_coefs, b_ticket;
     cudaGraphExec_t b_graph_exec = nullptr;
     std::vector<uint64_t> b_graph_key;
     uint64_t b_graph_kernels = 0;
@@ -522,17 +523,22 @@ __device__ __forceinline__ float fixed_to_float(long long K, int bits) {
 // agrp / agstart (optional): the same taps as aligned groups.  The taps of one (group, bin) are
 // consecutive shifts of one row, at offsets o_hi, o_hi - 1, .., o_lo; aligned group q holds those
 // of them in 4q .. 4q + 3 (TapGroup: off4 = 4q, the tap index of offset 4q, a bit per present
-// offset; groups listed from the highest q down, like the taps), so that a contraction can read the row values of four consecutive pixels for all of
-// a group's taps as two aligned 16-byte vectors.  agstart[g] is the first aligned group of
+// offset; groups listed from the highest q down, like the taps), so that a contraction can read the
+// row values of four consecutive pixels for all of a group's taps as two aligned 16-byte vectors.  agstart[g] is the first aligned group of
 // group g (G + 1 entries, last = total); block pb's groups start at agrp + pb * max_groups with
 // max_groups = max_taps + G n_mu (a (group, bin) with nk taps has at most nk + 1 groups).
+// grp_stride > 0: aligned groups of eight offsets 8q .. 8q + 7 instead of all the above (toff, gstart
+// and c64 are not written and may be null).  Block pb's groups start at agrp + pb * grp_stride, their
+// number is agstart[pb], TapGroup::tap0 is the group's class (grp_per_bin: class n_mu + bin), and the
+// coefficients are c32[(pb * grp_stride + group)][8][PB], offsets falling, 0 where there is no tap.
 __device__ __forceinline__ void build_taps_dev(const long long* __restrict__ kfix, int pb, int n_phases,
                                                int n_class, int n_mu, int n_taps, int tap_min, int PB, int mode,
                                                double inv_scale, int fx_bits, int64_t row_len, int64_t pad,
                                                long long* toff,
                                                int* gstart, double* c64, float* c32, int max_taps,
                                                long long* s_k, unsigned int* flags, int* bstart = nullptr,
-                                               TapGroup* agrp = nullptr, int* agstart = nullptr) {
+                                               TapGroup* agrp = nullptr, int* agstart = nullptr, int grp_stride = 0,
+                                               int grp_per_bin = 0) {
     __shared__ int s_lo[(1 + SOAP_MAX_CLASSES) * SOAP_MAX_MU];
     __shared__ int s_hi[(1 + SOAP_MAX_CLASSES) * SOAP_MAX_MU];
     __shared__ int s_off[(1 + SOAP_MAX_CLASSES) * SOAP_MAX_MU];
@@ -629,13 +635,41 @@ __device__ __forceinline__ void build_taps_dev(const long long* __restrict__ kfi
         }
         return s_total;
     };
+    const int sh = grp_stride > 0 ? 3 : 2;                     // offsets of a group: 8 or 4
     auto n_groups = [&](int t) -> int {
         if (s_hi[t] < s_lo[t]) return 0;
         const int64_t ob = (int64_t)(t % n_mu) * row_len + o_top;
-        return (int)(((ob - s_lo[t]) >> 2) - ((ob - s_hi[t]) >> 2) + 1);
+        return (int)(((ob - s_lo[t]) >> sh) - ((ob - s_hi[t]) >> sh) + 1);
     };
     const int total_groups = agrp ? scan(n_groups, s_goff) : 0;
     __syncthreads();
+    if (grp_stride > 0) {
+        // aligned groups of eight only, with eight coefficients each
+        if (threadIdx.x == 0) agstart[pb] = total_groups;
+        for (int t = warp; t < ngb; t += nw) {
+            const int ng = n_groups(t);
+            if (ng == 0) continue;
+            const int g = t / n_mu, b = t % n_mu;
+            const int64_t o_hi = (int64_t)b * row_len + o_top - s_lo[t], o_lo = (int64_t)b * row_len + o_top - s_hi[t];
+            const int64_t q_hi = o_hi >> 3, i0 = (int64_t)pb * grp_stride + s_goff[t];
+            for (int i = lane; i < ng; i += 32) {
+                TapGroup tg;
+                tg.off4 = 8 * (q_hi - i);
+                tg.tap0 = grp_per_bin ? t : g;                 // segment
+                tg.mask = 0;
+                for (int e = 0; e < 8; e++)
+                    if (tg.off4 + e >= o_lo && tg.off4 + e <= o_hi) tg.mask |= 1 << e;
+                agrp[i0 + i] = tg;
+            }
+            for (int x = lane; x < ng * 8 * PB; x += 32) {
+                const int pl = x % PB, e = 7 - x / PB % 8, i = x / (8 * PB);
+                const int64_t o = 8 * (q_hi - i) + e;
+                const long long K = o >= o_lo && o <= o_hi ? value(g, b, pl, s_lo[t] + (int)(o_hi - o)) : 0;
+                c32[i0 * (8 * PB) + x] = fixed_to_float(K, fx_bits);
+            }
+        }
+        return;
+    }
     const int total = scan([&](int t) { return s_hi[t] >= s_lo[t] ? s_hi[t] - s_lo[t] + 1 : 0; }, s_off);
     int* gs = gstart + (int64_t)pb * (G + 1);
     if (total > max_taps) {
