@@ -25,6 +25,8 @@
 
 namespace soap {
 
+constexpr int kQuietThreads = 64, kHistThreads = 256;
+
 struct BatchItemDev {
     double vsini, incl_deg;
     int first_region, n_regions, first_phase, n_phases;
@@ -70,18 +72,19 @@ __global__ void k_batch_star(int N, int n_mu, const double* __restrict__ cell_I,
     for (int t = threadIdx.x; t < n_mu; t += blockDim.x) IB[(int64_t)i * n_mu + t] = sb[t];
 }
 
-// Stage 2: block per configuration.
+// Stage 2: block per configuration (residual output needs its column table only).
 __global__ void k_batch_items(int N, int n_mu, int n_taps, int tap_min, double inv_c, double inv_delta,
                               double delta, double inv_expm1_delta, const BatchItemDev* __restrict__ items,
                               const long long* __restrict__ IB, int* __restrict__ colj,
-                              unsigned int* __restrict__ colw, long long* __restrict__ kq,
-                              long long* qtoff, int* qgs, float* qc32, int q_max_taps, double inv_scale,
-                              int fx_bits, int64_t row_len, int64_t pad, unsigned int* flags) {
+                              unsigned int* __restrict__ colw,
+                              TapGroup* qgrp, int* qcount, float* qc32, int q_stride, double inv_scale,
+                              int fx_bits, int64_t row_len, int64_t pad, unsigned int* flags, int residual) {
     extern __shared__ long long hist[];                  // [n_mu][n_taps]
     const int it = blockIdx.x;
     const int nb = n_mu * n_taps;
     const double vsini = items[it].vsini;
-    for (int t = threadIdx.x; t < nb; t += blockDim.x) hist[t] = 0;
+    if (!residual)
+        for (int t = threadIdx.x; t < nb; t += blockDim.x) hist[t] = 0;
     __syncthreads();
     for (int i = threadIdx.x; i < N; i += blockDim.x) {
         const double x = (double)(2 * i + 1 - N) / (double)N;
@@ -99,36 +102,80 @@ __global__ void k_batch_items(int N, int n_mu, int n_taps, int tap_min, double i
         }
         colj[(int64_t)it * N + i] = jt;
         colw[(int64_t)it * N + i] = wfx;
+        if (residual) continue;
         const int kk = jt - tap_min;
         for (int b = 0; b < n_mu; b++) {
             const long long ib = IB[(int64_t)i * n_mu + b];
             if (ib == 0) continue;
             long long k0, k1;
             split_fx(ib, wfx, k0, k1);
-            atomicAdd((unsigned long long*)&hist[b * n_taps + kk], (unsigned long long)k0);
-            atomicAdd((unsigned long long*)&hist[b * n_taps + kk - 1], (unsigned long long)k1);
+            add64_shared(&hist[b * n_taps + kk], k0);
+            add64_shared(&hist[b * n_taps + kk - 1], k1);
         }
     }
     __syncthreads();
-    long long* dst = kq + (int64_t)it * nb;
-    for (int t = threadIdx.x; t < nb; t += blockDim.x) dst[t] = hist[t];
-    __threadfence_block();
-    __syncthreads();
-    build_taps_dev(dst, 0, 1, 1, n_mu, n_taps, tap_min, 1, 0, inv_scale, fx_bits, row_len, pad,
-                   qtoff + (int64_t)it * q_max_taps, qgs + (int64_t)it * 2, nullptr,
-                   qc32 + (int64_t)it * q_max_taps, q_max_taps, hist, flags);
+    if (residual) return;
+    build_taps_dev(hist, 0, 1, 1, n_mu, n_taps, tap_min, 1, 0, inv_scale, fx_bits, row_len, pad, nullptr, nullptr,
+                   nullptr, qc32 + (int64_t)it * q_stride * 8, 0, hist, flags, nullptr, qgrp + (int64_t)it * q_stride,
+                   qcount + it, q_stride, 0, 1);
 }
 
-// Stage 3: grid (tiles, configurations).
-template <int R, int THREADS>
-__global__ void __launch_bounds__(THREADS)
-k_batch_quiet(int64_t n_px, Rows<float> rows, const long long* __restrict__ qtoff, const int* __restrict__ qgs,
-              const float* __restrict__ qc32, int q_max_taps, float* __restrict__ fq) {
-    const int it = blockIdx.y;
-    const TableContrast<float> con{nullptr, n_px, ClassTypes{}};
-    contract_tile<float, 1, R, THREADS>(n_px, rows, qtoff + (int64_t)it * q_max_taps, qgs + (int64_t)it * 2, 1,
-                                        qc32 + (int64_t)it * q_max_taps, con, nullptr, SOAP_EFFECT_TOT,
-                                        blockIdx.x, 1, fq + (int64_t)it * n_px);
+// Stage 3: grid (tiles, configurations).  As contract_tile_fold32 with one phase and X = S_q: a group's
+// eight taps, nearly all of them present, share two 32-byte loads (512 configurations x 16,834 pixels,
+// 250 taps: 183 us, 436 with a load per tap and pixel).
+__global__ void __launch_bounds__(kQuietThreads)
+k_batch_quiet(int64_t n_px, const float* __restrict__ q, const TapGroup* __restrict__ qgrp, const int* __restrict__ qcount,
+              const float* __restrict__ qc32, int q_stride, float* __restrict__ fq) {
+    constexpr int R = 8;
+    __shared__ Fold32Smem<1, R, kQuietThreads> sm;
+    constexpr int kChunk = Fold32Smem<1, R, kQuietThreads>::kChunk;
+    const int it = blockIdx.y, n_grp = qcount[it];
+    const int64_t m0 = (int64_t)blockIdx.x * kQuietThreads * R + threadIdx.x * R;
+    const float* base = q + m0;
+    float acc[R];
+#pragma unroll
+    for (int r = 0; r < R; r++) acc[r] = 0.0f;
+    for (int c0 = 0; c0 < n_grp; c0 += kChunk) {
+        const int nc = min(kChunk, n_grp - c0);
+        __syncthreads();
+        for (int i = threadIdx.x; i < nc; i += kQuietThreads) sm.g[i] = qgrp[(int64_t)it * q_stride + c0 + i];
+        const float4* src = reinterpret_cast<const float4*>(qc32 + ((int64_t)it * q_stride + c0) * 8);
+        for (int i = threadIdx.x; i < 2 * nc; i += kQuietThreads) sm.c[i] = src[i];
+        __syncthreads();
+#pragma unroll 2
+        for (int i = 0; i < nc; i++) {
+            float W[R + 8];
+            load_window<R>(base + sm.g[i].off4, W);
+            const int mask = sm.g[i].mask;
+            const float4 h = sm.c[2 * i], l = sm.c[2 * i + 1];
+            const float cv[8] = {l.w, l.z, l.y, l.x, h.w, h.z, h.y, h.x};      // by offset e
+            if (mask == 255) {
+#pragma unroll
+                for (int e = 7; e >= 0; e--)
+#pragma unroll
+                    for (int r = 0; r < R; r++) acc[r] = fmaf(cv[e], W[e + r], acc[r]);
+            } else {
+#pragma unroll
+                for (int e = 7; e >= 0; e--) {
+                    if (!((mask >> e) & 1)) continue;
+#pragma unroll
+                    for (int r = 0; r < R; r++) acc[r] = fmaf(cv[e], W[e + r], acc[r]);
+                }
+            }
+        }
+    }
+    float* out = fq + (int64_t)it * n_px;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float* s = reinterpret_cast<float*>(sm.row[warp][0]);
+#pragma unroll
+    for (int k = 0; k < R / 4; k++)
+        *reinterpret_cast<float4*>(s + lane * R + (lane >> 2) * 4 + 4 * k) =
+            make_float4(acc[4 * k], acc[4 * k + 1], acc[4 * k + 2], acc[4 * k + 3]);
+    __syncwarp();
+    const int64_t w0 = (int64_t)blockIdx.x * kQuietThreads * R + warp * 32 * R + lane;
+#pragma unroll
+    for (int k = 0; k < R; k++)
+        if (w0 + 32 * k < n_px) out[w0 + 32 * k] = s[36 * k + lane];
 }
 
 // Stage 4: thread per (phase, region slot).
@@ -190,8 +237,13 @@ __global__ void k_batch_hist(int N, int max_r, const int* __restrict__ phase_ite
             long long k0, k1;
             split_fx(cell_Ifx[c], cw[i], k0, k1);
             long long* h = hist + (sg[owner].cls * n_mu + b) * n_taps;
-            atomicAdd((unsigned long long*)&h[kk], (unsigned long long)k0);
-            atomicAdd((unsigned long long*)&h[kk - 1], (unsigned long long)k1);
+            if (use_smem) {
+                add64_shared(&h[kk], k0);
+                add64_shared(&h[kk - 1], k1);
+            } else {
+                atomicAdd((unsigned long long*)&h[kk], (unsigned long long)k0);
+                atomicAdd((unsigned long long*)&h[kk - 1], (unsigned long long)k1);
+            }
         }
     }
     if (use_smem) {
@@ -216,6 +268,67 @@ __global__ void k_batch_hist(int N, int max_r, const int* __restrict__ phase_ite
                        taps_smem ? hist_sm : nullptr, flags, nullptr, grp + (int64_t)pbk * gstride,
                        gcount + pbk, gstride);
     }
+}
+
+// Stage 5 where the kernels of a phase block fit in shared memory: block per phase block, its threads
+// shared evenly by the phases, the job table built from the kernels where they are (56,060 phases in
+// blocks of four: 300 us; a block per phase, which stores its kernels for the last one to read back,
+// 499).  Its instructions bound it, half of them the job table's.
+__global__ void __launch_bounds__(kHistThreads)
+k_batch_hist_block(int N, int max_r, const BatchItemDev* __restrict__ items, const PBlockDev* __restrict__ pblocks,
+                   const RegionGeo* __restrict__ geo, const double* __restrict__ cell_mu,
+                   const float* __restrict__ cell_mu32, const int32_t* __restrict__ cell_bin,
+                   const long long* __restrict__ cell_Ifx, const int* __restrict__ colj,
+                   const unsigned int* __restrict__ colw, int tap_min, int n_taps, int n_mu, int n_class, int PB,
+                   double inv_scale, int fx_bits, int64_t row_len, int64_t pad, TapGroup* grp, int* gcount, float* c32,
+                   int gstride, unsigned int* flags, const double* __restrict__ cell_x) {
+    extern __shared__ long long hist_sm[];                 // [PB][n_class][n_mu][n_taps], then [PB][max_r] regions
+    const int nb = n_class * n_mu * n_taps;
+    RegionGeo* geo_sm = reinterpret_cast<RegionGeo*>(hist_sm + (int64_t)PB * nb);
+    const PBlockDev pbd = pblocks[blockIdx.x];
+    const int nr = items[pbd.item].n_regions;
+    for (int t = threadIdx.x; t < pbd.np * nb; t += kHistThreads) hist_sm[t] = 0;
+    for (int t = threadIdx.x; t < pbd.np * nr; t += kHistThreads)
+        geo_sm[t / nr * max_r + t % nr] = geo[(int64_t)(pbd.first_phase + t / nr) * max_r + t % nr];
+    __syncthreads();
+    const int per = kHistThreads / PB, pl = threadIdx.x / per, lt = threadIdx.x % per;
+    const int* cj = colj + (int64_t)pbd.item * N;
+    const unsigned int* cw = colw + (int64_t)pbd.item * N;
+    const float invN = 1.0f / small_int_to_float(N);
+    if (pl < pbd.np) {
+        const RegionGeo* sg = geo_sm + pl * max_r;
+        long long* hist = hist_sm + (int64_t)pl * nb;
+        for (int r = 0; r < nr; r++) {
+            const int i0 = sg[r].box[0], i1 = sg[r].box[1], j0 = sg[r].box[2], j1 = sg[r].box[3];
+            if (i1 < i0 || j1 < j0) continue;
+            const int wdt = i1 - i0 + 1;
+            const int area = wdt * (j1 - j0 + 1);              // <= N^2 < 2^31
+            BoxWalk wk(lt, per, wdt);
+            for (int t = lt; t < area; t += per, wk.next()) {
+                const int i = i0 + wk.col, jj = j0 + wk.row;
+                if (in_earlier_box(sg, r, i, jj)) continue;
+                const int c = jj * N + i;                      // N^2 < 2^31
+                // all of the cell's values at once: one round trip, not one for each test
+                const int b = cell_bin[c], kk = cj[i] - tap_min;
+                const float muf = cell_mu32[c];
+                const long long I = cell_Ifx[c];
+                const unsigned int w = cw[i];
+                if (b < 0) continue;
+                const int owner = cell_owner(sg, nr, N, invN, i, jj, muf, cell_mu, c, cell_x);
+                if (owner < 0) continue;
+                if (kk < 1 || kk >= n_taps) { atomicOr(flags, kFlagTapRange); continue; }
+                long long k0, k1;
+                split_fx(I, w, k0, k1);
+                long long* h = hist + (sg[owner].cls * n_mu + b) * n_taps;
+                add64_shared(&h[kk], k0);
+                add64_shared(&h[kk - 1], k1);
+            }
+        }
+    }
+    __syncthreads();
+    build_taps_dev(hist_sm, 0, pbd.np, n_class, n_mu, n_taps, tap_min, PB, 2, inv_scale, fx_bits, row_len, pad, nullptr,
+                   nullptr, nullptr, c32 + (int64_t)blockIdx.x * gstride * (8 * PB), 0, hist_sm, flags, nullptr,
+                   grp + (int64_t)blockIdx.x * gstride, gcount + blockIdx.x, gstride, 0, 1);
 }
 
 // Stage 6: persistent.  A unit is one phase block over kUnitTiles pixel tiles; blocks take the next
@@ -277,7 +390,7 @@ struct BatchShape {
     int gstride, linear;
     int64_t nbk;               // per-phase kernel size n_class * n_mu * n_taps
     int use_smem, taps_smem;
-    size_t hist_smem;
+    size_t hist_smem, hist_block_smem;
 };
 
 // h c / (lambda_s k T): the Planck exponent at the first grid wavelength.
@@ -311,7 +424,7 @@ static soap_status launch_batch_contract(soap_ctx* c, const BatchShape& b, const
 // context's stream for a batch whose inputs are already on the device.
 static soap_status enqueue_batch(soap_ctx* c, const BatchShape& b, float* out, double* rv, const CcfPlan* rvp) {
     const int N = c->N;
-    const int q_max_taps = c->n_mu * c->n_taps;
+    const int q_stride = fold_groups(1, c->n_mu, c->n_taps);
     const double scale = std::ldexp(1.0, c->fx_bits);
     const double inv_scale = std::ldexp(1.0, -c->fx_bits);
     // 1 star
@@ -320,26 +433,24 @@ static soap_status enqueue_batch(soap_ctx* c, const BatchShape& b, float* out, d
                    N, c->n_mu, c->cell_I, c->cell_bin, scale, c->b_cellIfx.as<long long>(), c->b_IB.as<long long>());
                SOAP_LAUNCHED(c));
     // 2 configurations: column tables, quiet kernels and job tables
+    const int item_threads = std::min(256, std::max(128, (N + 31) / 32 * 32));   // a column each
     const size_t smem_q = (size_t)c->n_mu * c->n_taps * sizeof(long long);
     SOAP_CUDA(cudaFuncSetAttribute(k_batch_items, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_q));
     SOAP_TIMED(c, SOAP_TIMER_GEOMETRY,
-               k_batch_items<<<b.n_items, 128, smem_q, c->stream>>>(
+               k_batch_items<<<b.n_items, item_threads, smem_q, c->stream>>>(
                    N, c->n_mu, c->n_taps, c->tap_min, 1.0 / kCKms, 1.0 / c->delta, c->delta,
                    1.0 / std::expm1(c->delta), c->b_items.as<BatchItemDev>(), c->b_IB.as<long long>(),
-                   c->b_colj.as<int>(), c->b_colw.as<unsigned int>(), c->b_kq.as<long long>(),
-                   c->b_qtoff.as<long long>(), c->b_qgs.as<int>(), c->b_qc32.as<float>(), q_max_taps, inv_scale,
-                   c->fx_bits, c->row_len, c->pad, c->flags);
+                   c->b_colj.as<int>(), c->b_colw.as<unsigned int>(), c->b_qgroups.as<TapGroup>(),
+                   c->b_qcount.as<int>(), c->b_qc32.as<float>(), q_stride, inv_scale, c->fx_bits, c->row_len, c->pad,
+                   c->flags, b.residual);
                SOAP_LAUNCHED(c));
     // 3 quiet spectra (not needed for residual output)
     if (!b.residual) {
-        Rows<float> rows;
-        rows.q = c->q32; rows.a[0] = nullptr; rows.a[1] = nullptr;
-        const int64_t TILE = 128 * 4;
-        dim3 grid((unsigned)((c->n_px + TILE - 1) / TILE), (unsigned)b.n_items);
+        dim3 grid((unsigned)((c->n_px + kQuietThreads * 8 - 1) / (kQuietThreads * 8)), (unsigned)b.n_items);
         SOAP_TIMED(c, SOAP_TIMER_CONTRACT_QUIET,
-                   k_batch_quiet<4, 128><<<grid, 128, 0, c->stream>>>(
-                       c->n_px, rows, c->b_qtoff.as<long long>(), c->b_qgs.as<int>(), c->b_qc32.as<float>(),
-                       q_max_taps, c->b_fq.as<float>());
+                   k_batch_quiet<<<grid, kQuietThreads, 0, c->stream>>>(
+                       c->n_px, c->q32, c->b_qgroups.as<TapGroup>(), c->b_qcount.as<int>(), c->b_qc32.as<float>(), q_stride,
+                       c->b_fq.as<float>());
                    SOAP_LAUNCHED(c));
     }
     // 4 regions
@@ -352,21 +463,34 @@ static soap_status enqueue_batch(soap_ctx* c, const BatchShape& b, float* out, d
                    SOAP_LAUNCHED(c));
     }
     // 5 per-phase kernels + job tables
-    if (!b.use_smem)
-        SOAP_CUDA(cudaMemsetAsync(c->b_kfix.p, 0, (size_t)b.n_phases * b.nbk * sizeof(long long), c->stream));
-    SOAP_CUDA(cudaMemsetAsync(c->b_counters.p, 0, (size_t)b.n_pblocks * sizeof(int), c->stream));
-    SOAP_CUDA(cudaFuncSetAttribute(k_batch_hist, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b.hist_smem));
-    SOAP_TIMED(c, SOAP_TIMER_PHASE_HIST,
-               k_batch_hist<<<(unsigned)b.n_phases, 128, b.hist_smem, c->stream>>>(
-                   N, std::max(b.max_r, 1), c->b_phase_item.as<int>(), c->b_phase_block.as<int>(),
-                   c->b_items.as<BatchItemDev>(), c->b_pblocks.as<PBlockDev>(), c->b_geo.as<RegionGeo>(),
-                   c->cell_mu, c->cell_mu32, c->cell_bin, c->b_cellIfx.as<long long>(), c->b_colj.as<int>(),
-                   c->b_colw.as<unsigned int>(), c->tap_min, c->n_taps, c->n_mu, b.n_class,
-                   c->b_kfix.as<long long>(), b.use_smem, kVariants[b.variant].PB, inv_scale, c->fx_bits, c->row_len,
-                   c->pad,
-                   c->b_groups.as<TapGroup>(), c->b_gcount.as<int>(), c->b_coefs.as<float>(), b.gstride,
-                   c->b_counters.as<int>(), b.taps_smem, c->flags, c->cell_x);
-               SOAP_LAUNCHED(c));
+    if (b.hist_block_smem) {
+        SOAP_CUDA(cudaFuncSetAttribute(k_batch_hist_block, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)b.hist_block_smem));
+        SOAP_TIMED(c, SOAP_TIMER_PHASE_HIST,
+                   k_batch_hist_block<<<(unsigned)b.n_pblocks, kHistThreads, b.hist_block_smem, c->stream>>>(
+                       N, std::max(b.max_r, 1), c->b_items.as<BatchItemDev>(), c->b_pblocks.as<PBlockDev>(),
+                       c->b_geo.as<RegionGeo>(), c->cell_mu, c->cell_mu32, c->cell_bin, c->b_cellIfx.as<long long>(),
+                       c->b_colj.as<int>(), c->b_colw.as<unsigned int>(), c->tap_min, c->n_taps, c->n_mu, b.n_class,
+                       kVariants[b.variant].PB, inv_scale, c->fx_bits, c->row_len, c->pad, c->b_groups.as<TapGroup>(),
+                       c->b_gcount.as<int>(), c->b_coefs.as<float>(), b.gstride, c->flags, c->cell_x);
+                   SOAP_LAUNCHED(c));
+    } else {
+        if (!b.use_smem)
+            SOAP_CUDA(cudaMemsetAsync(c->b_kfix.p, 0, (size_t)b.n_phases * b.nbk * sizeof(long long), c->stream));
+        SOAP_CUDA(cudaMemsetAsync(c->b_counters.p, 0, (size_t)b.n_pblocks * sizeof(int), c->stream));
+        SOAP_CUDA(cudaFuncSetAttribute(k_batch_hist, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b.hist_smem));
+        SOAP_TIMED(c, SOAP_TIMER_PHASE_HIST,
+                   k_batch_hist<<<(unsigned)b.n_phases, 128, b.hist_smem, c->stream>>>(
+                       N, std::max(b.max_r, 1), c->b_phase_item.as<int>(), c->b_phase_block.as<int>(),
+                       c->b_items.as<BatchItemDev>(), c->b_pblocks.as<PBlockDev>(), c->b_geo.as<RegionGeo>(),
+                       c->cell_mu, c->cell_mu32, c->cell_bin, c->b_cellIfx.as<long long>(), c->b_colj.as<int>(),
+                       c->b_colw.as<unsigned int>(), c->tap_min, c->n_taps, c->n_mu, b.n_class,
+                       c->b_kfix.as<long long>(), b.use_smem, kVariants[b.variant].PB, inv_scale, c->fx_bits, c->row_len,
+                       c->pad,
+                       c->b_groups.as<TapGroup>(), c->b_gcount.as<int>(), c->b_coefs.as<float>(), b.gstride,
+                       c->b_counters.as<int>(), b.taps_smem, c->flags, c->cell_x);
+                   SOAP_LAUNCHED(c));
+    }
     // 6 persistent contraction
     SOAP_CUDA(cudaMemsetAsync(c->b_ticket.p, 0, sizeof(unsigned int), c->stream));
     const float* a0 = c->active_set[0] ? c->a32[0] : c->a32[1];
@@ -404,8 +528,8 @@ void batch_release(soap_ctx* c) {
     c->b_graph_exec = nullptr;
     c->b_graph_key.clear();
     DevBuf* bufs[] = {&c->b_items, &c->b_regions, &c->b_phases, &c->b_phase_item, &c->b_phase_block,
-                      &c->b_pblocks, &c->b_order, &c->b_cellIfx, &c->b_IB, &c->b_colj, &c->b_colw, &c->b_kq,
-                      &c->b_qtoff, &c->b_qgs, &c->b_qc32, &c->b_fq, &c->b_geo, &c->b_kfix,
+                      &c->b_pblocks, &c->b_order, &c->b_cellIfx, &c->b_IB, &c->b_colj, &c->b_colw,
+                      &c->b_qgroups, &c->b_qcount, &c->b_qc32, &c->b_fq, &c->b_geo, &c->b_kfix,
                       &c->b_counters, &c->b_groups, &c->b_gcount, &c->b_coefs, &c->b_ticket,
                       &c->b_win, &c->b_ccf.tab, &c->b_ccf.tmp, &c->b_ccf.m, &c->b_ccf.ramp.tab};
     for (DevBuf* b : bufs) release(*b);
@@ -559,6 +683,10 @@ soap_status batch_run(soap_ctx* c, const soap_batch_item* items, int n_items, co
     b.use_smem = hist_bytes <= 96 * 1024;
     b.taps_smem = kslice_bytes <= 160 * 1024;
     b.hist_smem = std::max(b.use_smem ? hist_bytes : (size_t)0, b.taps_smem ? kslice_bytes : (size_t)0);
+    // a block per phase block where at least two such blocks fit on an SM (else fewer threads would share
+    // the SM than with a block per phase)
+    const size_t hb = kslice_bytes + (size_t)V.PB * std::max(1, max_r) * sizeof(RegionGeo);
+    b.hist_block_smem = hb <= 96 * 1024 ? hb : 0;
     // units: phase blocks, largest estimated cost first
     std::vector<int> border(b.n_pblocks);
     std::iota(border.begin(), border.end(), 0);
@@ -578,14 +706,16 @@ soap_status batch_run(soap_ctx* c, const soap_batch_item* items, int n_items, co
     SOAP_TRY(ensure(c->b_IB, (size_t)N * c->n_mu * sizeof(long long)));
     SOAP_TRY(ensure(c->b_colj, (size_t)n_items * N * sizeof(int)));
     SOAP_TRY(ensure(c->b_colw, (size_t)n_items * N * sizeof(unsigned int)));
-    SOAP_TRY(ensure(c->b_kq, (size_t)n_items * c->n_mu * c->n_taps * sizeof(long long)));
-    SOAP_TRY(ensure(c->b_qtoff, (size_t)n_items * c->n_mu * c->n_taps * sizeof(long long)));
-    SOAP_TRY(ensure(c->b_qgs, (size_t)n_items * 2 * sizeof(int)));
-    SOAP_TRY(ensure(c->b_qc32, (size_t)n_items * c->n_mu * c->n_taps * sizeof(float)));
+    const size_t q_groups = (size_t)n_items * fold_groups(1, c->n_mu, c->n_taps);
+    if (!residual) SOAP_TRY(ensure(c->b_qgroups, q_groups * sizeof(TapGroup)));
+    if (!residual) SOAP_TRY(ensure(c->b_qcount, (size_t)n_items * sizeof(int)));
+    if (!residual) SOAP_TRY(ensure(c->b_qc32, q_groups * 8 * sizeof(float)));
     if (!residual) SOAP_TRY(ensure(c->b_fq, (size_t)n_items * c->n_px * sizeof(float)));
     SOAP_TRY(ensure(c->b_geo, (size_t)n_phases * std::max(1, max_r) * sizeof(RegionGeo)));
-    SOAP_TRY(ensure(c->b_kfix, (size_t)n_phases * std::max<int64_t>(1, b.nbk) * sizeof(long long)));
-    SOAP_TRY(ensure(c->b_counters, (size_t)b.n_pblocks * sizeof(int)));
+    if (!b.hist_block_smem) {
+        SOAP_TRY(ensure(c->b_kfix, (size_t)n_phases * std::max<int64_t>(1, b.nbk) * sizeof(long long)));
+        SOAP_TRY(ensure(c->b_counters, (size_t)b.n_pblocks * sizeof(int)));
+    }
     SOAP_TRY(ensure(c->b_groups, (size_t)b.n_pblocks * b.gstride * sizeof(TapGroup)));
     SOAP_TRY(ensure(c->b_gcount, (size_t)b.n_pblocks * sizeof(int)));
     SOAP_TRY(ensure(c->b_coefs, (size_t)b.n_pblocks * b.gstride * 8 * V.PB * sizeof(float)));
@@ -617,15 +747,15 @@ soap_status batch_run(soap_ctx* c, const soap_batch_item* items, int n_items, co
     auto putd = [&](double v) { uint64_t u; memcpy(&u, &v, 8); key.push_back(u); };
     auto putp = [&](const void* p) { key.push_back((uint64_t)(uintptr_t)p); };
     put(b.n_items); put(b.n_phases); put(b.max_r); put(b.n_pblocks); put(b.n_units); put(b.n_tiles);
-    put(b.variant); put(b.n_class); put(b.linear); put(b.residual); put(b.use_smem); put(b.taps_smem); put(b.hist_smem);
+    put(b.variant); put(b.n_class); put(b.linear); put(b.residual); put(b.use_smem); put(b.taps_smem); put(b.hist_smem); put(b.hist_block_smem);
     put(N); put(c->n_mu); put(c->n_taps); put((uint64_t)c->tap_min); put(c->fx_bits);
     put(c->n_px); put(c->row_len); put(c->pad);
     putd(c->delta); putd(c->lam_s); putd(c->t_quiet);
     putp(out); putp(c->stream); putp(c->q32); putp(c->a32[0]); putp(c->a32[1]); putp(c->cell_I);
     putp(c->cell_bin); putp(c->cell_mu); putp(c->cell_mu32); putp(c->flags); putp(c->cell_x);
     const DevBuf* bufs[] = {&c->b_items, &c->b_regions, &c->b_phases, &c->b_phase_item, &c->b_phase_block,
-                            &c->b_pblocks, &c->b_order, &c->b_cellIfx, &c->b_IB, &c->b_colj, &c->b_colw, &c->b_kq,
-                            &c->b_qtoff, &c->b_qgs, &c->b_qc32, &c->b_fq, &c->b_geo, &c->b_kfix,
+                            &c->b_pblocks, &c->b_order, &c->b_cellIfx, &c->b_IB, &c->b_colj, &c->b_colw,
+                            &c->b_qgroups, &c->b_qcount, &c->b_qc32, &c->b_fq, &c->b_geo, &c->b_kfix,
                             &c->b_counters, &c->b_groups, &c->b_gcount, &c->b_coefs, &c->b_ticket};
     for (const DevBuf* q : bufs) putp(q->p);
     putp(rv);

@@ -104,10 +104,16 @@ __global__ void k_phase_hist(int N, int n_regions, const RegionGeo* __restrict__
             const int owner = cell_owner(sg, n_regions, N, invN, i, jj, cell_mu32[c], cell_mu, c, cell_x);
             if (owner < 0) continue;
             const int kk = cell_j[c] - tap_min;
+            const long long k0 = cell_k0[c], k1 = cell_k1[c];
             if (kk < 1 || kk >= n_taps) { atomicOr(flags, kFlagTapRange); continue; }
             long long* h = hist + (sg[owner].cls * n_mu + b) * n_taps;
-            atomicAdd((unsigned long long*)&h[kk], (unsigned long long)cell_k0[c]);
-            atomicAdd((unsigned long long*)&h[kk - 1], (unsigned long long)cell_k1[c]);
+            if (use_smem) {
+                add64_shared(&h[kk], k0);
+                add64_shared(&h[kk - 1], k1);
+            } else {
+                atomicAdd((unsigned long long*)&h[kk], (unsigned long long)k0);
+                atomicAdd((unsigned long long*)&h[kk - 1], (unsigned long long)k1);
+            }
         }
     }
     if (use_smem) {

@@ -283,7 +283,7 @@ struct soap_ctx {
 
     // batched form: grow-only buffers, the captured graph and the key of what it baked in
     soap::DevBuf b_items, b_regions, b_phases, b_phase_item, b_phase_block, b_pblocks, b_order;
-    soap::DevBuf b_cellIfx, b_IB, b_colj, b_colw, b_kq, b_qtoff, b_qgs, b_qc32, b_fq;
+    soap::DevBuf b_cellIfx, b_IB, b_colj, b_colw, b_qgroups, b_qcount, b_qc32, b_fq;
     soap::DevBuf b_geo, b_kfix, b_counters, b_groups, b_gcount, b_coefs, b_ticket;
     cudaGraphExec_t b_graph_exec = nullptr;
     std::vector<uint64_t> b_graph_key;
@@ -458,6 +458,17 @@ __device__ __forceinline__ float fixed_to_float(long long K, int bits) {
     return __uint_as_float(sign | ((unsigned int)biased << 23) | (m & 0x7FFFFFu));
 }
 
+// p += v in shared memory, exact in any order: a 32-bit atomic per half, the carry taken from the low
+// half's old value.  (Many cells add to few taps; the 64-bit atomic on shared memory, tried again until
+// it meets no other, took the batch's quiet kernels of 3,001 configurations 183 us instead of 82.)
+__device__ __forceinline__ void add64_shared(long long* p, long long v) {
+    unsigned int* w = reinterpret_cast<unsigned int*>(p);
+    const unsigned int lo = (unsigned int)v, hi = (unsigned int)((unsigned long long)v >> 32);
+    const unsigned int old = atomicAdd(w, lo);
+    const unsigned int up = hi + (old + lo < old ? 1u : 0u);
+    if (up) atomicAdd(w + 1, up);
+}
+
 // ---------------------------------------------------------------------------------------
 // tap tables of the Toeplitz contraction (shared by geometry.cu, contract.cu and batch.cu)
 // ---------------------------------------------------------------------------------------
@@ -531,6 +542,7 @@ __device__ __forceinline__ float fixed_to_float(long long K, int bits) {
 // and c64 are not written and may be null).  Block pb's groups start at agrp + pb * grp_stride, their
 // number is agstart[pb], TapGroup::tap0 is the group's class (grp_per_bin: class n_mu + bin), and the
 // coefficients are c32[(pb * grp_stride + group)][8][PB], offsets falling, 0 where there is no tap.
+// s_k (optional): shared memory for the block's kernels; s_ready: they are in it already.
 __device__ __forceinline__ void build_taps_dev(const long long* __restrict__ kfix, int pb, int n_phases,
                                                int n_class, int n_mu, int n_taps, int tap_min, int PB, int mode,
                                                double inv_scale, int fx_bits, int64_t row_len, int64_t pad,
@@ -538,7 +550,7 @@ __device__ __forceinline__ void build_taps_dev(const long long* __restrict__ kfi
                                                int* gstart, double* c64, float* c32, int max_taps,
                                                long long* s_k, unsigned int* flags, int* bstart = nullptr,
                                                TapGroup* agrp = nullptr, int* agstart = nullptr, int grp_stride = 0,
-                                               int grp_per_bin = 0) {
+                                               int grp_per_bin = 0, int s_ready = 0) {
     __shared__ int s_lo[(1 + SOAP_MAX_CLASSES) * SOAP_MAX_MU];
     __shared__ int s_hi[(1 + SOAP_MAX_CLASSES) * SOAP_MAX_MU];
     __shared__ int s_off[(1 + SOAP_MAX_CLASSES) * SOAP_MAX_MU];
@@ -554,7 +566,9 @@ __device__ __forceinline__ void build_taps_dev(const long long* __restrict__ kfi
     // the block's slice of kernels, [np][n_class][n_mu][n_taps], staged with coalesced loads
     const long long* src = kfix + (int64_t)p0 * nb;
     const long long* K = src;
-    if (use_smem) {
+    if (use_smem && s_ready) {
+        K = s_k;
+    } else if (use_smem) {
         const int64_t n_el = (int64_t)np * nb;
         for (int64_t t0 = threadIdx.x; t0 < n_el; t0 += 8 * (int64_t)blockDim.x) {
             long long v[8];
@@ -584,25 +598,53 @@ __device__ __forceinline__ void build_taps_dev(const long long* __restrict__ kfi
         const int cl = mode == 0 ? 0 : (mode == 1 ? g - 1 : g);
         return kval(base + ((int64_t)cl * n_mu + b) * n_taps + kk);
     };
-    // tap range of each (group, bin) over the block's phases
-    for (int t = threadIdx.x; t < ngb; t += blockDim.x) {
-        const int g = t / n_mu, b = t % n_mu;
-        int lo = n_taps, hi = -1;
-        const int c0 = mode == 0 ? 0 : (mode == 2 ? g : (g == 0 ? 0 : g - 1));
-        const int c1 = (mode == 1 && g == 0) ? n_class : c0 + 1;
-        for (int pl = 0; pl < np; pl++) {
-            const long long* base = K + (int64_t)pl * nb;
-            for (int cl = c0; cl < c1; cl++) {
-                const long long* row = base + ((int64_t)cl * n_mu + b) * n_taps;
-                for (int kk = 0; kk < n_taps; kk++)
-                    if (kval(row + kk) != 0) { lo = min(lo, kk); hi = max(hi, kk); }
-            }
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    // tap range of each (group, bin) over the block's phases: a thread each where there is little to look
+    // through (the threads are then done in one pass), else 16 or 32 lanes each, one per tap
+    auto span = [&](int t, int& c0, int& c1) -> const long long* {
+        const int g = t / n_mu, b = t - g * n_mu;
+        c0 = mode == 0 ? 0 : (mode == 2 ? g : (g == 0 ? 0 : g - 1));
+        c1 = (mode == 1 && g == 0) ? n_class : c0 + 1;
+        return K + (int64_t)b * n_taps;
+    };
+    if (np * n_taps <= 64) {
+        for (int t = threadIdx.x; t < ngb; t += blockDim.x) {
+            int lo = n_taps, hi = -1, c0, c1;
+            const long long* base = span(t, c0, c1);
+            for (int pl = 0; pl < np; pl++)
+                for (int cl = c0; cl < c1; cl++)
+                    for (int kk = 0; kk < n_taps; kk++)
+                        if (kval(base + (int64_t)pl * nb + (int64_t)cl * n_mu * n_taps + kk) != 0) {
+                            lo = min(lo, kk);
+                            hi = max(hi, kk);
+                        }
+            s_lo[t] = lo; s_hi[t] = hi;
         }
-        s_lo[t] = lo; s_hi[t] = hi;
+    } else {
+        const int sw = n_taps <= 16 ? 16 : 32, sub = lane / sw, sl = lane % sw;
+        const unsigned int smask = sw == 32 ? 0xffffffffu : 0xffffu;
+        for (int t0 = warp * (32 / sw); t0 < ngb; t0 += nw * (32 / sw)) {
+            const int t = t0 + sub;
+            int lo = n_taps, hi = -1, c0, c1;
+            const long long* base = span(t, c0, c1);
+            for (int k0 = 0; k0 < n_taps; k0 += sw) {
+                const int kk = k0 + sl;
+                bool on = false;
+                if (t < ngb && kk < n_taps)
+                    for (int pl = 0; pl < np; pl++)
+                        for (int cl = c0; cl < c1; cl++)
+                            on |= kval(base + (int64_t)pl * nb + (int64_t)cl * n_mu * n_taps + kk) != 0;
+                const unsigned int any = __ballot_sync(0xffffffffu, on) >> (sub * sw) & smask;
+                if (any) {
+                    lo = min(lo, k0 + __ffs(any) - 1);
+                    hi = k0 + 31 - __clz(any);
+                }
+            }
+            if (sl == 0 && t < ngb) { s_lo[t] = lo; s_hi[t] = hi; }
+        }
     }
     // exclusive prefix sums (warp scans, chunks of blockDim.x) of the tap counts and of the
     // aligned-group counts per (group, bin)
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
     const int64_t o_top = pad - tap_min;                       // offset of tap 0 in bin 0
     auto scan = [&](auto count, int* dst) -> int {
         if (threadIdx.x == 0) s_total = 0;

@@ -64,13 +64,16 @@ def test_star(S, n_px, n_mu, vsini, px_kms, n_phases, limb):
     assert np.abs(got[S.SOAP_FP32] - ref).max() <= TOL32 * np.abs(ref).max()
 
 
-# pixels of 0.9 km/s take the contrast by a line, those of 20 km/s pixel by pixel
-@pytest.mark.parametrize("n_px,px_kms,vsini", [(1025, 0.9, 12.0), (1024, 0.9, 12.0), (515, 20.0, 12.0)])
+# pixels of 0.9 km/s take the contrast by a line, those of 20 km/s pixel by pixel; the kernels of the last
+# case's phase blocks (4 classes, 40 bins, 242 taps) do not fit in shared memory, those of the one before
+# with few phases a block only
+@pytest.mark.parametrize("n_px,px_kms,vsini,n_mu", [(1025, 0.9, 12.0, 12), (1024, 0.9, 12.0, 12), (515, 20.0, 12.0, 12),
+                                                    (600, 0.9, 30.0, 20), (700, 0.5, 60.0, 40)])
 @pytest.mark.parametrize("residual", [False, True])
-def test_batch(S, n_px, px_kms, vsini, residual):
+def test_batch(S, n_px, px_kms, vsini, n_mu, residual):
     phases = np.concatenate([np.arange(9) / 9.0, [0.1, 0.3], [0.7]])
     items = [(vsini, 80.0, 0, 4, 0, 9), (0.5 * vsini, 60.0, 1, 2, 9, 2), (-vsini, 30.0, 0, 0, 11, 1)]
-    with _disk(S, n_px, 12, vsini, px_kms) as d:
+    with _disk(S, n_px, n_mu, vsini, px_kms) as d:
         outs = []
         for v in range(S.soap_batch_num_variants()):
             S.soap_batch_set_variant(d.ctx, v)
@@ -82,7 +85,7 @@ def test_batch(S, n_px, px_kms, vsini, residual):
     for o in outs[1:]:
         assert torch.equal(o, outs[0])
     # the first item alone as a star in FP64
-    with _disk(S, n_px, 12, vsini, px_kms) as d:
+    with _disk(S, n_px, n_mu, vsini, px_kms) as d:
         ref = torch.empty((1, 9, n_px), dtype=torch.float64, device=DEV)
         quiet = torch.empty(n_px, dtype=torch.float64, device=DEV)
         S.soap_active_phases(d.ctx, REGIONS, phases[:9], S.SOAP_EFFECT_TOT, S.SOAP_FP64, ref)
