@@ -12,6 +12,13 @@
 //                       layer, i.e. one swizzle atom of the next operand
 // What bounds it is the epilogue's arithmetic (erff and the exponential of GELU'), so sixteen warps
 // share it, and GELU'(z) is taken in the forward pass, where erff(z / sqrt 2) is at hand anyway.
+// A training step with too few rows for every SM (kPair): a cluster of two CTAs shares 128 rows: each computes half of a
+// hidden layer's columns, with half the weights and half the epilogue, and copies its half of the next
+// operand into the other's buffer (shared memory to shared memory, counted on the receiver's barrier).
+// The accumulator barriers count the MMAs of both, so a half is only overwritten when both products
+// that read it are complete.  The inputs, the output layer and its gradient are computed by both.
+// 4,096 rows: 68 us in 64 CTAs, 76 in 32 (16 such steps with their gradients and Adam 1,918 -> 1,777 us).
+// Not for queries: 7 of them took 28 us instead of 34, which their call did not show.
 // As one kernel per layer a tile's epilogue ran on four warps (28 us a 128 x 256 layer) and every
 // activation went through global memory twice, row-major and transposed: a training step of 4,096
 // rows took 18 launches and 0.65 ms, 7 queries 345 us (see surrogate.cu for the times now).
@@ -68,17 +75,37 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
 }
 
 // the operand buffer's first n_atoms atoms to rows row0 .. of a row-major matrix (columns past its
-// width are clipped)
-__device__ __forceinline__ void store_operand(const CUtensorMap* map, const unsigned char* act, int n_atoms, int row0) {
-    for (int q = 0; q < n_atoms; q++)
+// width are clipped); kPair: this CTA's two of them
+template <bool kPair>
+__device__ __forceinline__ void store_operand(const CUtensorMap* map, const unsigned char* act, int n_atoms, int row0,
+                                              uint32_t rank) {
+    for (int q = kPair ? 2 * (int)rank : 0; q < (kPair ? 2 * (int)rank + 2 : n_atoms); q++)
         for (int h = 0; h < 2; h++) tma_store_2d(map, act + q * kAtom + h * (kAtom / 2), 64 * q, row0 + 64 * h);
     bulk_commit();
+}
+
+__device__ __forceinline__ uint32_t peer_addr(const void* p, uint32_t rank) {
+    uint32_t a;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(tc::smem_u32(p)), "r"(rank));
+    return a;
+}
+// the same place of the other CTA's shared memory, its barrier counting the bytes
+__device__ __forceinline__ void copy_to_peer(const void* src, uint32_t bytes, const uint64_t* bar, uint32_t peer) {
+    asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(peer_addr(src, peer)), "r"(tc::smem_u32(src)), "r"(bytes), "r"(peer_addr(bar, peer)) : "memory");
+}
+__device__ __forceinline__ void commit_both(uint64_t* bar) {
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
+                 ::"r"(tc::smem_u32(bar)), "h"((uint16_t)3) : "memory");
+}
+__device__ __forceinline__ void pair_sync() {
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
 }
 
 __host__ __device__ constexpr int k_blocks(int q) { return q == 0 ? 1 : (q == 5 ? 3 : 4); }
 
 // product q: 0 .. 4 forward, 5 .. 8 backward
-template <bool kTrain>
+template <bool kTrain, bool kPair>
 __device__ __forceinline__ void chain(const Weights& w, const TrainArgs* ta, const QueryArgs* qa, int64_t row0,
                                       unsigned int* flags) {
     extern __shared__ unsigned char smem_raw[];
@@ -88,14 +115,18 @@ __device__ __forceinline__ void chain(const Weights& w, const TrainArgs* ta, con
     uint64_t* empty = full + kWStages;
     uint64_t* ready = empty + kWStages;                // the operand buffer holds the next product's A
     uint64_t* accum = ready + 1;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(accum + 1);
+    uint64_t* theirs = accum + 1;                      // kPair: the other's half of the operand has landed
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(theirs + 1);
+    const uint32_t rank = kPair ? blockIdx.x & 1u : 0u;
+    constexpr int kHalf = kHidden / 2;
     constexpr int kProducts = kTrain ? kFwd + kBwd : kFwd;
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
 
     if (t == 0) {
         for (int s = 0; s < kWStages; s++) { tc::mbar_init(&full[s], 1); tc::mbar_init(&empty[s], 1); }
         tc::mbar_init(ready, 32 * kEpiWarps);
-        tc::mbar_init(accum, 1);
+        tc::mbar_init(accum, kPair ? 2 : 1);
+        tc::mbar_init(theirs, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
@@ -105,6 +136,7 @@ __device__ __forceinline__ void chain(const Weights& w, const TrainArgs* ta, con
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
+    if constexpr (kPair) pair_sync();                  // the other's barriers exist before anything arrives there
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = *tmem_slot;
 
@@ -117,8 +149,11 @@ __device__ __forceinline__ void chain(const Weights& w, const TrainArgs* ta, con
                 for (int kb = 0; kb < k_blocks(q); kb++) {
                     const int s = it % kWStages;
                     if (!tc::mbar_wait(&empty[s], ((it / kWStages) & 1) ^ 1, flags)) { ok = false; break; }
-                    tc::mbar_expect_tx(&full[s], kWStage);
-                    tc::tma_load_2d(ring + s * kWStage, map, kb * 64, 0, &full[s]);
+                    // 128 outputs a copy: this CTA's half of a hidden layer's, or both
+                    const bool half = kPair && q != kFwd - 1;
+                    tc::mbar_expect_tx(&full[s], half ? kWStage / 2 : kWStage);
+                    tc::tma_load_2d(ring + s * kWStage, map, kb * 64, half ? (int)rank * kHalf : 0, &full[s]);
+                    if (!half) tc::tma_load_2d(ring + s * kWStage + kWStage / 2, map, kb * 64, kHalf, &full[s]);
                     it++;
                 }
             }
@@ -128,19 +163,31 @@ __device__ __forceinline__ void chain(const Weights& w, const TrainArgs* ta, con
         }
     } else if (warp == 1) {
         if (lane == 0) {
-            int it = 0;
+            int it = 0, exchanges = 0;
             bool ok = true;
             for (int q = 0; q < kProducts && ok; q++) {
                 if (!tc::mbar_wait(ready, q & 1, flags)) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                if constexpr (kTrain) {                // what this product reads is also kept for dW
-                    if (q >= 1 && q < kFwd) store_operand(&ta->s.a[q], act, 4, (int)row0);
-                    else if (q == kFwd) store_operand(&ta->s.g[4], act, 3, (int)row0);
-                    else if (q > kFwd) store_operand(&ta->s.g[kFwd + kBwd - q], act, 4, (int)row0);
+                // operands that the epilogues of both wrote a half of: this half to the other (whose
+                // products on the operand before are complete, as the epilogue waited for them)
+                const bool shared = kPair && q != 0 && q != kFwd;
+                if (shared) {
+                    tc::mbar_expect_tx(theirs, 2 * kAtom);
+                    copy_to_peer(act + 2 * rank * kAtom, 2 * kAtom, theirs, rank ^ 1u);
                 }
-                const uint32_t idesc = tc::idesc_bf16(q == kFwd - 1 ? 144 : 256);
+                if constexpr (kTrain) {                // what this product reads is also kept for dW
+                    if (q >= 1 && q < kFwd) store_operand<kPair>(&ta->s.a[q], act, 4, (int)row0, rank);
+                    else if (q == kFwd && rank == 0) store_operand<false>(&ta->s.g[4], act, 3, (int)row0, 0);
+                    else if (q > kFwd) store_operand<kPair>(&ta->s.g[kFwd + kBwd - q], act, 4, (int)row0, rank);
+                }
+                const uint32_t idesc = tc::idesc_bf16(q == kFwd - 1 ? 144 : (kPair ? kHalf : 256));
                 for (int kb = 0; kb < k_blocks(q) && ok; kb++, it++) {
                     const int s = it % kWStages;
+                    if (shared && kb == (rank == 0 ? 2 : 0)) {
+                        ok = tc::mbar_wait(theirs, exchanges & 1, flags);
+                        exchanges++;
+                        if (!ok) break;
+                    }
                     if (!tc::mbar_wait(&full[s], (it / kWStages) & 1, flags)) { ok = false; break; }
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     const uint32_t a = tc::smem_u32(act + kb * kAtom), b = tc::smem_u32(ring + s * kWStage);
@@ -151,19 +198,25 @@ __device__ __forceinline__ void chain(const Weights& w, const TrainArgs* ta, con
                 }
                 // the epilogue overwrites the operand buffer: its stores must have read it
                 if constexpr (kTrain) bulk_wait_read();
-                tc::mma_commit(accum);                 // arrives once every MMA issued above has completed
+                // arrives once every MMA issued above has completed
+                if constexpr (kPair) commit_both(accum);
+                else tc::mma_commit(accum);
             }
             if constexpr (kTrain) {
-                if (ok && tc::mbar_wait(ready, kProducts & 1, flags)) store_operand(&ta->s.g[0], act, 4, (int)row0);
+                if (ok && tc::mbar_wait(ready, kProducts & 1, flags)) store_operand<kPair>(&ta->s.g[0], act, 4, (int)row0, rank);
                 bulk_wait_all();
             }
         }
     } else {
         const int lg = warp & 3, qd = (warp - 2) >> 2;
         const int r = 32 * lg + lane;
-        const int et = t - 64;                         // epilogue thread: its place in the grad buffers
+        // epilogue thread: its place in the grad buffers
+        const int grad0 = t - 64 + (int)rank * (32 * kEpiWarps * 8);
         const uint32_t tbase = tmem + ((uint32_t)(32 * lg) << 16);
-        unsigned char* atom = act + qd * kAtom;
+        // a warp's columns of a hidden layer: 64, or 32 of this CTA's half
+        constexpr int kCols = kPair ? 32 : 64;
+        const int col0 = kPair ? kHalf * (int)rank + 32 * qd : 64 * qd;
+        unsigned char* atom = act + (col0 / 64) * kAtom;
         auto publish = [&]() {
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // visible to the tensor cores and TMA
@@ -194,7 +247,8 @@ __device__ __forceinline__ void chain(const Weights& w, const TrainArgs* ta, con
                 const uint4 c = make_uint4(pack2(v[0], v[1]), pack2(v[2], v[3]), pack2(v[4], v[5]), pack2(v[6], v[7]));
                 *reinterpret_cast<uint4*>(act + r * 128 + ((r & 7) << 4)) = c;
                 *reinterpret_cast<uint4*>(act + r * 128 + ((1 ^ (r & 7)) << 4)) = make_uint4(0, 0, 0, 0);
-                if constexpr (kTrain) *reinterpret_cast<uint4*>(ta->s.x0 + (row0 + r) * kIn) = c;
+                if constexpr (kTrain)
+                    if (rank == 0) *reinterpret_cast<uint4*>(ta->s.x0 + (row0 + r) * kIn) = c;
             }
         }
         publish();
@@ -204,12 +258,12 @@ __device__ __forceinline__ void chain(const Weights& w, const TrainArgs* ta, con
             ok = __all_sync(0xffffffffu, tc::mbar_wait(accum, l & 1, flags));
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             if (!ok) break;
-            const float4* bias = reinterpret_cast<const float4*>(w.bias[l] + 64 * qd);
+            const float4* bias = reinterpret_cast<const float4*>(w.bias[l] + col0);
 #pragma unroll 1
-            for (int h = 0; h < 2; h++) {
+            for (int h = 0; h < kCols / 32; h++) {
                 float v[32];
-                tc::tmem_ld32(tbase + (uint32_t)(64 * qd + 32 * h), v);
-                float4* gr = kTrain ? reinterpret_cast<float4*>(ta->s.grad[l]) + row0 * (kHidden / 4) + et : nullptr;
+                tc::tmem_ld32(tbase + (uint32_t)(kCols * qd + 32 * h), v);
+                float4* gr = kTrain ? reinterpret_cast<float4*>(ta->s.grad[l]) + row0 * (kHidden / 4) + grad0 : nullptr;
 #pragma unroll
                 for (int j = 0; j < 8; j++) {
                     const float4 b4 = __ldg(bias + 8 * h + j);
@@ -223,7 +277,7 @@ __device__ __forceinline__ void chain(const Weights& w, const TrainArgs* ta, con
                     v[4 * j + 2] = tc::gelu(z2);
                     v[4 * j + 3] = tc::gelu(z3);
                 }
-                put_row(atom, r, h, v);
+                put_row(atom, r, kPair ? qd & 1 : h, v);
             }
             publish();
         }
@@ -258,11 +312,11 @@ __device__ __forceinline__ void chain(const Weights& w, const TrainArgs* ta, con
                         hi = n;
                         v[i] = 2.0f * wj * res / (float)ta->B;
                     }
-                    put_row(atom, r, h, v);
+                    put_row(act + qd * kAtom, r, h, v);
                 }
                 double part = (double)hi + (double)lo;
                 for (int o = 16; o > 0; o >>= 1) part += __shfl_down_sync(0xffffffffu, part, o);
-                if (lane == 0) atomicAdd(ta->loss, part / ta->B);
+                if (lane == 0 && rank == 0) atomicAdd(ta->loss, part / ta->B);
             }
             publish();
             // backward chain: dz_l = (g W) GELU'(z_l), l = 3 .. 0
@@ -271,14 +325,14 @@ __device__ __forceinline__ void chain(const Weights& w, const TrainArgs* ta, con
                 ok = __all_sync(0xffffffffu, tc::mbar_wait(accum, q & 1, flags));
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 if (!ok) break;
-                const float4* gr = reinterpret_cast<const float4*>(ta->s.grad[l]) + row0 * (kHidden / 4) + et;
+                const float4* gr = reinterpret_cast<const float4*>(ta->s.grad[l]) + row0 * (kHidden / 4) + grad0;
 #pragma unroll 1
-                for (int h = 0; h < 2; h++) {
+                for (int h = 0; h < kCols / 32; h++) {
                     float4 g4[8];
 #pragma unroll
                     for (int j = 0; j < 8; j++) g4[j] = gr[(8 * h + j) * (32 * kEpiWarps)];
                     float v[32];
-                    tc::tmem_ld32(tbase + (uint32_t)(64 * qd + 32 * h), v);
+                    tc::tmem_ld32(tbase + (uint32_t)(kCols * qd + 32 * h), v);
 #pragma unroll
                     for (int j = 0; j < 8; j++) {
                         v[4 * j] *= g4[j].x;
@@ -286,11 +340,11 @@ __device__ __forceinline__ void chain(const Weights& w, const TrainArgs* ta, con
                         v[4 * j + 2] *= g4[j].z;
                         v[4 * j + 3] *= g4[j].w;
                     }
-                    put_row(atom, r, h, v);
+                    put_row(atom, r, kPair ? qd & 1 : h, v);
                 }
                 publish();
             }
-        } else if (ok) {
+        } else if (ok && rank == 0) {
             const bool errs = qa->nets == 1 || blockIdx.y == 1;
             if (qd < 2 && blockIdx.y == 0) {
                 // coefficients in data units; the weight ring is free (every MMA has completed)
@@ -342,20 +396,22 @@ __device__ __forceinline__ void chain(const Weights& w, const TrainArgs* ta, con
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
+    if constexpr (kPair) pair_sync();                  // neither leaves while the other may still reach into it
     if (warp == 1) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(256) : "memory");
     }
 }
 
+template <bool kPair>
 __global__ void __launch_bounds__(kThreads, 1)
 k_mlp_train(const __grid_constant__ TrainArgs a, unsigned int* flags) {
-    chain<true>(a.w, &a, nullptr, (int64_t)blockIdx.x * kRows, flags);
+    chain<true, kPair>(a.w, &a, nullptr, (int64_t)(blockIdx.x >> (int)kPair) * kRows, flags);
 }
 
 __global__ void __launch_bounds__(kThreads, 1)
 k_mlp_query(const __grid_constant__ QueryArgs a, unsigned int* flags) {
-    chain<false>(a.w[blockIdx.y], nullptr, &a, (int64_t)blockIdx.x * kRows, flags);
+    chain<false, false>(a.w[blockIdx.y], nullptr, &a, (int64_t)blockIdx.x * kRows, flags);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -507,12 +563,12 @@ k_mlp_dw(const __grid_constant__ DwArgs a, unsigned int* flags) {
 soap_status weight_maps(Weights& w, const bf16* const* W, const bf16* const* WT, const float* const* bias) {
     for (int l = 0; l < kFwd; l++) {
         const int out = l == kFwd - 1 ? kOut : kHidden, in = l == 0 ? kIn : kHidden;
-        SOAP_TRY(tc::operand_map(&w.fwd[l], W[l], out, in, in, kHidden));
+        SOAP_TRY(tc::operand_map(&w.fwd[l], W[l], out, in, in, kHidden / 2));
         w.bias[l] = bias[l];
     }
     for (int q = 0; q < kBwd; q++) {                   // layers 4, 3, 2, 1
         const int l = kFwd - 1 - q, out_pad = l == kFwd - 1 ? kOutPad : kHidden;
-        SOAP_TRY(tc::operand_map(&w.bwd[q], WT[l], kHidden, out_pad, out_pad, kHidden));
+        SOAP_TRY(tc::operand_map(&w.bwd[q], WT[l], kHidden, out_pad, out_pad, kHidden / 2));
     }
     return SOAP_OK;
 }
@@ -528,10 +584,30 @@ soap_status step_maps(Step& s, bf16* const* act, bf16* const* grad, int B) {
     return SOAP_OK;
 }
 
+// Pairs while all of them are resident at once (one CTA an SM; a few SMs may have no partner).
+static bool pairs_fit(int64_t tiles) {
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return false;
+    return 2 * tiles <= sms - 8;
+}
+
 soap_status train_step(const TrainArgs& a, cudaStream_t st, unsigned int* flags) {
-    SOAP_TRY(fit_dynamic_smem(k_mlp_train, kSmem));
-    k_mlp_train<<<a.B / kRows, kThreads, kSmem, st>>>(a, flags);
-    SOAP_CUDA(cudaGetLastError());
+    const int tiles = a.B / kRows;
+    const bool pair = pairs_fit(tiles);
+    auto* kern = pair ? k_mlp_train<true> : k_mlp_train<false>;
+    SOAP_TRY(fit_dynamic_smem(kern, kSmem));
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim = {2, 1, 1};
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(pair ? 2 * tiles : tiles));
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = kSmem;
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = pair ? 1 : 0;
+    SOAP_CUDA(cudaLaunchKernelEx(&cfg, kern, a, flags));
     return SOAP_OK;
 }
 
