@@ -12,12 +12,14 @@
 //                       layer, i.e. one swizzle atom of the next operand
 // What bounds it is the epilogue's arithmetic (erff and the exponential of GELU'), so sixteen warps
 // share it, and GELU'(z) is taken in the forward pass, where erff(z / sqrt 2) is at hand anyway.
-// A training step with too few rows for every SM (kPair): a cluster of two CTAs shares 128 rows: each computes half of a
-// hidden layer's columns, with half the weights and half the epilogue, and copies its half of the next
+// A training step with too few rows for every SM (kPair): a cluster of two CTAs shares 128 rows.  Each
+// computes half of a hidden layer's columns, with half the weights and half the epilogue, and copies its half of the next
 // operand into the other's buffer (shared memory to shared memory, counted on the receiver's barrier).
 // The accumulator barriers count the MMAs of both, so a half is only overwritten when both products
 // that read it are complete.  The inputs, the output layer and its gradient are computed by both.
-// 4,096 rows: 68 us in 64 CTAs, 76 in 32 (16 such steps with their gradients and Adam 1,918 -> 1,777 us).
+// 4,096 rows: 68 us in 64 CTAs, 76 in 32 (16 such steps with their gradients and Adam 1,918 -> 1,777 us);
+// with a layer's biases, and the GELU' factors of the backward products, fetched while the product is
+// computed 65 (1,753).
 // Not for queries: 7 of them took 28 us instead of 34, which their call did not show.
 // As one kernel per layer a tile's epilogue ran on four warps (28 us a 128 x 256 layer) and every
 // activation went through global memory twice, row-major and transposed: a training step of 4,096
@@ -47,6 +49,13 @@ constexpr int kSmem = kActBytes + kWStages * kWStage + 1024 + 256;
 static_assert(kEpiWarps * 32 * 33 * 4 <= kWStages * kWStage, "the coefficient tiles reuse the weight ring");
 
 __device__ __forceinline__ float scale_in(float x, float lo, float hi) { return 2.0f * (x - lo) / (hi - lo) - 1.0f; }
+
+// volatile: the compiler would otherwise sink a read-only load past the wait to its use
+__device__ __forceinline__ float4 ld4(const float4* p) {
+    float4 v;
+    asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+    return v;
+}
 
 __device__ __forceinline__ uint32_t pack2(float a, float b) {
     const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
@@ -255,20 +264,27 @@ __device__ __forceinline__ void chain(const Weights& w, const TrainArgs* ta, con
         bool ok = true;
         // forward layers
         for (int l = 0; l < kFwd - 1 && ok; l++) {
+            // the first 32 columns' biases are fetched while the product is computed
+            const float4* bias = reinterpret_cast<const float4*>(w.bias[l] + col0);
+            float4 b4[8];
+#pragma unroll
+            for (int j = 0; j < 8; j++) b4[j] = ld4(bias + j);
             ok = __all_sync(0xffffffffu, tc::mbar_wait(accum, l & 1, flags));
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             if (!ok) break;
-            const float4* bias = reinterpret_cast<const float4*>(w.bias[l] + col0);
 #pragma unroll 1
             for (int h = 0; h < kCols / 32; h++) {
+                if (h > 0) {
+#pragma unroll
+                    for (int j = 0; j < 8; j++) b4[j] = ld4(bias + 8 * h + j);
+                }
                 float v[32];
                 tc::tmem_ld32(tbase + (uint32_t)(kCols * qd + 32 * h), v);
                 float4* gr = kTrain ? reinterpret_cast<float4*>(ta->s.grad[l]) + row0 * (kHidden / 4) + grad0 : nullptr;
 #pragma unroll
                 for (int j = 0; j < 8; j++) {
-                    const float4 b4 = __ldg(bias + 8 * h + j);
-                    const float z0 = v[4 * j] + b4.x, z1 = v[4 * j + 1] + b4.y, z2 = v[4 * j + 2] + b4.z,
-                                z3 = v[4 * j + 3] + b4.w;
+                    const float z0 = v[4 * j] + b4[j].x, z1 = v[4 * j + 1] + b4[j].y, z2 = v[4 * j + 2] + b4[j].z,
+                                z3 = v[4 * j + 3] + b4[j].w;
                     if constexpr (kTrain)
                         gr[(8 * h + j) * (32 * kEpiWarps)] =
                             make_float4(tc::gelu_grad(z0), tc::gelu_grad(z1), tc::gelu_grad(z2), tc::gelu_grad(z3));
@@ -322,15 +338,20 @@ __device__ __forceinline__ void chain(const Weights& w, const TrainArgs* ta, con
             // backward chain: dz_l = (g W) GELU'(z_l), l = 3 .. 0
             for (int q = kFwd; q < kProducts && ok; q++) {
                 const int l = kProducts - 1 - q;
+                // (as the biases)
+                const float4* gr = reinterpret_cast<const float4*>(ta->s.grad[l]) + row0 * (kHidden / 4) + grad0;
+                float4 g4[8];
+#pragma unroll
+                for (int j = 0; j < 8; j++) g4[j] = gr[j * (32 * kEpiWarps)];
                 ok = __all_sync(0xffffffffu, tc::mbar_wait(accum, q & 1, flags));
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 if (!ok) break;
-                const float4* gr = reinterpret_cast<const float4*>(ta->s.grad[l]) + row0 * (kHidden / 4) + grad0;
 #pragma unroll 1
                 for (int h = 0; h < kCols / 32; h++) {
-                    float4 g4[8];
+                    if (h > 0) {
 #pragma unroll
-                    for (int j = 0; j < 8; j++) g4[j] = gr[(8 * h + j) * (32 * kEpiWarps)];
+                        for (int j = 0; j < 8; j++) g4[j] = gr[(8 * h + j) * (32 * kEpiWarps)];
+                    }
                     float v[32];
                     tc::tmem_ld32(tbase + (uint32_t)(kCols * qd + 32 * h), v);
 #pragma unroll
