@@ -296,7 +296,7 @@ def run_ours(args):
     bytes_contract = (P * n_px * 4 + 2 * n_mu * n_px * 4 + n_class * n_px * 4 + n_px * 4)
     c_per = per_launch("contract")
     achieved = bytes_contract / (c_per * 1e-3) / 1e9
-    rl_contract = {"kernel": "k_contract<float,4,4,128> (Toeplitz contraction, active phases)", "bound": "hbm",
+    rl_contract = {"kernel": "k_contract_fold32<4,8,64> (Toeplitz contraction, active phases)", "bound": "hbm",
                    "achieved": round(achieved, 1), "peak": hbm_peak, "unit": "GB/s",
                    "frac": round(achieved / hbm_peak, 4),
                    "traffic": profiled_traffic("k_contract_f32_disk300_205800px.md") if full else None,

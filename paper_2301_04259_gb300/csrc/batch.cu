@@ -9,13 +9,13 @@
 //
 // Stages (all on the context's stream, captured once per batch shape into a CUDA graph):
 //  1 k_batch_star     per column: I per cell in fixed point, per-(column, bin) sums
-//  2 k_batch_items    per configuration: column table, quiet kernels, quiet job table
-//  3 k_batch_quiet    quiet spectrum per configuration (Toeplitz contraction)
+//  2 k_batch_items    per configuration: column table; for spectra the quiet kernels and tap groups
+//  3 k_batch_quiet    quiet spectrum per configuration (Toeplitz contraction; not for residuals)
 //  4 k_batch_regions  region centres / cell boxes per (phase, region)
-//  5 k_batch_hist     InfoMap + per-phase kernels; the last block of each phase block builds
-//                     its job table
-//  6 k_batch_contract persistent: blocks take phase blocks (all pixel tiles of one) from an
-//                     atomic ticket, in an order sorted by estimated cost (largest first)
+//  5 k_batch_hist_block  InfoMap, kernels and tap groups per phase block (k_batch_hist where its
+//                     kernels do not fit in shared memory: per phase, the last block builds the groups)
+//  6 k_batch_contract persistent: blocks take four pixel tiles of a phase block from an atomic
+//                     ticket, in an order sorted by estimated cost (largest first)
 #include <algorithm>
 #include <cmath>
 #include <numeric>
@@ -273,7 +273,7 @@ __global__ void k_batch_hist(int N, int max_r, const int* __restrict__ phase_ite
 // Stage 5 where the kernels of a phase block fit in shared memory: block per phase block, its threads
 // shared evenly by the phases, the job table built from the kernels where they are (56,060 phases in
 // blocks of four: 300 us; a block per phase, which stores its kernels for the last one to read back,
-// 499).  Its instructions bound it, half of them the job table's.
+// 499).  Its instructions bound it (67% of the issue slots).
 __global__ void __launch_bounds__(kHistThreads)
 k_batch_hist_block(int N, int max_r, const BatchItemDev* __restrict__ items, const PBlockDev* __restrict__ pblocks,
                    const RegionGeo* __restrict__ geo, const double* __restrict__ cell_mu,
@@ -747,7 +747,8 @@ soap_status batch_run(soap_ctx* c, const soap_batch_item* items, int n_items, co
     auto putd = [&](double v) { uint64_t u; memcpy(&u, &v, 8); key.push_back(u); };
     auto putp = [&](const void* p) { key.push_back((uint64_t)(uintptr_t)p); };
     put(b.n_items); put(b.n_phases); put(b.max_r); put(b.n_pblocks); put(b.n_units); put(b.n_tiles);
-    put(b.variant); put(b.n_class); put(b.linear); put(b.residual); put(b.use_smem); put(b.taps_smem); put(b.hist_smem); put(b.hist_block_smem);
+    put(b.variant); put(b.n_class); put(b.linear); put(b.residual); put(b.use_smem); put(b.taps_smem);
+    put(b.hist_smem); put(b.hist_block_smem);
     put(N); put(c->n_mu); put(c->n_taps); put((uint64_t)c->tap_min); put(c->fx_bits);
     put(c->n_px); put(c->row_len); put(c->pad);
     putd(c->delta); putd(c->lam_s); putd(c->t_quiet);

@@ -1,7 +1,7 @@
 // contract_dev.cuh -- device code of the Toeplitz contraction shared by the single-star
 // kernels (contract.cu) and the batched persistent kernel (batch.cu).
 //
-// contract_tile() computes one pixel tile of one block of PB phases:
+// contract_tile() (FP64; FP32 takes contract_tile_fold32) computes one pixel tile of PB phases:
 //   out[p][m] = F_q[m] - sum_b Q_p,b * S_q,b [m] + sum_cl C_cl[m] sum_b K_p,cl,b * S_a(cl),b [m]
 // (Eqs. 1-4 for the effect `eff`), from a tap table (group starts, per-tap row offsets,
 // coefficients [tap][PB]).  One thread owns R pixels m = m0 + threadIdx.x + r*THREADS; acc
@@ -30,13 +30,7 @@ struct EffectList {
 // 256-byte aligned and every job's block is a multiple of PB elements).
 template <typename T, int PB>
 __device__ __forceinline__ void load_coefs(const T* __restrict__ src, T (&cv)[PB]) {
-    if constexpr (sizeof(T) == 4 && PB % 4 == 0) {
-#pragma unroll
-        for (int q = 0; q < PB / 4; q++) {
-            const float4 t = __ldg(reinterpret_cast<const float4*>(src) + q);
-            cv[4 * q] = t.x; cv[4 * q + 1] = t.y; cv[4 * q + 2] = t.z; cv[4 * q + 3] = t.w;
-        }
-    } else if constexpr (sizeof(T) == 8 && PB % 2 == 0) {
+    if constexpr (sizeof(T) == 8 && PB % 2 == 0) {
 #pragma unroll
         for (int q = 0; q < PB / 2; q++) {
             const double2 t = __ldg(reinterpret_cast<const double2*>(src) + q);
@@ -310,7 +304,7 @@ __device__ __forceinline__ void contract_tile_fold64(int64_t n_px, const Rows<do
 // and mu bin are about 3.5 consecutive ones, in 1.3 groups of eight); the taps a group lacks are
 // skipped by its (uniform) mask.  The phase block's groups and coefficients are staged in shared
 // memory, which takes their latency out of the loop, and the registers are held to nine blocks of 64
-// threads an SM: the row loads (60% from L1, the others from L2) need the warps more than the next
+// threads an SM or more (96 registers, ten blocks): the row loads (60% from L1, the others from L2) need the warps more than the next
 // group's values in registers ahead of time.  Taps are added in falling order of offset, that is
 // rising tap, with the roundings of the form tap by tap; the accumulators of pixel pairs are updated
 // by two-wide FMAs (fma.rn.f32x2: two independent IEEE FMAs).  A contrast with a row per mu bin
