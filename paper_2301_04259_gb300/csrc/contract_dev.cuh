@@ -45,7 +45,7 @@ __device__ __forceinline__ void load_coefs(const T* __restrict__ src, T (&cv)[PB
 // Region classes as the contraction sees them: the type of class cl (which active rows it
 // convolves) and its contrast C_cl at pixel m.  TableContrast reads precomputed rows
 // [n_class][n_px]; PlanckContrast32 evaluates the Planck ratio of Sect. 4.3.1 in FP32 with the
-// same operations as k_contrast32 (so both give the same values).
+// same operations as k_contrast32 (so both give the same values, except where load() takes a line).
 template <typename T>
 struct TableContrast {
     const T* rows;
