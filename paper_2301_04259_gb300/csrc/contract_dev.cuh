@@ -304,10 +304,10 @@ __device__ __forceinline__ void contract_tile_fold64(int64_t n_px, const Rows<do
 // and mu bin are about 3.5 consecutive ones, in 1.3 groups of eight); the taps a group lacks are
 // skipped by its (uniform) mask.  The phase block's groups and coefficients are staged in shared
 // memory, which takes their latency out of the loop, and the registers are held to nine blocks of 64
-// threads an SM or more (96 registers, ten blocks): the row loads (60% from L1, the others from L2) need the warps more than the next
-// group's values in registers ahead of time.  Taps are added in falling order of offset, that is
-// rising tap, with the roundings of the form tap by tap; the accumulators of pixel pairs are updated
-// by two-wide FMAs (fma.rn.f32x2: two independent IEEE FMAs).  A contrast with a row per mu bin
+// threads an SM or more (96 registers, ten blocks): the row loads (60% from L1, the others from L2)
+// need the warps more than the next group's values in registers ahead of time.  Taps are added in
+// falling order of offset, that is rising tap, with the roundings of the form tap by tap; the
+// accumulators of pixel pairs are updated by two-wide FMAs (fma.rn.f32x2: two independent IEEE FMAs).  A contrast with a row per mu bin
 // (n_sub = n_mu) is a segment of one bin each.
 //
 // 100 phases x 205,800 pixels, 3 classes: 73 -> 57 us; 37 phases x 61,747 pixels, a contrast row per
