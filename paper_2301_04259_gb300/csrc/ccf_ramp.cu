@@ -33,6 +33,8 @@
 #include <cstring>
 #include <vector>
 
+#include <math_constants.h>
+
 #include "soap_internal.cuh"
 
 namespace soap {
@@ -72,7 +74,7 @@ __global__ void k_ramp_units(int l0, int l1, int L, const int* __restrict__ U, c
     for (int j = 0; j < n; j++) rank += sf[j] < f || (sf[j] == f && j < i);
     const int l = a + i;
     RampLine d;
-    d.w = valid[l] ? w64[l] : 0.0;                     // lines whose box leaves the grid: skipped
+    d.w = valid[l] ? w64[l] : 0.0;                     // lines whose box leaves the grid: weight zero
     d.wf = d.w * f;
     d.key = __double_as_longlong(f);
     d.U = U[l];
@@ -86,11 +88,43 @@ struct RampArgs {
     const int* ev_start;                         // [groups + 1]
     const RampFinal* fin;                        // [n_v]
     const int* U;                                // box starts of the lines in mask order, from the first used
+    const int* S;                                // [n_v] shifts of the velocities: pixels and fractions
+    const double* g;
     const double* spectra;
     double* partial;
+    double box;
     int64_t n_px;
     int n_lines, L, units, per_block, groups, n_events, n_slots, o_min, n_v, n_spec, max_rows;
 };
+
+// A running sum also holds the pixels that a velocity's boxes only reach in other pieces, and pixels under
+// lines of weight zero; what they add cancels, exactly in exact arithmetic.  An infinity or a NaN does not
+// cancel, and a pixel far above the others leaves its rounding behind.  So a block's sum of one velocity
+// is only taken where it is not small against the largest pixel times the sum of |weights| (a sum of n
+// lines is some n w b F of at most n w F_max: ratios of 2 to 40 for spectra, boxes of a quarter of a
+// pixel and more); elsewhere ramp_direct adds it line by line over the pixels that its boxes do cover.
+constexpr double kRampTrust = 256.0;
+
+__device__ __noinline__ double ramp_direct(const RampArgs& g, int spec, int k, int l0, int l1) {
+    const double* F = g.spectra + (int64_t)spec * g.n_px;
+    const int Sk = g.S[k];
+    const double gk = g.g[k];
+    double v = 0.0;
+    for (int l = l0; l < l1; l++) {
+        const RampLine c = g.lines[l];
+        if (c.w == 0.0) continue;                      // also the lines whose box leaves the grid
+        const double fr = __longlong_as_double(c.key) + gk;
+        const int carry = fr >= 1.0;
+        const double phi = fr - carry, rest = phi + g.box - 1.0;
+        const int64_t n = (int64_t)c.U + Sk + carry;
+        if (n >= 0 && n < g.n_px) v = fma(c.w * fmin(1.0 - phi, g.box), F[n], v);
+        if (rest > 0.0 && n + 1 >= 0 && n + 1 < g.n_px) v = fma(c.w * rest, F[n + 1], v);
+    }
+    return v;
+}
+
+// high word of |x|: ordered as |x| is, NaN above all
+__device__ __forceinline__ int abs_hi(double x) { return __double2hiint(x) & 0x7fffffff; }
 
 __global__ void __launch_bounds__(32 * kRampMaxGroups, 1)
 k_ccf_ramp(const __grid_constant__ RampArgs g, unsigned int* flags) {
@@ -100,11 +134,15 @@ k_ccf_ramp(const __grid_constant__ RampArgs g, unsigned int* flags) {
     double* tot = reinterpret_cast<double*>(lines + g.L);          // [groups][A, B][32]
     double* acc = tot + g.groups * 64;                             // [n_slots][8]
     unsigned char* win = reinterpret_cast<unsigned char*>(acc + g.n_slots * 8);
+    __shared__ int s_big[kRampSpec];                               // largest pixel of each spectrum
+    __shared__ double s_weights;                                   // sum of the lines' |weights|
     const int t = threadIdx.x, n_thr = blockDim.x, warp = t >> 5, lane = t & 31;
     const int q = lane >> 3, s8 = lane & 7;
     const int s0 = blockIdx.y * kRampSpec, ns = min(kRampSpec, g.n_spec - s0);
     for (int i = t; i < g.n_events; i += n_thr) ev[i] = g.events[i];
     for (int i = t; i < g.groups * 64 + g.n_slots * 8; i += n_thr) tot[i] = 0.0;
+    if (t < kRampSpec) s_big[t] = 0;
+    int big0 = 0, big1 = 0;                            // of the two spectra whose pixels this thread stages
     const int e0 = warp < g.groups ? g.ev_start[warp] : 0;
     const int u1 = min(g.units, (int)(blockIdx.x + 1) * g.per_block);
     for (int u = blockIdx.x * g.per_block; u < u1; u++) {
@@ -130,6 +168,8 @@ k_ccf_ramp(const __grid_constant__ RampArgs g, unsigned int* flags) {
             const double v0 = on && 2 * part < ns ? __ldg(src) : 0.0;
             const double v1 = on && 2 * part + 1 < ns ? __ldg(src + g.n_px) : 0.0;
             *reinterpret_cast<double2*>(win + x * kRampRow + 16 * part) = make_double2(v0, v1);
+            big0 = max(big0, abs_hi(v0));
+            big1 = max(big1, abs_hi(v1));
         }
         __syncthreads();
         if (warp < g.groups) {
@@ -163,6 +203,15 @@ k_ccf_ramp(const __grid_constant__ RampArgs g, unsigned int* flags) {
             tot[warp * 64 + 32 + lane] += B;
         }
     }
+    atomicMax(&s_big[2 * (t & 3)], big0);
+    atomicMax(&s_big[2 * (t & 3) + 1], big1);
+    const int b0 = min(g.n_lines, (int)blockIdx.x * g.per_block * g.L), b1 = min(g.n_lines, u1 * g.L);
+    if (warp == 0) {
+        double sum = 0.0;
+        for (int l = b0 + lane; l < b1; l += 32) sum += fabs(g.lines[l].w);
+        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        if (lane == 0) s_weights = sum;
+    }
     __syncthreads();
     // last pieces, slots, one partial row per spectrum
     for (int i = t; i < g.n_v * kRampSpec; i += n_thr) {
@@ -179,6 +228,8 @@ k_ccf_ramp(const __grid_constant__ RampArgs g, unsigned int* flags) {
                 v = fma(f.beta[j], tot[at + 32], v);
             }
         }
+        const double most = __hiloint2double(s_big[s], 0) * s_weights;
+        if (!(most <= kRampTrust * fabs(v) && most < CUDART_INF)) v = ramp_direct(g, s0 + s, k, b0, b1);
         g.partial[((int64_t)blockIdx.x * g.n_spec + s0 + s) * g.n_v + k] = v;
     }
 }
@@ -347,6 +398,9 @@ soap_status ccf_ramp(soap_ctx* c, const CcfState& st, const CcfPlan& p, const do
     a.ev_start = reinterpret_cast<const int*>(base + r.o_start);
     a.fin = reinterpret_cast<const RampFinal*>(base + r.o_fin);
     a.U = p.U + r.l0;
+    a.S = p.S;
+    a.g = p.g64;
+    a.box = 2.0 * p.h;
     a.spectra = spectra;
     a.partial = partial;
     a.n_px = c->n_px;
