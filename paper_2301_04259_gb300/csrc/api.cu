@@ -37,6 +37,7 @@ soap_status ensure(DevBuf& b, size_t bytes) {
     cudaError_t e = cudaMalloc(&b.p, nb);
     if (e != cudaSuccess) {
         b.p = nullptr;
+        cudaGetLastError();                            // reported here, not by the next launch
         set_error("cudaMalloc(%zu) failed: %s", nb, cudaGetErrorString(e));
         return SOAP_ENOMEM;
     }
@@ -58,6 +59,7 @@ soap_status ensure_host(HostBuf& b, size_t bytes) {
     cudaError_t e = cudaMallocHost(&b.p, bytes);
     if (e != cudaSuccess) {
         b.p = nullptr;
+        cudaGetLastError();
         set_error("cudaMallocHost(%zu) failed: %s", bytes, cudaGetErrorString(e));
         return SOAP_ENOMEM;
     }
@@ -96,6 +98,7 @@ soap_status upload_small(soap_ctx* c, void* dst, const void* src, size_t bytes) 
         void* h = nullptr;
         cudaError_t e = cudaMallocHost(&h, kRingBytes);
         if (e != cudaSuccess) {
+            cudaGetLastError();
             set_error("cudaMallocHost(%zu) failed: %s", kRingBytes, cudaGetErrorString(e));
             return SOAP_ENOMEM;
         }

@@ -1329,7 +1329,7 @@ soap_status ccf_prepare(soap_ctx* c, CcfState& st, const double* mask_lambda, co
     }
     if (!same_tab) st.ramp.ok = false;
     // FP64 spectra, boxes no wider than a pixel, sorted mask
-    const bool ramp = sorted && !f32 && ccf_ramp_plan(c, st, mask_lambda, p, sms);
+    if (sorted && !f32) SOAP_TRY(ccf_ramp_plan(c, st, mask_lambda, p, sms));
     // tensor-core form (FP32 spectra, sorted mask): pixel chunks of one wave of CTAs
     if (tc && f32 && sorted && ccf_tc_fits(n_v)) {
         p.tc_chunk = ccf_tc_chunk(c->n_px, n_spec, sms);
@@ -1403,7 +1403,7 @@ soap_status ccf_prepare(soap_ctx* c, CcfState& st, const double* mask_lambda, co
         if (tb) timer_end(c, SOAP_TIMER_CCF_AUX, tb);
     }
     if (p.tc_chunk && !st.m_ok) SOAP_TRY(ccf_tc_build_m(c, st, p));
-    if (ramp) SOAP_TRY(ccf_ramp_build(c, st, p));
+    if (p.ramp_L) SOAP_TRY(ccf_ramp_build(c, st, p));
     return SOAP_OK;
 }
 

@@ -308,18 +308,18 @@ static void ramp_velocities(RampState& r, double v_lo, double v_step, int n_v, d
     r.n_events = (int)events.size();
 }
 
-// Lines per unit and units per block for this mask and number of spectra; false where the form does
-// not apply.  A unit's rows and tables take one block's whole shared memory: the more lines a unit
+// Lines per unit and units per block for this mask and number of spectra; p.ramp_L stays 0 where the form
+// does not apply.  A unit's rows and tables take one block's whole shared memory: the more lines a unit
 // has, the fewer events there are to a line.
-bool ccf_ramp_plan(soap_ctx* c, CcfState& st, const double* mask_lambda, CcfPlan& p, int sms) {
+soap_status ccf_ramp_plan(soap_ctx* c, CcfState& st, const double* mask_lambda, CcfPlan& p, int sms) {
     RampState& r = st.ramp;
     const double b = 2.0 * p.h;
-    if (p.f32 || !(b <= 1.0)) return false;
+    if (p.f32 || !(b <= 1.0)) return SOAP_OK;
     const double s_lo = std::atanh(p.v_lo / kCKms) / c->delta;
     const double s_hi = std::atanh((p.v_lo + p.v_step * (p.n_v - 1)) / kCKms) / c->delta;
-    if (!((s_hi - s_lo + 4.0) / 4.0 + 1.0 <= kRampMaxGroups) || std::fabs(s_lo) > 1e6 || std::fabs(s_hi) > 1e6) return false;
+    if (!((s_hi - s_lo + 4.0) / 4.0 + 1.0 <= kRampMaxGroups) || std::fabs(s_lo) > 1e6 || std::fabs(s_hi) > 1e6) return SOAP_OK;
     const int tiles = (p.n_spec + kRampSpec - 1) / kRampSpec;
-    if (tiles > 65535) return false;
+    if (tiles > 65535) return SOAP_OK;
     if (!r.ok) {
         // the lines that can be valid (two pixels of margin: the others weigh nothing)
         const double lo = c->lam_s * std::exp((-0.5 - s_lo + p.h - 2.0) * c->delta);
@@ -331,17 +331,16 @@ bool ccf_ramp_plan(soap_ctx* c, CcfState& st, const double* mask_lambda, CcfPlan
         std::vector<int> start;
         std::vector<RampFinal> fin;
         ramp_velocities(r, p.v_lo, p.v_step, p.n_v, c->delta, b, events, start, fin);
-        if (r.groups > kRampMaxGroups || r.l1 <= r.l0) return false;
+        if (r.groups > kRampMaxGroups || r.l1 <= r.l0) return SOAP_OK;
         auto al = [](size_t x) { return (x + 255) / 256 * 256; };
         r.o_start = al(events.size() * sizeof(RampEvent));
         r.o_fin = al(r.o_start + start.size() * sizeof(int));
         r.o_lines = al(r.o_fin + fin.size() * sizeof(RampFinal));
-        if (ensure(r.tab, r.o_lines + (size_t)(r.l1 - r.l0) * sizeof(RampLine)) != SOAP_OK) return false;
+        SOAP_TRY(ensure(r.tab, r.o_lines + (size_t)(r.l1 - r.l0) * sizeof(RampLine)));
         char* base = r.tab.as<char>();
-        if (upload_small(c, base, events.data(), events.size() * sizeof(RampEvent)) != SOAP_OK ||
-            upload_small(c, base + r.o_start, start.data(), start.size() * sizeof(int)) != SOAP_OK ||
-            upload_small(c, base + r.o_fin, fin.data(), fin.size() * sizeof(RampFinal)) != SOAP_OK)
-            return false;
+        SOAP_TRY(upload_small(c, base, events.data(), events.size() * sizeof(RampEvent)));
+        SOAP_TRY(upload_small(c, base + r.o_start, start.data(), start.size() * sizeof(int)));
+        SOAP_TRY(upload_small(c, base + r.o_fin, fin.data(), fin.size() * sizeof(RampFinal)));
         r.ok = true;
         r.built_L = 0;
     }
@@ -368,13 +367,13 @@ bool ccf_ramp_plan(soap_ctx* c, CcfState& st, const double* mask_lambda, CcfPlan
             if (L == 1) break;
         }
     }
-    if (!r.L) return false;
+    if (!r.L) return SOAP_OK;
     p.ramp_L = r.L;
     p.ramp_rows = r.rows;
     p.ramp_units = (n + r.L - 1) / r.L;
     p.ramp_per_block = r.per_block;
     p.n_chunks = (p.ramp_units + r.per_block - 1) / r.per_block;
-    return true;
+    return SOAP_OK;
 }
 
 // The unit-ordered line tables (after the line tables they are made from).

@@ -424,7 +424,7 @@ int64_t ccf_tc_chunk(int64_t n_px, int n_spec, int sms);
 // Mask matrix of the tensor-core form for the tables of `st` (once per mask and grid).
 soap_status ccf_tc_build_m(soap_ctx* c, CcfState& st, const CcfPlan& p);
 // the FP64 CCF of boxes no wider than a pixel (ccf_ramp.cu)
-bool ccf_ramp_plan(soap_ctx* c, CcfState& st, const double* mask_lambda, CcfPlan& p, int sms);
+soap_status ccf_ramp_plan(soap_ctx* c, CcfState& st, const double* mask_lambda, CcfPlan& p, int sms);
 soap_status ccf_ramp_build(soap_ctx* c, CcfState& st, const CcfPlan& p);
 soap_status ccf_ramp(soap_ctx* c, const CcfState& st, const CcfPlan& p, const double* spectra, double* partial);
 soap_status ccf_tc(soap_ctx* c, CcfState& st, const CcfPlan& p, const float* spectra, float* partial);
