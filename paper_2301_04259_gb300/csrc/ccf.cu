@@ -1327,7 +1327,8 @@ soap_status ccf_prepare(soap_ctx* c, CcfState& st, const double* mask_lambda, co
             p.n_chunks = p.tile_blocks;
         }
     }
-    if (!same_tab) st.ramp.ok = false;
+    // what is kept of the tables before is gone from here on: a call that fails below has left parts of its own
+    if (!same_tab) st.lines_ok = st.m_ok = st.ramp.ok = false;
     // FP64 spectra, boxes no wider than a pixel, sorted mask
     if (sorted && !f32) SOAP_TRY(ccf_ramp_plan(c, st, mask_lambda, p, sms));
     // tensor-core form (FP32 spectra, sorted mask): pixel chunks of one wave of CTAs
@@ -1359,12 +1360,7 @@ soap_status ccf_prepare(soap_ctx* c, CcfState& st, const double* mask_lambda, co
     size_t o_y = al(o_ccf + (size_t)n_spec * n_v * 8);
     size_t total = o_y + (size_t)n_spec * n_v * 8;
     SOAP_TRY(ensure(st.tmp, total));
-    if (!same_tab) {
-        // a grown table buffer moves: the old tables (and the mask matrix) are gone with it
-        st.lines_ok = false;
-        st.m_ok = false;
-        SOAP_TRY(ensure(st.tab, tab_total));
-    }
+    if (!same_tab) SOAP_TRY(ensure(st.tab, tab_total));
     char* tab = st.tab.as<char>();
     char* base = st.tmp.as<char>();
     double* d_lam = (double*)(tab + o_lam);
