@@ -763,7 +763,7 @@ soap_status batch_run(soap_ctx* c, const soap_batch_item* items, int n_items, co
     if (rv) {
         putp(c->b_win.p); putp(c->b_ccf.tab.p); putp(c->b_ccf.tmp.p); putp(c->b_ccf.m.p); putp(c->b_ccf.ramp.tab.p);
         put(rvp.n_lines); put(rvp.n_v); put(rvp.n_chunks); put(rvp.n_wgroups); put(rvp.windowed);
-        put(rvp.win_lines); put(rvp.win_nb);
+        put(rvp.chunk_lines); put(rvp.win_lines); put(rvp.win_nb);
         put(rvp.ramp_L); put(rvp.ramp_rows); put(rvp.ramp_units); put(rvp.ramp_per_block);
         put(rvp.tile_np); put(rvp.tile_blocks); put(rvp.tile_lines); put((uint64_t)rvp.tc_chunk);
         putd(rvp.v_lo); putd(rvp.v_step); putd(rvp.h);

@@ -27,7 +27,7 @@
 namespace soap {
 
 constexpr int kLinesPerChunk = 128;      // generic kernel (at most)
-constexpr int kWinLines = 32;             // windowed kernel: lines per chunk at most
+constexpr int kWinLines = 32;             // windowed kernel: lines per chunk and window at most
 constexpr int kWinMax = 768;              // staged pixels per block (window budget)
 constexpr int kWinSB32 = 16, kWinSB64 = 8; // windowed kernel: spectra per block (FP32, FP64)
 constexpr int kReduceSplit = 8;
@@ -116,16 +116,16 @@ __global__ void k_ccf_partial(int n_lines, const int* __restrict__ U, const T* _
 // lines can reach, for its SB spectra, in shared memory as [pixel][SB] (one 16-byte vector per
 // 4 spectra), so each overlap costs SB/4 vector loads instead of SB scattered global loads.
 // Blocks whose window would not fit fall back to global loads.
-// Windowed form for masks sorted by wavelength.  Block = (group of line chunks, SB spectra);
-// thread = velocity k.  Per chunk the block stages the pixels its lines can reach, for its SB
-// spectra, in shared memory as padded rows [pixel][SB] (one 16-byte vector per VW spectra).
+// Windowed form for masks sorted by wavelength.  Block = (chunk of lines, SB spectra); thread =
+// velocity k.  Per window (some of the chunk's lines) the block stages the pixels its lines can reach, for
+// its SB spectra, in shared memory as padded rows [pixel][SB] (one 16-byte vector per VW spectra).
 // For each line the box position (integer pixel + fraction) is computed once and reused for
 // all SB spectra; the box covers at most NB pixels, handled branch-free (zero overlaps add
-// zero).  Chunks whose window does not fit fall back to global loads.  win_lines (at most
-// kWinLines) lines per chunk: see ccf_window_lines.
+// zero).  Windows that do not fit fall back to global loads.  chunk_lines lines per chunk, win_lines
+// (at most kWinLines) per window: see ccf_chunk_lines and ccf_window_lines.
 template <typename T, int SB, int NB>
 __global__ void __launch_bounds__(256)
-k_ccf_window(int n_lines, int win_lines, const int* __restrict__ U, const T* __restrict__ f,
+k_ccf_window(int n_lines, int chunk_lines, int win_lines, const int* __restrict__ U, const T* __restrict__ f,
              const int* __restrict__ valid, const T* __restrict__ wl_, int n_v,
              const int* __restrict__ S, const T* __restrict__ g, double box, int64_t n_px,
              int n_spec, const T* __restrict__ spectra, T* __restrict__ partial) {
@@ -140,7 +140,7 @@ k_ccf_window(int n_lines, int win_lines, const int* __restrict__ U, const T* __r
     T* win = reinterpret_cast<T*>(smraw);
     const int s0 = blockIdx.y * SB;
     const int ns = min(SB, n_spec - s0);
-    const int n_chunks = (n_lines + win_lines - 1) / win_lines;
+    const int l_end = min(n_lines, ((int)blockIdx.x + 1) * chunk_lines);
     const T boxT = (T)box;
     const int k = threadIdx.x;
     const bool active = k < n_v;
@@ -149,15 +149,14 @@ k_ccf_window(int n_lines, int win_lines, const int* __restrict__ U, const T* __r
     T acc[SB];
 #pragma unroll
     for (int s = 0; s < SB; s++) acc[s] = T(0);
-    for (int chunk = blockIdx.x; chunk < n_chunks; chunk += gridDim.x) {
-        const int l0 = chunk * win_lines;
-        const int l1 = min(n_lines, l0 + win_lines);
+    for (int l0 = (int)blockIdx.x * chunk_lines; l0 < l_end; l0 += win_lines) {
+        const int l1 = min(l_end, l0 + win_lines);
         // window [n_lo, n_hi) with a margin on both sides; pixels off the grid stage as 0
         const int64_t n_lo = (int64_t)U[l0] + S[0] - 2;
         const int64_t n_hi = (int64_t)U[l1 - 1] + S[n_v - 1] + NB + 2;
         const int W = (int)(n_hi - n_lo);
         const bool staged = W >= NB && W <= kWinMax;
-        __syncthreads();                                  // previous chunk done with the window
+        __syncthreads();                                  // done with the window before
         for (int j = threadIdx.x; j < l1 - l0; j += blockDim.x) {
             const int l = l0 + j;
             sB[j] = (int)((int64_t)U[l] - n_lo);
@@ -1237,16 +1236,24 @@ static cudaError_t fit_f32_launch(int n_spec, cudaStream_t st, bool early, int n
 // pixels a box of half width h covers at most, as a window's NB
 static int ccf_window_nb(double h) { return 2.0 * h <= 1.0 ? 2 : (2.0 * h <= 7.0 ? 8 : 16); }
 
-// Lines per chunk of the windowed kernel.  A chunk of kWinLines lines costs one window, so it is
-// the cheapest per line, but a chunk is a block's whole work: with few lines there must be fewer
-// to a chunk for every SM to get some (four blocks per SM: 30 lines of a 4,096-pixel grid and 25
-// spectra in 2 blocks took 346 us; now one line to a chunk, and the whole
-// call of that size 117 us instead of 307), and where lines are sparse (136 pixels apart there), their
-// windows together must still fit the stage, else every overlap reads global memory.
-static int ccf_window_lines(int n_lines, int64_t n_px, double sweep, int nb, int spec_blocks, int sms) {
+// Lines per chunk of the windowed kernel, that is per partial sum.  A chunk is a block's whole work: with
+// few lines there must be fewer than kWinLines to a chunk for every SM to get some (four blocks per SM: 30
+// lines of a 4,096-pixel grid and 25 spectra in 2 blocks took 346 us; now one line to a chunk, and the
+// whole call of that size 117 us instead of 307).  Chunks are shorter for no other reason, so there are
+// n_lines / kWinLines partial sums a spectrum and velocity, or as many as four blocks per SM write.
+static int ccf_chunk_lines(int n_lines, int spec_blocks, int sms) {
     const double fill = (double)n_lines * spec_blocks / (4.0 * sms);
+    return std::max(1, (int)std::min<double>(kWinLines, fill));
+}
+
+// Lines per window: as many of a chunk's as fit the stage together, else every overlap reads global
+// memory; all of them where the velocities alone sweep over more than the stage, and none would fit.
+// 1,000 FP32 spectra, pixels of 0.122 km/s: 3,000 lines 133 pixels apart, a sweep of 490 pixels (two
+// lines a window) 2.19 ms and 178 MB of scratch, 3.49 ms and 5.5 GB with a partial sum per window; 5,000
+// lines, a sweep of 820 pixels 9.2 ms and 244 MB, 12.0 ms and 7.7 GB a line at a time.
+static int ccf_window_lines(int chunk_lines, int n_lines, int64_t n_px, double sweep, int nb) {
     const double fit = (kWinMax - sweep - nb - 6) / ((double)n_px / n_lines);
-    return std::max(1, (int)std::min<double>(kWinLines, std::min(fill, fit)));
+    return fit >= 1.0 ? (int)std::min<double>(chunk_lines, fit) : chunk_lines;
 }
 
 bool ccf_mask_same(const CcfState& st, const double* mask_lambda, const double* mask_weight,
@@ -1291,10 +1298,11 @@ soap_status ccf_prepare(soap_ctx* c, CcfState& st, const double* mask_lambda, co
     SOAP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const int win_sb = f32 ? kWinSB32 : kWinSB64;
     p.win_nb = ccf_window_nb(p.h);
-    p.win_lines = ccf_window_lines(n_lines, c->n_px,
+    p.chunk_lines = ccf_chunk_lines(n_lines, (n_spec + win_sb - 1) / win_sb, sms);
+    p.win_lines = ccf_window_lines(p.chunk_lines, n_lines, c->n_px,
                                    (std::atanh((v_lo + (n_v - 1) * v_step) / kCKms) - std::atanh(v_lo / kCKms)) / c->delta,
-                                   p.win_nb, (n_spec + win_sb - 1) / win_sb, sms);
-    p.n_wgroups = (n_lines + p.win_lines - 1) / p.win_lines;   // one chunk of lines per block
+                                   p.win_nb);
+    p.n_wgroups = (n_lines + p.chunk_lines - 1) / p.chunk_lines;   // one chunk of lines per block
     p.n_chunks = p.windowed ? p.n_wgroups : (n_lines + kLinesPerChunk - 1) / kLinesPerChunk;
     // register-tiled kernel (FP32, sorted mask): pixels a group of kTileVT velocities can reach
     // for one line, from the largest spread of kTileVT consecutive box positions
@@ -1446,7 +1454,7 @@ soap_status ccf_enqueue(soap_ctx* c, CcfState& st, const CcfPlan& p, const void*
             SOAP_CUDA(cudaFuncSetAttribute(k_ccf_window<T, SB, NB>,                                \
                                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM)); \
             k_ccf_window<T, SB, NB><<<GRID, threads, SMEM, c->stream>>>(                          \
-                n_lines, p.win_lines, p.U, F, p.valid, WT, n_v, p.S, G, box, c->n_px, n_spec,      \
+                n_lines, p.chunk_lines, p.win_lines, p.U, F, p.valid, WT, n_v, p.S, G, box, c->n_px, n_spec,      \
                 (const T*)SPEC, reinterpret_cast<T*>(d_part));                                     \
         } while (0)
         if (p.f32) {
@@ -1602,8 +1610,7 @@ extern "C" soap_status soap_rv_ccf_static(double lambda_start_A, double lambda_e
     SOAP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     int chunk_lines = kLinesPerChunk;
     if (spectra_f32)
-        chunk_lines = ccf_window_lines(n_lines, n_px, (std::atanh(v_hi / kCKms) - std::atanh(v_lo / kCKms)) / delta,
-                                       ccf_window_nb(h), (n_spec + kWinSB32 - 1) / kWinSB32, sms);
+        chunk_lines = ccf_chunk_lines(n_lines, (n_spec + kWinSB32 - 1) / kWinSB32, sms);
     // scratch layout, as in rv_ccf_run (generic line order kernel); chunks of kLinesPerChunk where the
     // shorter ones' partial sums would not fit
     if (((int64_t)(n_lines / chunk_lines) + 3) * n_spec * n_v * 8 + (int64_t)n_lines * 24 + n_v * 16 + 4096 >

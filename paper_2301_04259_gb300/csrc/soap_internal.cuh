@@ -145,7 +145,7 @@ struct CcfPlan {
     int n_spec = 0, n_lines = 0, n_v = 0, f32 = 0;
     double v_lo = 0, v_step = 0, h = 0;
     bool windowed = false;
-    int n_wgroups = 0, n_chunks = 0, win_lines = 0, win_nb = 0;
+    int n_wgroups = 0, n_chunks = 0, chunk_lines = 0, win_lines = 0, win_nb = 0;
     int tile_np = 0, tile_blocks = 0, tile_lines = 0;
     int64_t tc_chunk = 0;
     int tc_smin = 0, tc_smax = 0;
