@@ -1366,7 +1366,8 @@ soap_status ccf_prepare(soap_ctx* c, CcfState& st, const double* mask_lambda, co
     size_t o_part = 0;
     size_t o_ccf = al(o_part + (size_t)p.n_chunks * n_spec * n_v * 8);
     size_t o_y = al(o_ccf + (size_t)n_spec * n_v * 8);
-    size_t total = o_y + (size_t)n_spec * n_v * 8;
+    size_t o_bad = al(o_y + (size_t)n_spec * n_v * 8);
+    size_t total = o_bad + (p.ramp_L ? ccf_ramp_scratch(p) : 0);
     SOAP_TRY(ensure(st.tmp, total));
     if (!same_tab) SOAP_TRY(ensure(st.tab, tab_total));
     char* tab = st.tab.as<char>();
@@ -1384,6 +1385,7 @@ soap_status ccf_prepare(soap_ctx* c, CcfState& st, const double* mask_lambda, co
     p.part = (double*)(base + o_part);
     p.ccf = (double*)(base + o_ccf);
     p.y = (double*)(base + o_y);
+    p.ramp_bad = (unsigned int*)(base + o_bad);
     if (!same_tab) {
         cudaEvent_t tb = c->profiling ? timer_begin(c) : nullptr;
         const double v_hi = v_lo + v_step * (n_v - 1);

@@ -26,6 +26,14 @@
 // as shared memory allows.  100 spectra of 205,800 pixels, 12,900 lines, 177 velocities: about
 // 0.5 ms, against 1.71 with the windowed kernel (two multiply-adds and ten more FP64 instructions per
 // line and velocity for eight spectra).
+// Values that the running sums do not give are added line by line by a kernel of their own (k_ramp_direct):
+// 5 us a call where there are none, 0.35 ms for a NaN in the same pixel of all those spectra, 1.3 ms when
+// none of the values can be taken.
+//
+// Precision (the sums of 1,170 lines against extended precision, root mean square of the relative error over
+// velocities): 2.8e-16 for boxes of 0.94 pixels, 5.6e-16 for a quarter of a pixel, 2.0e-15 for a twentieth,
+// where the sums that cancel are the larger the narrower the box; overlap by overlap, in chunks of 32
+// lines, 1.9e-16, 1.8e-16 and 3.5e-16.
 // In FP32, where the instructions around the multiply-adds count, the same form took 125 us for 317
 // spectra of 102,901 pixels against 104 of the register-tiled kernel.
 #include <algorithm>
@@ -92,6 +100,7 @@ struct RampArgs {
     const double* g;
     const double* spectra;
     double* partial;
+    unsigned int* bad;            // by (blocks of lines, of spectra), a byte of spectra for each velocity
     double box;
     int64_t n_px;
     int n_lines, L, units, per_block, groups, n_events, n_slots, o_min, n_v, n_spec, max_rows;
@@ -101,27 +110,10 @@ struct RampArgs {
 // lines of weight zero; what they add cancels, exactly in exact arithmetic.  An infinity or a NaN does not
 // cancel, and a pixel far above the others leaves its rounding behind.  So a block's sum of one velocity
 // is only taken where it is not small against the largest pixel times the sum of |weights| (a sum of n
-// lines is some n w b F of at most n w F_max: ratios of 2 to 40 for spectra, boxes of a quarter of a
-// pixel and more); elsewhere ramp_direct adds it line by line over the pixels that its boxes do cover.
+// lines is some n w b F of at most n w F_max: ratios of 2 to 40 for spectra and boxes of a quarter of a pixel
+// and more); k_ramp_direct replaces the others.  (Boxes below about a hundredth of a pixel leave it all
+// of them: 2.1 ms for the RVs of 100 spectra of 205,800 pixels, 1.9 with the windowed kernel.)
 constexpr double kRampTrust = 256.0;
-
-__device__ __noinline__ double ramp_direct(const RampArgs& g, int spec, int k, int l0, int l1) {
-    const double* F = g.spectra + (int64_t)spec * g.n_px;
-    const int Sk = g.S[k];
-    const double gk = g.g[k];
-    double v = 0.0;
-    for (int l = l0; l < l1; l++) {
-        const RampLine c = g.lines[l];
-        if (c.w == 0.0) continue;                      // also the lines whose box leaves the grid
-        const double fr = __longlong_as_double(c.key) + gk;
-        const int carry = fr >= 1.0;
-        const double phi = fr - carry, rest = phi + g.box - 1.0;
-        const int64_t n = (int64_t)c.U + Sk + carry;
-        if (n >= 0 && n < g.n_px) v = fma(c.w * fmin(1.0 - phi, g.box), F[n], v);
-        if (rest > 0.0 && n + 1 >= 0 && n + 1 < g.n_px) v = fma(c.w * rest, F[n + 1], v);
-    }
-    return v;
-}
 
 // high word of |x|: ordered as |x| is, NaN above all
 __device__ __forceinline__ int abs_hi(double x) { return __double2hiint(x) & 0x7fffffff; }
@@ -214,24 +206,87 @@ k_ccf_ramp(const __grid_constant__ RampArgs g, unsigned int* flags) {
     }
     __syncthreads();
     // last pieces, slots, one partial row per spectrum
-    for (int i = t; i < g.n_v * kRampSpec; i += n_thr) {
-        const int s = i / g.n_v, k = i - s * g.n_v;
-        if (s >= ns) break;
+    // (lane: velocity lane / 8 of four, spectrum lane mod 8)
+    for (int k0 = 4 * warp; k0 < g.n_v; k0 += n_thr / 8) {
+        const int k = min(k0 + q, g.n_v - 1);
+        const bool on = k0 + q < g.n_v && s8 < ns;
         const RampFinal f = g.fin[k];
         double v = 0.0;
 #pragma unroll
         for (int j = 0; j < 2; j++) {
-            if (f.slot[j] >= 0) v += acc[f.slot[j] * 8 + s];
+            if (f.slot[j] >= 0) v += acc[f.slot[j] * 8 + s8];
             if (f.o[j] >= 0) {
-                const int at = (f.o[j] >> 2) * 64 + 8 * (f.o[j] & 3) + s;
+                const int at = (f.o[j] >> 2) * 64 + 8 * (f.o[j] & 3) + s8;
                 v = fma(f.alpha[j], tot[at], v);
                 v = fma(f.beta[j], tot[at + 32], v);
             }
         }
-        const double most = __hiloint2double(s_big[s], 0) * s_weights;
-        if (!(most <= kRampTrust * fabs(v) && most < CUDART_INF)) v = ramp_direct(g, s0 + s, k, b0, b1);
-        g.partial[((int64_t)blockIdx.x * g.n_spec + s0 + s) * g.n_v + k] = v;
+        const double most = __hiloint2double(s_big[s8], 0) * s_weights;
+        const unsigned int bad = __ballot_sync(0xffffffffu, on && !(most <= kRampTrust * fabs(v) && most < CUDART_INF));
+        if (lane == 0) g.bad[((int64_t)blockIdx.x * gridDim.y + blockIdx.y) * ((g.n_v + 3) / 4) + k0 / 4] = bad;
+        if (on) g.partial[((int64_t)blockIdx.x * g.n_spec + s0 + s8) * g.n_v + k] = v;
     }
+}
+
+// The block sums of k_ccf_ramp that are not to be taken, line by line over the pixels that the boxes do
+// cover.  Block = (lines and spectra of a block there, 32 velocities); lane = velocity, so that a warp's
+// pixels are neighbours; eight warps share the lines.  A box's overlaps are FP64 instructions, which bound
+// this: computed once for all spectra, compared on their bits.  Where there is nothing to replace, a block
+// only reads its eight words.
+constexpr int kDirectWarps = 8;
+__global__ void __launch_bounds__(32 * kDirectWarps)
+k_ramp_direct(const __grid_constant__ RampArgs g) {
+    __shared__ double part[kDirectWarps][kRampSpec][32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int k = 32 * blockIdx.z + lane, n_words = (g.n_v + 3) / 4;
+    const unsigned int* word = g.bad + ((int64_t)blockIdx.x * gridDim.y + blockIdx.y) * n_words;
+    const unsigned int mine = k < g.n_v ? (word[k / 4] >> (8 * (k & 3))) & 255u : 0u;
+    const unsigned int any = __reduce_or_sync(0xffffffffu, mine);
+    if (any == 0) return;
+    const int s0 = blockIdx.y * kRampSpec, kk = min(k, g.n_v - 1), Sk = g.S[kk];
+    const double gk = g.g[kk];
+    const int u1 = min(g.units, (int)(blockIdx.x + 1) * g.per_block);
+    const int l0 = min(g.n_lines, (int)blockIdx.x * g.per_block * g.L), l1 = min(g.n_lines, u1 * g.L);
+    double a[kRampSpec];
+#pragma unroll
+    for (int s = 0; s < kRampSpec; s++) a[s] = 0.0;
+    for (int l = l0 + warp; l < l1; l += kDirectWarps) {
+        const RampLine c = g.lines[l];
+        if ((__double_as_longlong(c.w) << 1) == 0) continue;   // also the lines whose box leaves the grid
+        double phi = __longlong_as_double(c.key) + gk;
+        const int carry = __double2hiint(phi) >= 0x3ff00000;
+        if (carry) phi -= 1.0;
+        const double left = 1.0 - phi, rest = phi + g.box - 1.0;
+        const double ov = __double_as_longlong(left) < __double_as_longlong(g.box) ? left : g.box;
+        const int64_t n = (int64_t)c.U + Sk + carry;
+        const bool first = n >= 0 && n < g.n_px;
+        const bool second = __double_as_longlong(rest) > 0 && n + 1 >= 0 && n + 1 < g.n_px;
+        const double w0 = c.w * ov, w1 = c.w * rest;
+        const double* x = g.spectra + (int64_t)s0 * g.n_px + n;
+        double X[kRampSpec], Y[kRampSpec];
+#pragma unroll
+        for (int s = 0; s < kRampSpec; s++) {
+            const bool on = (any >> s) & 1;
+            X[s] = on && first ? __ldg(x) : 0.0;
+            Y[s] = on && second ? __ldg(x + 1) : 0.0;
+            x += g.n_px;
+        }
+#pragma unroll
+        for (int s = 0; s < kRampSpec; s++) {
+            if (!((any >> s) & 1)) continue;
+            a[s] = fma(w0, X[s], a[s]);
+            if (second) a[s] = fma(w1, Y[s], a[s]);
+        }
+    }
+#pragma unroll
+    for (int s = 0; s < kRampSpec; s++) part[warp][s][lane] = a[s];
+    __syncthreads();
+    const int s = warp;                                // one spectrum each
+    static_assert(kDirectWarps == kRampSpec, "a warp per spectrum");
+    double v = 0.0;
+#pragma unroll
+    for (int w = 0; w < kDirectWarps; w++) v += part[w][s][lane];
+    if ((mine >> s) & 1) g.partial[((int64_t)blockIdx.x * g.n_spec + s0 + s) * g.n_v + k] = v;
 }
 
 // ---------------------------------------------------------------------------------------
@@ -388,6 +443,10 @@ soap_status ccf_ramp_build(soap_ctx* c, CcfState& st, const CcfPlan& p) {
     return SOAP_OK;
 }
 
+size_t ccf_ramp_scratch(const CcfPlan& p) {
+    return (size_t)p.n_chunks * ((p.n_spec + kRampSpec - 1) / kRampSpec) * ((p.n_v + 3) / 4) * sizeof(unsigned int);
+}
+
 soap_status ccf_ramp(soap_ctx* c, const CcfState& st, const CcfPlan& p, const double* spectra, double* partial) {
     const RampState& r = st.ramp;
     const char* base = static_cast<const char*>(r.tab.p);
@@ -399,6 +458,7 @@ soap_status ccf_ramp(soap_ctx* c, const CcfState& st, const CcfPlan& p, const do
     a.U = p.U + r.l0;
     a.S = p.S;
     a.g = p.g64;
+    a.bad = p.ramp_bad;
     a.box = 2.0 * p.h;
     a.spectra = spectra;
     a.partial = partial;
@@ -418,6 +478,8 @@ soap_status ccf_ramp(soap_ctx* c, const CcfState& st, const CcfPlan& p, const do
     SOAP_TRY(fit_dynamic_smem(k_ccf_ramp, smem));
     const dim3 grid((unsigned)p.n_chunks, (unsigned)((p.n_spec + kRampSpec - 1) / kRampSpec));
     k_ccf_ramp<<<grid, 32 * std::max(r.groups, 4), smem, c->stream>>>(a, c->flags);
+    SOAP_LAUNCHED(c);
+    k_ramp_direct<<<dim3(grid.x, grid.y, (unsigned)((p.n_v + 31) / 32)), 32 * kDirectWarps, 0, c->stream>>>(a);
     SOAP_CUDA(cudaGetLastError());                     // (the caller counts the CCF kernel)
     return SOAP_OK;
 }

@@ -150,6 +150,7 @@ struct CcfPlan {
     int64_t tc_chunk = 0;
     int tc_smin = 0, tc_smax = 0;
     int ramp_L = 0, ramp_rows = 0, ramp_units = 0, ramp_per_block = 0;
+    unsigned int* ramp_bad = nullptr;    // (in CcfState::tmp)
     // device tables (in CcfState::tab) and scratch (in CcfState::tmp)
     int* U = nullptr; double* f64 = nullptr; float* f32t = nullptr; float* w32 = nullptr;
     int* valid = nullptr; double* w64 = nullptr;
@@ -426,6 +427,7 @@ soap_status ccf_tc_build_m(soap_ctx* c, CcfState& st, const CcfPlan& p);
 // the FP64 CCF of boxes no wider than a pixel (ccf_ramp.cu)
 soap_status ccf_ramp_plan(soap_ctx* c, CcfState& st, const double* mask_lambda, CcfPlan& p, int sms);
 soap_status ccf_ramp_build(soap_ctx* c, CcfState& st, const CcfPlan& p);
+size_t ccf_ramp_scratch(const CcfPlan& p);
 soap_status ccf_ramp(soap_ctx* c, const CcfState& st, const CcfPlan& p, const double* spectra, double* partial);
 soap_status ccf_tc(soap_ctx* c, CcfState& st, const CcfPlan& p, const float* spectra, float* partial);
 
