@@ -179,11 +179,11 @@ __global__ void __launch_bounds__(THREADS, 4)
 k_contract(int64_t n_px, Rows<T> rows, const long long* __restrict__ toff, const int* __restrict__ gstart,
            int G, int max_taps, const T* __restrict__ coefs, ClassTypes ctype, const T* __restrict__ contrast,
            const T* __restrict__ fq, int n_phases, EffectList effs, T* __restrict__ out,
-           const int* __restrict__ bstart, int n_mu, int fold) {
+           const int* __restrict__ bstart, int n_mu, int fold, int pb0) {
     // a kernel launched after this one with an early start (the tensor-core CCF) may begin once
     // every CTA here has started: it waits for this grid before it reads the output
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const int pb = blockIdx.y;
+    const int pb = pb0 + (int)blockIdx.y;
     const int np = min(PB, n_phases - pb * PB);
     T* out_rows = out + (int64_t)blockIdx.z * n_phases * n_px + (int64_t)pb * PB * n_px;
     const TableContrast<T> con{contrast, n_px, ctype};
@@ -226,12 +226,15 @@ static soap_status launch_contract(soap_ctx* c, int n_blocks, int G, int max_tap
     Rows<T> rows;
     rows.q = q; rows.a[0] = a0; rows.a[1] = a1;
     int64_t tiles = (c->n_px + (int64_t)THREADS * R - 1) / ((int64_t)THREADS * R);
-    dim3 grid((unsigned)tiles, (unsigned)n_blocks, (unsigned)n_eff);
-    SOAP_TIMED(c, fq ? SOAP_TIMER_CONTRACT : SOAP_TIMER_CONTRACT_QUIET,
-               k_contract<T, PB, R, THREADS><<<grid, THREADS, 0, c->stream>>>(
-                   c->n_px, rows, toff, gstart, G, max_taps, coefs, ct, contrast, fq, n_phases, el, out,
-                   bstart, c->n_mu, fold);
-               SOAP_LAUNCHED(c));
+    // at most 65,535 phase blocks a launch, a grid's limit in y
+    for (int pb0 = 0; pb0 < n_blocks; pb0 += 65535) {
+        dim3 grid((unsigned)tiles, (unsigned)std::min(n_blocks - pb0, 65535), (unsigned)n_eff);
+        SOAP_TIMED(c, fq ? SOAP_TIMER_CONTRACT : SOAP_TIMER_CONTRACT_QUIET,
+                   k_contract<T, PB, R, THREADS><<<grid, THREADS, 0, c->stream>>>(
+                       c->n_px, rows, toff, gstart, G, max_taps, coefs, ct, contrast, fq, n_phases, el, out,
+                       bstart, c->n_mu, fold, pb0);
+                   SOAP_LAUNCHED(c));
+    }
     return SOAP_OK;
 }
 
