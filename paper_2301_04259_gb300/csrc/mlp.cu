@@ -33,6 +33,8 @@
 // Waits are bounded as in tc_gemm.cuh.
 #include "mlp.cuh"
 
+#include <cfloat>
+
 using bf16 = __nv_bfloat16;
 
 namespace soap {
@@ -306,7 +308,8 @@ __device__ __forceinline__ void chain(const Weights& w, const TrainArgs* ta, con
         if constexpr (kTrain) {
             // L = sum_b sum_j w_j (y - t)^2 / B, dL/dy = 2 w_j (y - t) / B.  The products are exact
             // pairs of floats (the rounding error of a product by an FMA, of a sum by TwoSum): the
-            // loss to ~48 bits without FP64 arithmetic, which runs at 1/64 rate.
+            // loss to ~48 bits without FP64 arithmetic, which runs at 1/64 rate.  A warp whose squares or
+            // sums leave FP32's range takes them again in FP64.
             if (ok && qd < 3) {
                 float hi = 0.0f, lo = 0.0f;
                 const float* trow = ta->t + src * kOut;
@@ -331,6 +334,24 @@ __device__ __forceinline__ void chain(const Weights& w, const TrainArgs* ta, con
                     put_row(act + qd * kAtom, r, h, v);
                 }
                 double part = (double)hi + (double)lo;
+                const float size = fabsf(hi + lo);
+                if (__any_sync(0xffffffffu, !(size <= FLT_MAX) || (size > 0.0f && size < 0x1p-70f))) {
+                    part = 0.0;
+#pragma unroll 1
+                    for (int h = 0; h < 2; h++) {
+                        const int c = 64 * qd + 32 * h;
+                        if (c >= kOut) break;
+                        float v[32];
+                        tc::tmem_ld32(tbase + (uint32_t)c, v);
+#pragma unroll
+                        for (int i = 0; i < 32; i++) {
+                            const int j = c + i;
+                            if (j >= kOut) continue;
+                            const double res = v[i] + __ldg(bias + j) - __ldg(trow + j);
+                            part += (double)__ldg(ta->w_out + j) * res * res;
+                        }
+                    }
+                }
                 for (int o = 16; o > 0; o >>= 1) part += __shfl_down_sync(0xffffffffu, part, o);
                 if (lane == 0 && rank == 0) atomicAdd(ta->loss, part / ta->B);
             }
