@@ -3,21 +3,26 @@
 The fastest variant (phases per block, pixels per thread) depends on the shape of the
 problem: pixels per spectrum, velocity-kernel taps, mu bins, grid size and the GPU.  The first
 run on a shape calls soap_batch_autotune and stores the winner in a JSON table keyed by that
-shape; later runs read it back and set it with soap_batch_set_variant.
+shape and by what the variants are, so that a table written when an index meant another variant
+is not read; later runs read it back and set it with soap_batch_set_variant.
 """
 from __future__ import annotations
 
 import json
 import os
 from pathlib import Path
-from typing import Callable, Optional
+from typing import Callable, Optional, Sequence, Tuple
 
 DEFAULT_PATH = Path(os.environ.get("SOAP_TUNING_CACHE",
                                    Path.home() / ".cache" / "soap_gb300" / "batch_tuning.json"))
 
 
-def tuning_key(n_px: int, n_taps: int, n_mu: int, grid_n: int, device: str) -> str:
-    return f"{device}|npx={int(n_px)}|taps={int(n_taps)}|mu={int(n_mu)}|grid={int(grid_n)}"
+def tuning_key(n_px: int, n_taps: int, n_mu: int, grid_n: int, device: str,
+               variants: Sequence[Tuple[int, int]] = ()) -> str:
+    key = f"{device}|npx={int(n_px)}|taps={int(n_taps)}|mu={int(n_mu)}|grid={int(grid_n)}"
+    if variants:
+        key += "|variants=" + ",".join(f"{int(pb)}x{int(r)}" for pb, r in variants)
+    return key
 
 
 def load_table(path: Path) -> dict:
@@ -66,7 +71,8 @@ def tune_batch(ctx, star, items, regions, phases, out, path: Optional[Path] = No
 
     info = soap.soap_get_star_info(ctx)
     key = tuning_key(star.n_px, info.n_taps, len(star.mu_values), star.grid_n,
-                     torch.cuda.get_device_name(out.device))
+                     torch.cuda.get_device_name(out.device),
+                     [soap.soap_batch_variant_info(v) for v in range(soap.soap_batch_num_variants())])
     return choose_variant(
         key,
         lambda: soap.soap_batch_autotune(ctx, items, regions, phases, out, reps=reps),
