@@ -332,17 +332,14 @@ k_project_nonfinite(Args g) {
     }
 }
 
-// Status word of the context-free entry point.
-static __device__ unsigned int g_project_flags;
-
 soap_status project(const float* x, int64_t n, int64_t p, const float* mean, const float* basis, int k, float* coef,
                     cudaStream_t st) {
     int dev = 0, sms = 0;
     SOAP_CUDA(cudaGetDevice(&dev));
     SOAP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    CallStatus status(st);
     unsigned int* flags = nullptr;
-    SOAP_CUDA(cudaGetSymbolAddress((void**)&flags, g_project_flags));
-    SOAP_CUDA(cudaMemsetAsync(flags, 0, sizeof(unsigned int), st));
+    SOAP_TRY(status.begin(&flags));
     Args a{};
     a.x = x; a.mean = mean; a.basis = basis; a.coef = coef;
     a.n = n; a.p = p; a.k = k;
@@ -368,8 +365,7 @@ soap_status project(const float* x, int64_t n, int64_t p, const float* mean, con
     k_project_nonfinite<<<(unsigned)std::min<int64_t>((n * k + 255) / 256, 8 * sms), 256, 0, st>>>(a);
     SOAP_CUDA(cudaGetLastError());
     unsigned int h = 0;
-    SOAP_CUDA(cudaMemcpyAsync(&h, flags, sizeof(h), cudaMemcpyDeviceToHost, st));
-    SOAP_CUDA(cudaStreamSynchronize(st));
+    SOAP_TRY(status.finish(&h));
     if (h) { set_error("the projection kernel gave up waiting (status 0x%x)", h); return SOAP_ETIMEOUT; }
     return SOAP_OK;
 }

@@ -327,6 +327,24 @@ inline soap_status fit_dynamic_smem(Kernel kernel, size_t dynamic) {
     return SOAP_OK;
 }
 
+// A cleared device status word of one call of an entry point without a context, on the call's stream
+// (tc_gemm.cu).  Held until finish() has read it, or until the stream is idle on any other way out.
+class CallStatus {
+public:
+    explicit CallStatus(cudaStream_t st) : st_(st) {}
+    CallStatus(const CallStatus&) = delete;
+    CallStatus& operator=(const CallStatus&) = delete;
+    ~CallStatus();
+    soap_status begin(unsigned int** word);
+    soap_status finish(unsigned int* value);         // waits for the stream
+
+private:
+    cudaStream_t st_;
+    int index_ = -1;
+    unsigned int* word_ = nullptr;
+    bool done_ = false;
+};
+
 // PCA projection coef = (X - mean) basis^T on the tensor cores at FP32 accuracy (pca_tc.cu);
 // synchronises the stream
 namespace pca {

@@ -4,6 +4,7 @@
 #include <algorithm>
 #include <mutex>
 
+#include "status_words.cuh"
 #include "tc_gemm.cuh"
 
 namespace soap {
@@ -104,8 +105,38 @@ soap_status gemm_tn(const __nv_bfloat16* A, int64_t lda, const __nv_bfloat16* B,
 
 using namespace soap;
 
-// Status word of the context-free GEMM entry point.
-static __device__ unsigned int g_gemm_flags;
+namespace soap {
+
+// Status words of the entry points without a context, one per call in flight: so many calls at a time
+// on all threads.
+constexpr int kCallWords = 256;
+static __device__ unsigned int g_call_words[kCallWords];
+static StatusWords<kCallWords> g_call_status;
+
+soap_status CallStatus::begin(unsigned int** word) {
+    unsigned int* words = nullptr;
+    SOAP_CUDA(cudaGetSymbolAddress((void**)&words, g_call_words));
+    index_ = g_call_status.claim();
+    word_ = words + index_;
+    SOAP_CUDA(cudaMemsetAsync(word_, 0, sizeof(unsigned int), st_));
+    *word = word_;
+    return SOAP_OK;
+}
+
+soap_status CallStatus::finish(unsigned int* value) {
+    SOAP_CUDA(cudaMemcpyAsync(value, word_, sizeof(unsigned int), cudaMemcpyDeviceToHost, st_));
+    SOAP_CUDA(cudaStreamSynchronize(st_));
+    done_ = true;
+    return SOAP_OK;
+}
+
+CallStatus::~CallStatus() {
+    if (index_ < 0) return;
+    if (!done_) cudaStreamSynchronize(st_);          // its kernels may still write the word
+    g_call_status.give_back(index_);
+}
+
+}  // namespace soap
 
 extern "C" soap_status soap_gemm_bf16_tn(int32_t M, int32_t N, int32_t K, const void* A, int64_t lda,
                                          const void* B, int64_t ldb, const float* bias, int32_t activation,
@@ -115,9 +146,9 @@ extern "C" soap_status soap_gemm_bf16_tn(int32_t M, int32_t N, int32_t K, const 
     if (activation != 0 && activation != 1) { set_error("activation must be 0 (none) or 1 (GELU)"); return SOAP_EINVAL; }
     if (ldc < N) { set_error("ldc < N"); return SOAP_EINVAL; }
     cudaStream_t st = (cudaStream_t)cuda_stream;
+    CallStatus status(st);
     unsigned int* flags = nullptr;
-    SOAP_CUDA(cudaGetSymbolAddress((void**)&flags, g_gemm_flags));
-    SOAP_CUDA(cudaMemsetAsync(flags, 0, sizeof(unsigned int), st));
+    SOAP_TRY(status.begin(&flags));
     tc::Epilogue ep{};
     ep.bias = bias;
     ep.gelu = activation;
@@ -125,8 +156,7 @@ extern "C" soap_status soap_gemm_bf16_tn(int32_t M, int32_t N, int32_t K, const 
     ep.ldc = ldc;
     SOAP_TRY(tc::gemm_tn((const __nv_bfloat16*)A, lda, (const __nv_bfloat16*)B, ldb, M, N, K, ep, st, flags));
     unsigned int h = 0;
-    SOAP_CUDA(cudaMemcpyAsync(&h, flags, sizeof(h), cudaMemcpyDeviceToHost, st));
-    SOAP_CUDA(cudaStreamSynchronize(st));
+    SOAP_TRY(status.finish(&h));
     if (h) { set_error("GEMM kernel gave up waiting (status 0x%x)", h); return SOAP_ETIMEOUT; }
     return SOAP_OK;
 }
