@@ -174,23 +174,23 @@ k_contract_fold32(int64_t n_px, Rows<float> rows, const TapGroup* __restrict__ g
 
 // FP64 (and the quiet star).  One block: pixel tile blockIdx.x of phase block blockIdx.y, effect
 // blockIdx.z; four blocks per SM: the pipe needs few warps and its accumulators many registers.
-template <typename T, int PB, int R, int THREADS>
+template <int PB, int R, int THREADS>
 __global__ void __launch_bounds__(THREADS, 4)
-k_contract(int64_t n_px, Rows<T> rows, const long long* __restrict__ toff, const int* __restrict__ gstart,
-           int G, int max_taps, const T* __restrict__ coefs, ClassTypes ctype, const T* __restrict__ contrast,
-           const T* __restrict__ fq, int n_phases, EffectList effs, T* __restrict__ out,
+k_contract(int64_t n_px, Rows<double> rows, const long long* __restrict__ toff, const int* __restrict__ gstart,
+           int G, int max_taps, const double* __restrict__ coefs, ClassTypes ctype, const double* __restrict__ contrast,
+           const double* __restrict__ fq, int n_phases, EffectList effs, double* __restrict__ out,
            const int* __restrict__ bstart, int n_mu, int fold, int pb0) {
     // a kernel launched after this one with an early start (the tensor-core CCF) may begin once
     // every CTA here has started: it waits for this grid before it reads the output
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int pb = pb0 + (int)blockIdx.y;
     const int np = min(PB, n_phases - pb * PB);
-    T* out_rows = out + (int64_t)blockIdx.z * n_phases * n_px + (int64_t)pb * PB * n_px;
-    const TableContrast<T> con{contrast, n_px, ctype};
+    double* out_rows = out + (int64_t)blockIdx.z * n_phases * n_px + (int64_t)pb * PB * n_px;
+    const TableContrast<double> con{contrast, n_px, ctype};
     if (fold) {
         const long long* tt = toff + (int64_t)pb * max_taps;
         const int* gs = gstart + (int64_t)pb * (G + 1);
-        const T* cb = coefs + (int64_t)pb * max_taps * PB;
+        const double* cb = coefs + (int64_t)pb * max_taps * PB;
         const int eff = effs.e[blockIdx.z];
         if (eff == SOAP_EFFECT_FLUX)
             contract_tile_fold64<PB, R, THREADS, SOAP_EFFECT_FLUX>(n_px, rows, tt, gs, G, cb, con, fq, blockIdx.x, np,
@@ -203,9 +203,9 @@ k_contract(int64_t n_px, Rows<T> rows, const long long* __restrict__ toff, const
                                                                   out_rows);
         return;
     }
-    contract_tile<T, PB, R, THREADS>(n_px, rows, toff + (int64_t)pb * max_taps, gstart + (int64_t)pb * (G + 1), G,
-                                     coefs + (int64_t)pb * max_taps * PB, con, fq, effs.e[blockIdx.z], blockIdx.x,
-                                     np, out_rows, bstart ? bstart + (int64_t)pb * (G * n_mu + 1) : nullptr, n_mu);
+    contract_tile<PB, R, THREADS>(n_px, rows, toff + (int64_t)pb * max_taps, gstart + (int64_t)pb * (G + 1), G,
+                                  coefs + (int64_t)pb * max_taps * PB, con, fq, effs.e[blockIdx.z], blockIdx.x,
+                                  np, out_rows, bstart ? bstart + (int64_t)pb * (G * n_mu + 1) : nullptr, n_mu);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -216,21 +216,21 @@ static int grid_cap(int64_t n, int threads, int cap) {
     return (int)(g < 1 ? 1 : (g > cap ? cap : g));
 }
 
-template <typename T, int PB, int R, int THREADS>
+template <int PB, int R, int THREADS>
 static soap_status launch_contract(soap_ctx* c, int n_blocks, int G, int max_taps,
-                                   const long long* toff, const int* gstart, const T* coefs,
-                                   const ClassTypes& ct, const T* contrast, const T* fq,
-                                   int n_phases, const EffectList& el, int n_eff, T* out,
-                                   const T* q, const T* a0, const T* a1, const int* bstart = nullptr,
+                                   const long long* toff, const int* gstart, const double* coefs,
+                                   const ClassTypes& ct, const double* contrast, const double* fq,
+                                   int n_phases, const EffectList& el, int n_eff, double* out,
+                                   const double* q, const double* a0, const double* a1, const int* bstart = nullptr,
                                    int fold = 0) {
-    Rows<T> rows;
+    Rows<double> rows;
     rows.q = q; rows.a[0] = a0; rows.a[1] = a1;
     int64_t tiles = (c->n_px + (int64_t)THREADS * R - 1) / ((int64_t)THREADS * R);
     // at most 65,535 phase blocks a launch, a grid's limit in y
     for (int pb0 = 0; pb0 < n_blocks; pb0 += 65535) {
         dim3 grid((unsigned)tiles, (unsigned)std::min(n_blocks - pb0, 65535), (unsigned)n_eff);
         SOAP_TIMED(c, fq ? SOAP_TIMER_CONTRACT : SOAP_TIMER_CONTRACT_QUIET,
-                   k_contract<T, PB, R, THREADS><<<grid, THREADS, 0, c->stream>>>(
+                   k_contract<PB, R, THREADS><<<grid, THREADS, 0, c->stream>>>(
                        c->n_px, rows, toff, gstart, G, max_taps, coefs, ct, contrast, fq, n_phases, el, out,
                        bstart, c->n_mu, fold, pb0);
                    SOAP_LAUNCHED(c));
@@ -255,9 +255,9 @@ static soap_status launch_contract(soap_ctx* c, int n_blocks, int G, int max_tap
 constexpr int kPB64 = SOAP_PB64, kR64 = SOAP_R64, kT64 = 128;
 constexpr int kPB32 = SOAP_PB32, kR32 = SOAP_R32, kT32 = 512 / SOAP_R32;
 
-// tap-table + coefficient scratch for a kernel set kfix with n_phases "phases" in blocks of PB
+// FP64 tap-table + coefficient scratch for a kernel set kfix with n_phases "phases" in blocks of PB
 static soap_status tap_buffers(soap_ctx* c, int n_phases, int n_class, int PB, int mode, long long** toff,
-                               int** gstart, double** c64, float** c32, int* n_blocks, int* G, int* max_taps,
+                               int** gstart, double** c64, int* n_blocks, int* G, int* max_taps,
                                int** bstart = nullptr) {
     *G = mode == 0 ? 1 : (mode == 1 ? 1 + n_class : n_class);
     *n_blocks = (n_phases + PB - 1) / PB;
@@ -269,13 +269,10 @@ static soap_status tap_buffers(soap_ctx* c, int n_phases, int n_class, int PB, i
     size_t bb = bstart ? (size_t)*n_blocks * (*G * c->n_mu + 1) * sizeof(int) : 0;
     SOAP_TRY(ensure(c->jobs, off_b + bb));
     if (bstart) *bstart = (int*)(c->jobs.as<char>() + off_b);
-    size_t cb64 = (size_t)*n_blocks * *max_taps * PB * sizeof(double);
-    size_t off32 = (cb64 + 255) / 256 * 256;
-    SOAP_TRY(ensure(c->coefs, off32 + (size_t)*n_blocks * *max_taps * PB * sizeof(float)));
+    SOAP_TRY(ensure(c->coefs, (size_t)*n_blocks * *max_taps * PB * sizeof(double)));
     *toff = c->jobs.as<long long>();
     *gstart = (int*)(c->jobs.as<char>() + off_g);
     *c64 = c->coefs.as<double>();
-    *c32 = (float*)(c->coefs.as<char>() + off32);
     return SOAP_OK;
 }
 
@@ -338,8 +335,8 @@ soap_status toeplitz_quiet(soap_ctx* c, int precision, void* dst) {
     ClassTypes ct{};
     EffectList el{{SOAP_EFFECT_TOT, 0, 0}};
     if (precision == SOAP_FP64)
-        return launch_contract<double, 1, 1, 128>(c, nbk, G, mt, c->qtoff, c->qgstart, c->qc64, ct, nullptr,
-                                                 nullptr, 1, el, 1, (double*)dst, c->q64, nullptr, nullptr);
+        return launch_contract<1, 1, 128>(c, nbk, G, mt, c->qtoff, c->qgstart, c->qc64, ct, nullptr, nullptr, 1, el, 1,
+                                          (double*)dst, c->q64, nullptr, nullptr);
     const unsigned blocks = (unsigned)((c->n_px + 4 * 128 - 1) / (4 * 128));
     SOAP_TIMED(c, SOAP_TIMER_CONTRACT_QUIET,
                k_quiet_groups<<<blocks, 128, 0, c->stream>>>(c->n_px, c->q32, c->qgrp, c->qgrp_start, c->qc32,
@@ -455,7 +452,7 @@ soap_status toeplitz_active(soap_ctx* c, const RegionDev* regions_host, int n_re
     const int n_sub = per_bin ? c->n_mu : 1;
     const int gstride = f64 ? 0 : fold_groups(ncl, c->n_mu, c->n_taps);
     if (f64) {
-        SOAP_TRY(tap_buffers(c, n_phases, ncl, PB, tmode, &toff, &gstart, &c64, &c32, &nbk, &G, &mt,
+        SOAP_TRY(tap_buffers(c, n_phases, ncl, PB, tmode, &toff, &gstart, &c64, &nbk, &G, &mt,
                              per_bin ? &bstart : nullptr));
     } else {
         const size_t g_bytes = ((size_t)nbk * gstride * sizeof(TapGroup) + 255) / 256 * 256;
@@ -527,9 +524,9 @@ soap_status toeplitz_active(soap_ctx* c, const RegionDev* regions_host, int n_re
         return toeplitz_tc(c, kfix, n_phases, ncl, class_type, a32s, a32f, con32, per_bin, el.e, n_eff, (float*)dst);
     }
     if (f64)
-        return launch_contract<double, kPB64, kR64, kT64>(c, nbk, G, mt, toff, gstart, c64, ct, con64,
-                                                         c->fq.as<double>(), n_phases, el, n_eff,
-                                                         (double*)dst, c->q64, a64s, a64f, bstart, tmode == 2);
+        return launch_contract<kPB64, kR64, kT64>(c, nbk, G, mt, toff, gstart, c64, ct, con64, c->fq.as<double>(),
+                                                  n_phases, el, n_eff, (double*)dst, c->q64, a64s, a64f, bstart,
+                                                  tmode == 2);
     Rows<float> rows;
     rows.q = c->q32; rows.a[0] = a32s; rows.a[1] = a32f;
     const dim3 grid((unsigned)((c->n_px + kT32 * kR32 - 1) / (kT32 * kR32)), (unsigned)nbk, (unsigned)n_eff);

@@ -1,7 +1,8 @@
 // contract_dev.cuh -- device code of the Toeplitz contraction shared by the single-star
 // kernels (contract.cu) and the batched persistent kernel (batch.cu).
 //
-// contract_tile() (FP64; FP32 takes contract_tile_fold32) computes one pixel tile of PB phases:
+// contract_tile() (the FP64 quiet star, and FP64 contrasts with a row per mu bin; else
+// contract_tile_fold64 and contract_tile_fold32) computes one pixel tile of PB phases:
 //   out[p][m] = F_q[m] - sum_b Q_p,b * S_q,b [m] + sum_cl C_cl[m] sum_b K_p,cl,b * S_a(cl),b [m]
 // (Eqs. 1-4 for the effect `eff`), from a tap table (group starts, per-tap row offsets,
 // coefficients [tap][PB]).  One thread owns R pixels m = m0 + threadIdx.x + r*THREADS; acc
@@ -28,9 +29,9 @@ struct EffectList {
 
 // PB coefficients of one tap (16-byte vector loads when PB allows; coefficient slabs are
 // 256-byte aligned and every job's block is a multiple of PB elements).
-template <typename T, int PB>
-__device__ __forceinline__ void load_coefs(const T* __restrict__ src, T (&cv)[PB]) {
-    if constexpr (sizeof(T) == 8 && PB % 2 == 0) {
+template <int PB>
+__device__ __forceinline__ void load_coefs(const double* __restrict__ src, double (&cv)[PB]) {
+    if constexpr (PB % 2 == 0) {
 #pragma unroll
         for (int q = 0; q < PB / 2; q++) {
             const double2 t = __ldg(reinterpret_cast<const double2*>(src) + q);
@@ -98,15 +99,14 @@ struct PlanckContrast32 {
     }
 };
 
-// bs (optional): per-(group, mu bin) tap starts [G n_mu + 1]; with it each class is folded
-// per bin, acc += C_(cl n_mu + b)[m] . sum_(taps of bin b) (a contrast row per class and bin:
+// bs: per-(group, mu bin) tap starts [G n_mu + 1] (not for the quiet group alone, G = 1): each class is
+// folded per bin, acc += C_(cl n_mu + b)[m] . sum_(taps of bin b) (a contrast row per class and bin:
 // mu-dependent facula temperatures).
-template <typename T, int PB, int R, int THREADS, class Con>
-__device__ __forceinline__ void contract_tile(int64_t n_px, const Rows<T>& rows, const long long* __restrict__ toff,
-                                              const int* __restrict__ gs, int G, const T* __restrict__ cb,
-                                              const Con& con, const T* __restrict__ fq, int eff, int64_t tile,
-                                              int np, T* __restrict__ out_rows, const int* __restrict__ bs = nullptr,
-                                              int n_mu = 0) {
+template <int PB, int R, int THREADS, class Con>
+__device__ __forceinline__ void contract_tile(int64_t n_px, const Rows<double>& rows, const long long* __restrict__ toff,
+                                              const int* __restrict__ gs, int G, const double* __restrict__ cb,
+                                              const Con& con, const double* __restrict__ fq, int eff, int64_t tile,
+                                              int np, double* __restrict__ out_rows, const int* __restrict__ bs, int n_mu) {
     // Rows are padded past round_up(n_px, 1024) + max tap, so every tap of every pixel of the
     // last tile reads inside its row; only the per-pixel inputs below need a clamped index.
     const int64_t m0 = tile * THREADS * R + threadIdx.x;
@@ -118,23 +118,23 @@ __device__ __forceinline__ void contract_tile(int64_t n_px, const Rows<T>& rows,
     }
     // The tap sums accumulate from zero and F_q is added once at the store: every FMA then
     // rounds at the scale of the residual, not of the continuum (about 8x finer in FP32).
-    T acc[PB][R];
+    double acc[PB][R];
 #pragma unroll
     for (int r = 0; r < R; r++)
 #pragma unroll
-        for (int p = 0; p < PB; p++) acc[p][r] = T(0);
+        for (int p = 0; p < PB; p++) acc[p][r] = 0.0;
     // group 0: subtract (active star) or add (quiet star) the quiet-row convolutions
     {
-        const T* base = rows.q + m0;
+        const double* base = rows.q + m0;
         const int t1 = gs[1];
 #pragma unroll 4
         for (int t = gs[0]; t < t1; t++) {
-            const T* row = base + __ldg(toff + t);
-            T s[R];
+            const double* row = base + __ldg(toff + t);
+            double s[R];
 #pragma unroll
             for (int r = 0; r < R; r++) s[r] = __ldg(row + r * THREADS);
-            T cv[PB];
-            load_coefs<T, PB>(cb + (int64_t)t * PB, cv);
+            double cv[PB];
+            load_coefs<PB>(cb + (int64_t)t * PB, cv);
 #pragma unroll
             for (int p = 0; p < PB; p++)
 #pragma unroll
@@ -142,70 +142,36 @@ __device__ __forceinline__ void contract_tile(int64_t n_px, const Rows<T>& rows,
         }
     }
     // classes with a contrast row per mu bin: fold each bin's sum separately
-    if (bs) {
-        for (int g = 1; g < G; g++) {
-            if (gs[g] == gs[g + 1]) continue;
-            const int cl = g - 1;
-            const T* base = (eff == SOAP_EFFECT_FLUX ? rows.q : rows.a[con.type(cl) == SOAP_FACULA ? 1 : 0]) + m0;
-            for (int b = 0; b < n_mu; b++) {
-                const int t0 = bs[g * n_mu + b], t1 = bs[g * n_mu + b + 1];
-                if (t0 == t1) continue;
-                T tmp[PB][R];
-#pragma unroll
-                for (int p = 0; p < PB; p++)
-#pragma unroll
-                    for (int r = 0; r < R; r++) tmp[p][r] = T(0);
-                for (int t = t0; t < t1; t++) {
-                    const T* row = base + __ldg(toff + t);
-                    T s[R];
-#pragma unroll
-                    for (int r = 0; r < R; r++) s[r] = __ldg(row + r * THREADS);
-                    T cv[PB];
-                    load_coefs<T, PB>(cb + (int64_t)t * PB, cv);
-#pragma unroll
-                    for (int p = 0; p < PB; p++)
-#pragma unroll
-                        for (int r = 0; r < R; r++) tmp[p][r] = fma(cv[p], s[r], tmp[p][r]);
-                }
-#pragma unroll
-                for (int r = 0; r < R; r++) {
-                    const T cr = eff == SOAP_EFFECT_BCONV ? T(1) : con.at(cl * n_mu + b, mcl[r]);
-#pragma unroll
-                    for (int p = 0; p < PB; p++) acc[p][r] = fma(cr, tmp[p][r], acc[p][r]);
-                }
-            }
-        }
-        G = 1;                                             // classes done
-    }
-    // classes: tmp = sum_b K_cl,b * S, then acc += C_cl . tmp (TOT, FLUX) or tmp (BCONV)
     for (int g = 1; g < G; g++) {
-        const int t0 = gs[g], t1 = gs[g + 1];
-        if (t0 == t1) continue;
+        if (gs[g] == gs[g + 1]) continue;
         const int cl = g - 1;
-        const T* base = (eff == SOAP_EFFECT_FLUX ? rows.q : rows.a[con.type(cl) == SOAP_FACULA ? 1 : 0]) + m0;
-        T tmp[PB][R];
-#pragma unroll
-        for (int p = 0; p < PB; p++)
-#pragma unroll
-            for (int r = 0; r < R; r++) tmp[p][r] = T(0);
-#pragma unroll 4
-        for (int t = t0; t < t1; t++) {
-            const T* row = base + __ldg(toff + t);
-            T s[R];
-#pragma unroll
-            for (int r = 0; r < R; r++) s[r] = __ldg(row + r * THREADS);
-            T cv[PB];
-            load_coefs<T, PB>(cb + (int64_t)t * PB, cv);
+        const double* base = (eff == SOAP_EFFECT_FLUX ? rows.q : rows.a[con.type(cl) == SOAP_FACULA ? 1 : 0]) + m0;
+        for (int b = 0; b < n_mu; b++) {
+            const int t0 = bs[g * n_mu + b], t1 = bs[g * n_mu + b + 1];
+            if (t0 == t1) continue;
+            double tmp[PB][R];
 #pragma unroll
             for (int p = 0; p < PB; p++)
 #pragma unroll
-                for (int r = 0; r < R; r++) tmp[p][r] = fma(cv[p], s[r], tmp[p][r]);
-        }
+                for (int r = 0; r < R; r++) tmp[p][r] = 0.0;
+            for (int t = t0; t < t1; t++) {
+                const double* row = base + __ldg(toff + t);
+                double s[R];
 #pragma unroll
-        for (int r = 0; r < R; r++) {
-            const T cr = eff == SOAP_EFFECT_BCONV ? T(1) : con.at(cl, mcl[r]);
+                for (int r = 0; r < R; r++) s[r] = __ldg(row + r * THREADS);
+                double cv[PB];
+                load_coefs<PB>(cb + (int64_t)t * PB, cv);
 #pragma unroll
-            for (int p = 0; p < PB; p++) acc[p][r] = fma(cr, tmp[p][r], acc[p][r]);
+                for (int p = 0; p < PB; p++)
+#pragma unroll
+                    for (int r = 0; r < R; r++) tmp[p][r] = fma(cv[p], s[r], tmp[p][r]);
+            }
+#pragma unroll
+            for (int r = 0; r < R; r++) {
+                const double cr = eff == SOAP_EFFECT_BCONV ? 1.0 : con.at(cl * n_mu + b, mcl[r]);
+#pragma unroll
+                for (int p = 0; p < PB; p++) acc[p][r] = fma(cr, tmp[p][r], acc[p][r]);
+            }
         }
     }
     // store out_rows[p][m]
@@ -219,7 +185,6 @@ __device__ __forceinline__ void contract_tile(int64_t n_px, const Rows<T>& rows,
         }
     }
 }
-
 
 // Folded form for tap tables without the quiet group (builder mode 2: group g = class g): the
 // quiet rows enter each class's operand, X_cl[m - k] = Ca_cl[m] S_a(cl)[m - k] + Cq_cl[m] S_q[m - k]
@@ -267,7 +232,7 @@ __device__ __forceinline__ void contract_tile_fold64(int64_t n_px, const Rows<do
         for (int t = t0; t < t1; t++) {
             const long long off = __ldg(toff + t);
             double cv[PB];
-            load_coefs<double, PB>(cb + (int64_t)t * PB, cv);
+            load_coefs<PB>(cb + (int64_t)t * PB, cv);
             double x[R];
 #pragma unroll
             for (int r = 0; r < R; r++) {

@@ -543,7 +543,8 @@ __device__ __forceinline__ float fixed_to_float(long long K, int bits) {
 //   gstart[G+1]   first tap of each group (group 0: quiet rows; group g >= 1: class g-1)
 //   toff[tap]     element offset bin * row_len + pad - k: the row value S_b[m - k] of pixel m
 //                 is rows[toff + m]
-//   coef[tap][PB] kernel value of each phase of the block (0 where a phase has none)
+//   coef[tap][PB] kernel value of each phase of the block (0 where a phase has none; c64 and c32, each
+//                 may be null)
 // kfix: [n_phases][n_class][n_mu][n_taps] in units of 2^-fx_bits (inv_scale = 2^-fx_bits).
 // mode 0 (quiet): one group, +K of class 0.  mode 1 (active): group 0 = -sum_cl K (quiet rows),
 // group g = +K of class g-1.  mode 2 (active, quiet rows folded into the classes' operands):
@@ -555,8 +556,8 @@ __device__ __forceinline__ float fixed_to_float(long long K, int bits) {
 // consecutive shifts of one row, at offsets o_hi, o_hi - 1, .., o_lo; aligned group q holds those
 // of them in 4q .. 4q + 3 (TapGroup: off4 = 4q, the tap index of offset 4q, a bit per present
 // offset; groups listed from the highest q down, like the taps), so that a contraction can read the
-// row values of four consecutive pixels for all of a group's taps as two aligned 16-byte vectors.  agstart[g] is the first aligned group of
-// group g (G + 1 entries, last = total); block pb's groups start at agrp + pb * max_groups with
+// row values of four consecutive pixels for all of a group's taps as two aligned 16-byte vectors.
+// agstart[g] is the first aligned group of group g (G + 1 entries, last = total); block pb's groups start at agrp + pb * max_groups with
 // max_groups = max_taps + G n_mu (a (group, bin) with nk taps has at most nk + 1 groups).
 // grp_stride > 0: aligned groups of eight offsets 8q .. 8q + 7 instead of all the above (toff, gstart
 // and c64 are not written and may be null).  Block pb's groups start at agrp + pb * grp_stride, their
@@ -781,7 +782,7 @@ __device__ __forceinline__ void build_taps_dev(const long long* __restrict__ kfi
             const int kk = e / PB, pl = e % PB;
             const long long K = value(g, b, pl, s_lo[t] + kk);
             if (c64) c64[tap0 * PB + e] = (double)K * inv_scale;
-            c32[tap0 * PB + e] = fixed_to_float(K, fx_bits);
+            if (c32) c32[tap0 * PB + e] = fixed_to_float(K, fx_bits);
         }
     }
 }

@@ -181,8 +181,7 @@ struct Smem {
 // Row-major store of a warp's 32 x 32 block through its shared tile: lane r holds row r's 32
 // values; after the transpose, lane j writes column j of each row in turn, so every store
 // instruction covers 32 consecutive elements of one row.
-template <typename T>
-__device__ __forceinline__ void store_rows(float (*tile)[33], const float (&v)[32], int lane, T* base, int64_t ld,
+__device__ __forceinline__ void store_rows(float (*tile)[33], const float (&v)[32], int lane, float* base, int64_t ld,
                                            int m_first, int M, int n_first, int N) {
 #pragma unroll
     for (int i = 0; i < 32; i++) tile[lane][i] = v[i];
@@ -193,9 +192,7 @@ __device__ __forceinline__ void store_rows(float (*tile)[33], const float (&v)[3
         for (int r = 0; r < 32; r++) {
             const int m = m_first + r;
             if (m >= M) break;
-            const float x = tile[r][lane];
-            if constexpr (sizeof(T) == 4) base[(int64_t)m * ld + n] = x;
-            else base[(int64_t)m * ld + n] = __float2bfloat16_rn(x);
+            base[(int64_t)m * ld + n] = tile[r][lane];
         }
     }
     __syncwarp();
