@@ -399,7 +399,8 @@ enum {
  *  out        float32 [n_phases][n_px], row p for phase p, host or device per out_on_device.
  * Arithmetic as SOAP_FP32 (FP64 velocities and shift positions, FP32 contraction and
  * accumulation); a cell's interpolation weight is held to 32 fractional bits; the contrast
- * (Sect. 4.3.1) is evaluated per pixel in FP32.  Needs diff_rot_alpha = 0 (a cell's velocity is
+ * (Sect. 4.3.1) is evaluated in FP32, per pixel or, where its curvature allows (|error| below 2^-26
+ * of it, for the grids and temperatures in use), by a line over every eight pixels.  Needs diff_rot_alpha = 0 (a cell's velocity is
  * then vsini x, so one table per item and grid column replaces per-cell geometry) and at most
  * SOAP_MAX_CLASSES distinct (type, temperature) pairs within each item.  Work is cut into
  * phase blocks run by one persistent kernel in decreasing order of estimated cost; the kernel

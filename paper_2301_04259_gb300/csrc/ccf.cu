@@ -1492,8 +1492,11 @@ soap_status ccf_enqueue(soap_ctx* c, CcfState& st, const CcfPlan& p, const void*
     if ((p.windowed || p.tile_np || p.tc_chunk) && p.f32) {  // FP32 partial sums (converted exactly to FP64 here)
         cudaLaunchAttribute attr[1];
         const int64_t outputs = (int64_t)n_spec * n_v;
+        int dev = 0, sms = 0;
+        SOAP_CUDA(cudaGetDevice(&dev));
+        SOAP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
         // a thread per output while the chunks fit its registers and the outputs fill the GPU
-        if (p.n_chunks <= kReduceFew && outputs >= 152 * 2048) {
+        if (p.n_chunks <= kReduceFew && outputs >= (int64_t)sms * 2048) {
             const cudaLaunchConfig_t cfg = pdl_config(dim3((unsigned)((outputs + 255) / 256)), dim3(256), c->stream, early, attr);
             SOAP_CUDA(cudaLaunchKernelEx(&cfg, k_ccf_reduce_few, p.n_chunks, outputs,
                                          reinterpret_cast<const float*>(d_part), d_ccf));

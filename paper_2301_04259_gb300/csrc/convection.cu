@@ -245,7 +245,10 @@ soap_status inject_bisectors(soap_ctx* c, const double* in, double* out, int n_r
         SOAP_TRY(upload_small(c, c->bis_tab.p, lin.data(), lin.size() * sizeof(double)));
         const unsigned tiles = (unsigned)((c->n_px + kBisThreads - 1) / kBisThreads);
         // the per-thread conversions serve a few rows, while the blocks still fill the GPU
-        const int per = std::max(1, std::min(4, (int)((int64_t)tiles * n_rows / (152 * 32))));
+        int dev = 0, sms = 0;
+        SOAP_CUDA(cudaGetDevice(&dev));
+        SOAP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+        const int per = std::max(1, std::min(4, (int)((int64_t)tiles * n_rows / (sms * 32))));
         const dim3 grid(tiles, (unsigned)std::min(65535, (n_rows + per - 1) / per));
         SOAP_TIMED(c, SOAP_TIMER_BISECTORS,
                    (k_bisectors_small<<<grid, kBisThreads, 0, c->stream>>>(

@@ -306,10 +306,10 @@ __device__ __forceinline__ void chain(const Weights& w, const TrainArgs* ta, con
         }
         const float* bias = w.bias[kFwd - 1];
         if constexpr (kTrain) {
-            // L = sum_b sum_j w_j (y - t)^2 / B, dL/dy = 2 w_j (y - t) / B.  The products are exact
-            // pairs of floats (the rounding error of a product by an FMA, of a sum by TwoSum): the
-            // loss to ~48 bits without FP64 arithmetic, which runs at 1/64 rate.  A warp whose squares or
-            // sums leave FP32's range takes them again in FP64.
+            // L = sum_b sum_j w_j (y - t)^2 / B, dL/dy = 2 w_j (y - t) / B.  A thread's part of L, which is
+            // reported and enters no gradient, is a pair of floats (the rounding error of a product by an
+            // FMA, of a sum by TwoSum): ~48 bits, five fewer than FP64's, without FP64 arithmetic, which
+            // runs at 1/64 rate.  A warp whose squares or sums leave FP32's range takes them in FP64.
             if (ok && qd < 3) {
                 float hi = 0.0f, lo = 0.0f;
                 const float* trow = ta->t + src * kOut;

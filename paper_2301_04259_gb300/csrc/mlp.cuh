@@ -11,7 +11,7 @@ constexpr int kIn = 8, kHidden = 256, kCoef = 128, kOut = kCoef + 1, kOutPad = 1
 constexpr int kFwd = 5;                      // forward products
 constexpr int kBwd = 4;                      // products of the backward chain (dz)
 
-// BF16 weights of one network as TMA maps (boxes of 64 K columns x 256 rows, 128-byte swizzle):
+// BF16 weights of one network as TMA maps (boxes of 64 K columns x 128 rows, 128-byte swizzle):
 // W_l [out][in] for the forward products, W_l^T [in][out_pad] of layers 4 .. 1 for the backward.
 struct Weights {
     CUtensorMap fwd[kFwd];

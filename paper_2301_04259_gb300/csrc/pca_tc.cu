@@ -17,7 +17,7 @@
 // mean, split and store both operands as 128-byte-swizzled K-major tiles.  Four more warps: a lane
 // of the first issues the MMAs, all four drain the accumulators.  The running sums live in tensor
 // memory: in registers (of the splitters or of warps of their own) they made the splitters' prefetch
-// spill, and a spilled value waits for its load (763 us as below with 20 bytes spilled, 1,110 with 260).
+// spill, and a spilled value waits for its load (the call below 763 us with 20 bytes spilled, 1,110 with 260).
 // 20,011 x 16,834 x 128: 0.57 ms a call (2.4 TB/s of X), against 5.5 ms as an FP32 SIMT product of
 // 64 x 64 tiles and a product of one row (the mean) on two SMs; without the loads it takes 0.45, and
 // without the MMAs 0.47: splitting (about eleven instructions per pixel pair and operand) and the
