@@ -1210,7 +1210,7 @@ constexpr int kFwWholeBlockMax = 2 * 152;
 
 // early: programmatic dependent launch (the kernel before it releases it; it waits for that
 // kernel before it reads anything)
-static cudaLaunchConfig_t pdl_config(dim3 grid, dim3 block, cudaStream_t st, bool early, cudaLaunchAttribute* attr) {
+cudaLaunchConfig_t pdl_config(dim3 grid, dim3 block, cudaStream_t st, bool early, cudaLaunchAttribute* attr) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid;
     cfg.blockDim = block;
@@ -1487,7 +1487,8 @@ soap_status ccf_enqueue(soap_ctx* c, CcfState& st, const CcfPlan& p, const void*
     tb = c->profiling ? timer_begin(c) : nullptr;
     const unsigned rblocks = (unsigned)(((int64_t)n_spec * n_v + 31) / 32);
     // after the tensor-core CCF (which releases its dependents as it starts) the reduction and the
-    // fit are launched early, so that their launches overlap the kernel before them
+    // fit are launched early, so that their launches overlap the kernel before them; so is the
+    // reduction behind the FP64 running sums
     const bool early = p.tc_chunk != 0;
     if ((p.windowed || p.tile_np || p.tc_chunk) && p.f32) {  // FP32 partial sums (converted exactly to FP64 here)
         cudaLaunchAttribute attr[1];
@@ -1505,9 +1506,12 @@ soap_status ccf_enqueue(soap_ctx* c, CcfState& st, const CcfPlan& p, const void*
             SOAP_CUDA(cudaLaunchKernelEx(&cfg, k_ccf_reduce<float>, p.n_chunks, n_spec, n_v,
                                          reinterpret_cast<const float*>(d_part), d_ccf));
         }
-    } else
-        k_ccf_reduce<double><<<rblocks, dim3(32, kReduceSplit), 0, c->stream>>>(p.n_chunks, n_spec, n_v,
-                                                                                d_part, d_ccf);
+    } else {
+        cudaLaunchAttribute attr[1];
+        const cudaLaunchConfig_t cfg = pdl_config(dim3(rblocks), dim3(32, kReduceSplit), c->stream, p.ramp_L != 0, attr);
+        SOAP_CUDA(cudaLaunchKernelEx(&cfg, k_ccf_reduce<double>, p.n_chunks, n_spec, n_v,
+                                     static_cast<const double*>(d_part), d_ccf));
+    }
     SOAP_LAUNCHED(c);
     if (tb) timer_end(c, SOAP_TIMER_CCF_AUX, tb);
     if (p.f32)      // float32 spectra: FP32 fit, one warp per spectrum

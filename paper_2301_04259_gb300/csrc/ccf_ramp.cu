@@ -27,7 +27,7 @@
 // 0.5 ms, against 1.71 with the windowed kernel (two multiply-adds and ten more FP64 instructions per
 // line and velocity for eight spectra).
 // Values that the running sums do not give are added line by line by a kernel of their own (k_ramp_direct):
-// 5 us a call where there are none, 0.35 ms for a NaN in the same pixel of all those spectra, 1.3 ms when
+// launched early behind the sums, 0 to 3 us a call where there are none (5 without), 0.35 ms for a NaN in the same pixel of all those spectra, 1.3 ms when
 // none of the values can be taken.
 //
 // Precision (the sums of 1,170 lines against extended precision, root mean square of the relative error over
@@ -205,6 +205,8 @@ k_ccf_ramp(const __grid_constant__ RampArgs g, unsigned int* flags) {
         if (lane == 0) s_weights = sum;
     }
     __syncthreads();
+    // the kernel behind this one may be launched: it waits for this one's end
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     // last pieces, slots, one partial row per spectrum
     // (lane: velocity lane / 8 of four, spectrum lane mod 8)
     for (int k0 = 4 * warp; k0 < g.n_v; k0 += n_thr / 8) {
@@ -237,6 +239,9 @@ constexpr int kDirectWarps = 8;
 __global__ void __launch_bounds__(32 * kDirectWarps)
 k_ramp_direct(const __grid_constant__ RampArgs g) {
     __shared__ double part[kDirectWarps][kRampSpec][32];
+    // launched early behind k_ccf_ramp, as the reduction behind this one
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int k = 32 * blockIdx.z + lane, n_words = (g.n_v + 3) / 4;
     const unsigned int* word = g.bad + ((int64_t)blockIdx.x * gridDim.y + blockIdx.y) * n_words;
@@ -479,8 +484,10 @@ soap_status ccf_ramp(soap_ctx* c, const CcfState& st, const CcfPlan& p, const do
     const dim3 grid((unsigned)p.n_chunks, (unsigned)((p.n_spec + kRampSpec - 1) / kRampSpec));
     k_ccf_ramp<<<grid, 32 * std::max(r.groups, 4), smem, c->stream>>>(a, c->flags);
     SOAP_LAUNCHED(c);
-    k_ramp_direct<<<dim3(grid.x, grid.y, (unsigned)((p.n_v + 31) / 32)), 32 * kDirectWarps, 0, c->stream>>>(a);
-    SOAP_CUDA(cudaGetLastError());                     // (the caller counts the CCF kernel)
+    cudaLaunchAttribute attr[1];
+    const cudaLaunchConfig_t cfg = pdl_config(dim3(grid.x, grid.y, (unsigned)((p.n_v + 31) / 32)), dim3(32 * kDirectWarps),
+                                              c->stream, true, attr);
+    SOAP_CUDA(cudaLaunchKernelEx(&cfg, k_ramp_direct, a));     // (the caller counts it)
     return SOAP_OK;
 }
 

@@ -445,6 +445,8 @@ soap_status ccf_tc_build_m(soap_ctx* c, CcfState& st, const CcfPlan& p);
 // the FP64 CCF of boxes no wider than a pixel (ccf_ramp.cu)
 soap_status ccf_ramp_plan(soap_ctx* c, CcfState& st, const double* mask_lambda, CcfPlan& p, int sms);
 soap_status ccf_ramp_build(soap_ctx* c, CcfState& st, const CcfPlan& p);
+// launch with programmatic stream serialization where `early` (ccf.cu); attr outlives the launch
+cudaLaunchConfig_t pdl_config(dim3 grid, dim3 block, cudaStream_t st, bool early, cudaLaunchAttribute* attr);
 size_t ccf_ramp_scratch(const CcfPlan& p);
 soap_status ccf_ramp(soap_ctx* c, const CcfState& st, const CcfPlan& p, const double* spectra, double* partial);
 soap_status ccf_tc(soap_ctx* c, CcfState& st, const CcfPlan& p, const float* spectra, float* partial);
