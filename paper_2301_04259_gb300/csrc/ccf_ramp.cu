@@ -27,8 +27,8 @@
 // 0.5 ms, against 1.71 with the windowed kernel (two multiply-adds and ten more FP64 instructions per
 // line and velocity for eight spectra).
 // Values that the running sums do not give are added line by line by a kernel of their own (k_ramp_direct):
-// launched early behind the sums, 0 to 3 us a call where there are none (5 without), 0.35 ms for a NaN in the same pixel of all those spectra, 1.3 ms when
-// none of the values can be taken.
+// launched early behind the sums, 0 to 3 us a call where there are none (5 without), 0.35 ms for a NaN in the
+// same pixel of all those spectra, 1.3 ms when none of the values can be taken.
 //
 // Precision (the sums of 1,170 lines against extended precision, root mean square of the relative error over
 // velocities): 2.8e-16 for boxes of 0.94 pixels, 5.6e-16 for a quarter of a pixel, 2.0e-15 for a twentieth,
@@ -40,8 +40,6 @@
 #include <cmath>
 #include <cstring>
 #include <vector>
-
-#include <math_constants.h>
 
 #include "soap_internal.cuh"
 
@@ -100,7 +98,7 @@ struct RampArgs {
     const double* g;
     const double* spectra;
     double* partial;
-    unsigned int* bad;            // by (blocks of lines, of spectra), a byte of spectra for each velocity
+    unsigned int* bad;            // [blocks of lines][blocks of spectra]: spectra whose sums are not to be taken
     double box;
     int64_t n_px;
     int n_lines, L, units, per_block, groups, n_events, n_slots, o_min, n_v, n_spec, max_rows;
@@ -108,15 +106,12 @@ struct RampArgs {
 
 // A running sum also holds the pixels that a velocity's boxes only reach in other pieces, and pixels under
 // lines of weight zero; what they add cancels, exactly in exact arithmetic.  An infinity or a NaN does not
-// cancel, and a pixel far above the others leaves its rounding behind.  So a block's sum of one velocity
-// is only taken where it is not small against the largest pixel times the sum of |weights| (a sum of n
-// lines is some n w b F of at most n w F_max: ratios of 2 to 40 for spectra and boxes of a quarter of a pixel
-// and more); k_ramp_direct replaces the others.  (Boxes below about a hundredth of a pixel leave it all
-// of them: 2.1 ms for the RVs of 100 spectra of 205,800 pixels, 1.9 with the windowed kernel.)
-constexpr double kRampTrust = 256.0;
-
-// high word of |x|: ordered as |x| is, NaN above all
-__device__ __forceinline__ int abs_hi(double x) { return __double2hiint(x) & 0x7fffffff; }
+// cancel, and a pixel far above the others leaves its rounding behind.  So a block's sums of a spectrum
+// are only taken while its largest pixel is finite and within 2^kRampSpread of the geometric mean of its
+// pixels that are not zero (by their exponents: whole numbers, a few integer instructions a pixel;
+// spectra are within 2^4); k_ramp_direct replaces the others.  At the limit the largest pixel's rounding
+// is 2^10 2^-53 of a line's share of the sum, 1e-15 of it with the thousand lines of a block.
+constexpr int kRampSpread = 10;
 
 __global__ void __launch_bounds__(32 * kRampMaxGroups, 1)
 k_ccf_ramp(const __grid_constant__ RampArgs g, unsigned int* flags) {
@@ -126,15 +121,18 @@ k_ccf_ramp(const __grid_constant__ RampArgs g, unsigned int* flags) {
     double* tot = reinterpret_cast<double*>(lines + g.L);          // [groups][A, B][32]
     double* acc = tot + g.groups * 64;                             // [n_slots][8]
     unsigned char* win = reinterpret_cast<unsigned char*>(acc + g.n_slots * 8);
-    __shared__ int s_big[kRampSpec];                               // largest pixel of each spectrum
-    __shared__ double s_weights;                                   // sum of the lines' |weights|
+    // of each spectrum: high word of the largest |pixel| (as ordered; NaN above all), and the number and the
+    // exponents' sum of the pixels that are not zero
+    __shared__ int s_big[kRampSpec], s_count[kRampSpec];
+    __shared__ unsigned long long s_exp[kRampSpec];
     const int t = threadIdx.x, n_thr = blockDim.x, warp = t >> 5, lane = t & 31;
     const int q = lane >> 3, s8 = lane & 7;
     const int s0 = blockIdx.y * kRampSpec, ns = min(kRampSpec, g.n_spec - s0);
     for (int i = t; i < g.n_events; i += n_thr) ev[i] = g.events[i];
     for (int i = t; i < g.groups * 64 + g.n_slots * 8; i += n_thr) tot[i] = 0.0;
-    if (t < kRampSpec) s_big[t] = 0;
-    int big0 = 0, big1 = 0;                            // of the two spectra whose pixels this thread stages
+    if (t < kRampSpec) s_big[t] = s_count[t] = s_exp[t] = 0;
+    int big[2] = {0, 0}, count[2] = {0, 0};            // of the two spectra that this thread stages
+    unsigned long long expo[2] = {0, 0};
     const int e0 = warp < g.groups ? g.ev_start[warp] : 0;
     const int u1 = min(g.units, (int)(blockIdx.x + 1) * g.per_block);
     for (int u = blockIdx.x * g.per_block; u < u1; u++) {
@@ -160,8 +158,13 @@ k_ccf_ramp(const __grid_constant__ RampArgs g, unsigned int* flags) {
             const double v0 = on && 2 * part < ns ? __ldg(src) : 0.0;
             const double v1 = on && 2 * part + 1 < ns ? __ldg(src + g.n_px) : 0.0;
             *reinterpret_cast<double2*>(win + x * kRampRow + 16 * part) = make_double2(v0, v1);
-            big0 = max(big0, abs_hi(v0));
-            big1 = max(big1, abs_hi(v1));
+#pragma unroll
+            for (int h = 0; h < 2; h++) {
+                const int hi = __double2hiint(h ? v1 : v0) & 0x7fffffff;
+                big[h] = max(big[h], hi);
+                count[h] += hi >= 0x00100000;
+                expo[h] += (unsigned int)hi >> 20;
+            }
         }
         __syncthreads();
         if (warp < g.groups) {
@@ -195,19 +198,22 @@ k_ccf_ramp(const __grid_constant__ RampArgs g, unsigned int* flags) {
             tot[warp * 64 + 32 + lane] += B;
         }
     }
-    atomicMax(&s_big[2 * (t & 3)], big0);
-    atomicMax(&s_big[2 * (t & 3) + 1], big1);
-    const int b0 = min(g.n_lines, (int)blockIdx.x * g.per_block * g.L), b1 = min(g.n_lines, u1 * g.L);
-    if (warp == 0) {
-        double sum = 0.0;
-        for (int l = b0 + lane; l < b1; l += 32) sum += fabs(g.lines[l].w);
-        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-        if (lane == 0) s_weights = sum;
+#pragma unroll
+    for (int h = 0; h < 2; h++) {
+        atomicMax(&s_big[2 * (t & 3) + h], big[h]);
+        atomicAdd(&s_count[2 * (t & 3) + h], count[h]);
+        atomicAdd(&s_exp[2 * (t & 3) + h], expo[h]);
     }
     __syncthreads();
     // the kernel behind this one may be launched: it waits for this one's end
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     // last pieces, slots, one partial row per spectrum
+    if (warp == 0) {
+        const bool bad = lane < ns && (s_big[lane] >= 0x7ff00000 ||
+                                       (int64_t)((s_big[lane] >> 20) - kRampSpread) * s_count[lane] > (int64_t)s_exp[lane]);
+        const unsigned int mask = __ballot_sync(0xffffffffu, bad);
+        if (lane == 0) g.bad[blockIdx.x * gridDim.y + blockIdx.y] = mask;
+    }
     // (lane: velocity lane / 8 of four, spectrum lane mod 8)
     for (int k0 = 4 * warp; k0 < g.n_v; k0 += n_thr / 8) {
         const int k = min(k0 + q, g.n_v - 1);
@@ -223,9 +229,6 @@ k_ccf_ramp(const __grid_constant__ RampArgs g, unsigned int* flags) {
                 v = fma(f.beta[j], tot[at + 32], v);
             }
         }
-        const double most = __hiloint2double(s_big[s8], 0) * s_weights;
-        const unsigned int bad = __ballot_sync(0xffffffffu, on && !(most <= kRampTrust * fabs(v) && most < CUDART_INF));
-        if (lane == 0) g.bad[((int64_t)blockIdx.x * gridDim.y + blockIdx.y) * ((g.n_v + 3) / 4) + k0 / 4] = bad;
         if (on) g.partial[((int64_t)blockIdx.x * g.n_spec + s0 + s8) * g.n_v + k] = v;
     }
 }
@@ -234,7 +237,7 @@ k_ccf_ramp(const __grid_constant__ RampArgs g, unsigned int* flags) {
 // cover.  Block = (lines and spectra of a block there, 32 velocities); lane = velocity, so that a warp's
 // pixels are neighbours; eight warps share the lines.  A box's overlaps are FP64 instructions, which bound
 // this: computed once for all spectra, compared on their bits.  Where there is nothing to replace, a block
-// only reads its eight words.
+// only reads its word.
 constexpr int kDirectWarps = 8;
 __global__ void __launch_bounds__(32 * kDirectWarps)
 k_ramp_direct(const __grid_constant__ RampArgs g) {
@@ -243,10 +246,8 @@ k_ramp_direct(const __grid_constant__ RampArgs g) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int k = 32 * blockIdx.z + lane, n_words = (g.n_v + 3) / 4;
-    const unsigned int* word = g.bad + ((int64_t)blockIdx.x * gridDim.y + blockIdx.y) * n_words;
-    const unsigned int mine = k < g.n_v ? (word[k / 4] >> (8 * (k & 3))) & 255u : 0u;
-    const unsigned int any = __reduce_or_sync(0xffffffffu, mine);
+    const int k = 32 * blockIdx.z + lane;
+    const unsigned int any = g.bad[blockIdx.x * gridDim.y + blockIdx.y];
     if (any == 0) return;
     const int s0 = blockIdx.y * kRampSpec, kk = min(k, g.n_v - 1), Sk = g.S[kk];
     const double gk = g.g[kk];
@@ -291,7 +292,7 @@ k_ramp_direct(const __grid_constant__ RampArgs g) {
     double v = 0.0;
 #pragma unroll
     for (int w = 0; w < kDirectWarps; w++) v += part[w][s][lane];
-    if ((mine >> s) & 1) g.partial[((int64_t)blockIdx.x * g.n_spec + s0 + s) * g.n_v + k] = v;
+    if (((any >> s) & 1) && k < g.n_v) g.partial[((int64_t)blockIdx.x * g.n_spec + s0 + s) * g.n_v + k] = v;
 }
 
 // ---------------------------------------------------------------------------------------
@@ -449,7 +450,7 @@ soap_status ccf_ramp_build(soap_ctx* c, CcfState& st, const CcfPlan& p) {
 }
 
 size_t ccf_ramp_scratch(const CcfPlan& p) {
-    return (size_t)p.n_chunks * ((p.n_spec + kRampSpec - 1) / kRampSpec) * ((p.n_v + 3) / 4) * sizeof(unsigned int);
+    return (size_t)p.n_chunks * ((p.n_spec + kRampSpec - 1) / kRampSpec) * sizeof(unsigned int);
 }
 
 soap_status ccf_ramp(soap_ctx* c, const CcfState& st, const CcfPlan& p, const double* spectra, double* partial) {
